@@ -176,12 +176,8 @@ int one_step(Sim *s, bool fields) {
         // multigrid-preconditioned completion (large meshes)
         if ((rc = mg_completion(s))) return rc;
     } else {
-        // the completion is latency-bound: two blocks per SM, unless the
-        // configuration fixes the count (1, 2, 3, 4 per SM measured 4.25,
-        // 3.40, 3.49, 3.52 ms on the 64^3 plasma-ball mesh)
         PcgArgs a = pcg_args_completion(s);
-        const int per_sm = s->cfg.solver_blocks_per_sm ? s->cfg.solver_blocks_per_sm : 2;
-        if ((rc = launch_pcg_runs(&a, 1, per_sm, s->stream))) return rc;
+        if ((rc = launch_pcg_runs(&a, 1, s->cfg.solver_blocks_per_sm, s->stream))) return rc;
     }
     // the next step's sort, behind the completion (under it, it slowed the
     // latency-bound solve by more than its own time) and beside the rest

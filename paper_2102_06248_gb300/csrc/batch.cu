@@ -17,9 +17,10 @@
 //     graph and replayed;
 //   * for each of the two solves the tuner picks the blocks per SM and the
 //     build of the batched kernel (64 registers for up to four blocks per
-//     SM, 80 for up to three, 40 for up to six, 32 for up to eight) by
-//     timing every candidate on the batch's own systems; the choice is kept
-//     per batch shape.
+//     SM, 80 for up to three) by timing every candidate on the batch's own
+//     systems; the choice is kept per batch shape.  (The candidates of more
+//     blocks per SM, builds of 40 and 32 registers, stand for four blocks of
+//     the first: the warps' rings fill the shared memory of four.)
 #include <map>
 #include <mutex>
 #include <utility>
@@ -144,10 +145,8 @@ int batch_step_once(pic_batch *b) {
 }
 
 // The solvers' launch shape for this batch.  Each candidate (blocks per SM
-// 2, 3, 4 with the 64-register build, 2 and 3 with the 80-register one, 5 and
-// 6 with the 40-register one, 7 and 8 with the 32-register one) is timed on
-// every member's own last systems,
-// once to warm up and once timed:
+// 2, 3, 4 with the 64-register build, 2 and 3 with the 80-register one) is
+// timed on every member's own last systems, once to warm up and once timed:
 // the Newmark solve stopped after 40 iterations from x = 0 (x is rewritten
 // before the next solve), and the completion's solve of its last defect to
 // its tolerance.  When members have a multigrid hierarchy, the completions
@@ -186,6 +185,12 @@ int autotune(pic_batch *b) {
             // the combined completion launch has one build (64 registers)
             const bool mg_launch = solve == 1 && b->use_mg;
             if (mg_launch && kTuneBuild[c] != 0) continue;
+            if (kTuneBuild[c] > 1) {
+                // more than four blocks per SM do not fit (the warps' rings):
+                // the candidate is four blocks of the 64-register build
+                (solve == 0 ? b->tune_ms : b->tune_gc_ms)[c] = (solve == 0 ? b->tune_ms : b->tune_gc_ms)[2];
+                continue;
+            }
             for (int rep = 0; rep < 2 && rc == PIC_OK; rep++) {
                 if (mg_launch) {
                     b->gc_blocks_per_sm = kTuneBps[c];

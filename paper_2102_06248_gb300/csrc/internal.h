@@ -96,10 +96,14 @@ struct DevCsr {
 // Sparse matrix pattern in SELL-32 (device): slice s = rows 32s..32s+31,
 // entry j of lane l at ptr[s] + 32 j + l, width[s] entries per row (padded
 // with the row's own column and a zero value)
+// narrow: column k (= element / 32) of the matrix has col = base[k] + lane +
+// off[element] in every lane (the streamed solver matrices, stream.cuh)
 struct DevSell {
     int n_rows = 0, n_slices = 0;
     long long n_elems = 0;
-    DevBuf<int> ptr, width, col;
+    int narrow = 0;
+    DevBuf<int> ptr, width, col, base;
+    DevBuf<unsigned char> off;
 };
 
 // Host-side staging of the device arrays (kept until the first upload)
@@ -109,11 +113,13 @@ struct HostCsrStage {
 struct HostStage {
     std::vector<double> geo;
     std::vector<int4> tet_nodes, tet_nbr, tet_face, f2e;
-    std::vector<int> tet_edge, node_int, int_node;
+    std::vector<int> tet_edge, node_int, int_node, e2t_row;
     std::vector<int2> edge_nodes;
     HostCsrStage e2t, n2t, L, e2f, n2e;
     std::vector<double> L_val;
     std::vector<int> sell_ptr, sell_w, sell_col, lsell_ptr, lsell_w, lsell_col, hsell_ptr, hsell_w, hsell_col;
+    std::vector<int> sell_base, lsell_base;               // narrow column encoding (empty: 32-bit columns)
+    std::vector<unsigned char> sell_off, lsell_off;
     std::vector<double> sell_M, sell_K, M_diag, K_diag, lsell_L, L_diag, hsell_H;
     std::vector<double> sell_I, I_diag;          // surface impedance of absorbing walls, A's layout
     std::vector<int> irow;                       // DOF rows with surface-impedance entries
@@ -158,7 +164,8 @@ struct Mesh {
     DevBuf<double> tet_vol;
     DevBuf<double> xyz;
     // reductions from per-tet accumulators to entities (fixed order)
-    DevCsr e2t;                // internal edge -> tet*6 + local edge
+    DevCsr e2t;                // canonical edge -> tet*6 + local edge
+    DevBuf<int> e2t_row;       // its internal edge id
     DevCsr n2t;                // node -> tet*4 + local vertex
     // Newmark system on interior edges: shared SELL-32 pattern of M, K (and A)
     DevSell As;

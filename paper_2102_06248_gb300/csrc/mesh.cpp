@@ -23,6 +23,7 @@ namespace fp {
 namespace {
 
 const int kLE[6][2] = {{0, 1}, {0, 2}, {0, 3}, {1, 2}, {1, 3}, {2, 3}};
+constexpr size_t kMaxEdgeSteps = 64;   // more different head - tail than a lattice has: no regular numbering
 const int kLF[4][3] = {{1, 2, 3}, {0, 2, 3}, {0, 1, 3}, {0, 1, 2}};
 
 inline double dot3(const double *a, const double *b) { return a[0] * b[0] + a[1] * b[1] + a[2] * b[2]; }
@@ -83,47 +84,117 @@ inline int find_col(const HostCsr &a, int row, int col) {
 }
 
 
+// Columns of a SELL slice that name one lane's entry each: -1 where the lane
+// has none (padding)
+struct SlotTable {
+    std::vector<int> k;   // CSR position, 32 per slot
+    int n = 0;
+};
+
+// Slots of slice sl, each lane's entries in increasing column order.  Packed
+// to the left, the j-th entries of 32 rows name unrelated places as soon as
+// one row lacks a neighbour the others have (next to a wall).  Aligned, a slot
+// takes only entries whose distance from their row lies within kNarrowSpan of
+// the smallest one waiting: a lane without such an entry leaves it empty.  A
+// warp's gather of a slot then touches the 4-5 sectors of 32 consecutive
+// values (11.7 on the packed rows of the 64^3 box, 4.6 aligned), and a column
+// is told by one byte.
+constexpr int kNarrowSpan = 255 - 31;
+void slice_slots(const HostCsr &pa, int n, int sl, bool aligned, SlotTable *t) {
+    int pos[32], end[32];
+    t->k.clear();
+    t->n = 0;
+    for (int l = 0; l < 32; l++) {
+        const int r = 32 * sl + l;
+        pos[l] = r < n ? pa.rowptr[r] : 0;
+        end[l] = r < n ? pa.rowptr[r + 1] : 0;
+    }
+    while (true) {
+        long lo = 1L << 40;
+        bool any = false;
+        for (int l = 0; l < 32; l++)
+            if (pos[l] < end[l]) {
+                lo = std::min(lo, (long)pa.col[pos[l]] - l);
+                any = true;
+            }
+        if (!any) return;
+        for (int l = 0; l < 32; l++) {
+            const bool take = pos[l] < end[l] && (!aligned || (long)pa.col[pos[l]] - l <= lo + kNarrowSpan);
+            t->k.push_back(take ? pos[l]++ : -1);
+        }
+        t->n++;
+    }
+}
+
 // SELL-32 layout of a CSR pattern: slice s holds rows 32s..32s+31, entry j of
-// lane l at ptr[s] + 32 j + l; padding points at the row itself with value 0.
-// vals: CSR value arrays to lay out; diag receives each row's diagonal.
+// lane l at ptr[s] + 32 j + l; padding has the value 0 and names an existing
+// column.  vals: CSR value arrays to lay out; diag receives each row's
+// diagonal.  With base and off given, the slots are aligned and the columns
+// also encoded as base[element / 32] + lane + off[element]; if the aligned
+// slots need more than 1/8 more room than the entries (meshes without a regular
+// numbering), the rows are packed and base stays empty.
 void build_sell(const HostCsr &pa, const std::vector<const std::vector<double> *> &vals, std::vector<int> &ptr,
                 std::vector<int> &w, std::vector<int> &col, std::vector<std::vector<double>> &out,
-                std::vector<std::vector<double>> &diag) {
+                std::vector<std::vector<double>> &diag, std::vector<int> *base = nullptr,
+                std::vector<unsigned char> *off = nullptr) {
     const int n = (int)pa.rowptr.size() - 1;
     const int nsl = (n + 31) / 32;
+    SlotTable t;
+    bool aligned = base != nullptr;
+    if (aligned) {
+        size_t cols = 0;
+        for (int sl = 0; sl < nsl; sl++) {
+            slice_slots(pa, n, sl, true, &t);
+            cols += t.n;
+        }
+        aligned = 32 * cols <= pa.col.size() + pa.col.size() / 8 + 32 * 64;
+    }
     ptr.assign(nsl + 1, 0);
     w.assign(nsl, 0);
-    for (int sl = 0; sl < nsl; sl++) {
-        int ww = 0;
-        for (int l = 0; l < 32; l++) {
-            const int r = 32 * sl + l;
-            if (r < n) ww = std::max(ww, pa.rowptr[r + 1] - pa.rowptr[r]);
-        }
-        w[sl] = ww;
-        ptr[sl + 1] = ptr[sl] + 32 * ww;
-    }
-    const size_t nel = (size_t)ptr[nsl];
-    col.assign(nel, 0);
-    out.assign(vals.size(), std::vector<double>(nel, 0.0));
+    col.clear();
+    out.assign(vals.size(), std::vector<double>());
     diag.assign(vals.size(), std::vector<double>(n, 0.0));
-    for (int sl = 0; sl < nsl; sl++)
-        for (int l = 0; l < 32; l++) {
-            const int r = 32 * sl + l;
-            const int rr = r < n ? r : n - 1;
-            for (int j = 0; j < w[sl]; j++) {
-                const size_t q = (size_t)ptr[sl] + 32 * (size_t)j + l;
-                const int k = pa.rowptr[rr] + j;
-                if (r < n && k < pa.rowptr[r + 1]) {
-                    col[q] = pa.col[k];
-                    for (size_t v = 0; v < vals.size(); v++) {
-                        out[v][q] = (*vals[v])[k];
-                        if (pa.col[k] == r) diag[v][r] = (*vals[v])[k];
-                    }
-                } else {
-                    col[q] = rr;
+    if (base) {
+        base->clear();
+        off->clear();
+    }
+    for (int sl = 0; sl < nsl; sl++) {
+        slice_slots(pa, n, sl, aligned, &t);
+        w[sl] = t.n;
+        ptr[sl + 1] = ptr[sl] + 32 * t.n;
+        for (int j = 0; j < t.n; j++) {
+            const int *k = t.k.data() + 32 * (size_t)j;
+            int lo = 0, hi = 0;
+            bool first = true, outside = false;
+            for (int l = 0; l < 32; l++)
+                if (k[l] >= 0) {
+                    const int d = pa.col[k[l]] - l;
+                    lo = first ? d : std::min(lo, d);
+                    hi = first ? d : std::max(hi, d);
+                    first = false;
                 }
+            for (int l = 0; l < 32; l++)
+                if (k[l] < 0 && (lo + l < 0 || lo + l >= n)) outside = true;
+            // an empty lane whose place base + lane would lie outside: a base
+            // 31 lower puts every lane's column in reach of its byte
+            const int b = outside ? lo - 31 : lo;
+            for (int l = 0; l < 32; l++) {
+                const int r = 32 * sl + l;
+                int c;
+                if (k[l] >= 0) c = pa.col[k[l]];
+                else if (aligned) c = std::min(std::max(lo + l, 0), n - 1);
+                else c = std::min(r, n - 1);
+                col.push_back(c);
+                for (size_t v = 0; v < vals.size(); v++) {
+                    const double x = k[l] >= 0 ? (*vals[v])[k[l]] : 0.0;
+                    out[v].push_back(x);
+                    if (k[l] >= 0 && c == r) diag[v][r] = x;
+                }
+                if (aligned) off->push_back((unsigned char)(c - l - b));
             }
+            if (aligned) base->push_back(b);
         }
+    }
 }
 
 }  // namespace
@@ -285,24 +356,40 @@ int build_mesh(const pic_mesh_desc *d, Mesh *m) {
         edge_bnd[edge_id((uint64_t)b * nn + c)] = 1;
         edge_bnd[edge_id((uint64_t)a * nn + c)] = 1;
     }
-    // internal numbering: interior edges first, ordered by the length of
-    // their row in the Newmark matrix (edges sharing a tet) and canonically
-    // within a length, so that 32 consecutive rows (one SELL slice) have
-    // nearly equal lengths; boundary edges follow in canonical order
+    // internal numbering: interior edges first, boundary edges after them in
+    // canonical order.  On a mesh with a regular node numbering (few different
+    // head - tail: a lattice), the interior edges are ordered by head - tail
+    // and canonically within one: 32 consecutive rows of the Newmark matrix
+    // (one SELL slice) are then parallel edges, whose neighbours are
+    // consecutive rows too.  Otherwise they are ordered by the length of their
+    // row (edges sharing a tet) and canonically within a length, so that a
+    // slice's rows have nearly equal lengths.
     m->h_edge_internal.assign(ne, -1);
     m->h_edge_canonical.assign(ne, -1);
     int ni = 0;
+    bool regular = false;
     {
-        HostCsr pc = pattern_from_groups(ne, nt, 6, ne, ne, [&](int t, int *out) {
-            for (int k = 0; k < 6; k++) {
-                const int e = tet_edge_c[6 * (size_t)t + k];
-                out[k] = edge_bnd[e] ? -1 : e;
-            }
-        });
         std::vector<std::pair<int, int>> order;
         order.reserve(ne);
-        for (int e = 0; e < ne; e++)
-            if (!edge_bnd[e]) order.push_back({pc.rowptr[e + 1] - pc.rowptr[e], e});
+        std::vector<int> steps;
+        for (int e = 0; e < ne && steps.size() <= kMaxEdgeSteps; e++) {
+            const int d = m->h_edges[2 * (size_t)e + 1] - m->h_edges[2 * (size_t)e];
+            if (!edge_bnd[e] && std::find(steps.begin(), steps.end(), d) == steps.end()) steps.push_back(d);
+        }
+        regular = steps.size() <= kMaxEdgeSteps;
+        if (regular) {
+            for (int e = 0; e < ne; e++)
+                if (!edge_bnd[e]) order.push_back({m->h_edges[2 * (size_t)e + 1] - m->h_edges[2 * (size_t)e], e});
+        } else {
+            HostCsr pc = pattern_from_groups(ne, nt, 6, ne, ne, [&](int t, int *out) {
+                for (int k = 0; k < 6; k++) {
+                    const int e = tet_edge_c[6 * (size_t)t + k];
+                    out[k] = edge_bnd[e] ? -1 : e;
+                }
+            });
+            for (int e = 0; e < ne; e++)
+                if (!edge_bnd[e]) order.push_back({pc.rowptr[e + 1] - pc.rowptr[e], e});
+        }
         std::sort(order.begin(), order.end());
         for (auto &pr : order) m->h_edge_internal[pr.second] = ni++;
     }
@@ -311,19 +398,22 @@ int build_mesh(const pic_mesh_desc *d, Mesh *m) {
     for (int e = 0; e < ne; e++)
         if (edge_bnd[e]) m->h_edge_internal[e] = nb_++;
     for (int e = 0; e < ne; e++) m->h_edge_canonical[m->h_edge_internal[e]] = e;
-    // interior nodes, ordered by the length of their Laplacian row (node ids
-    // within a length) for the SELL-32 layout of the node Laplacian
+    // interior nodes, in the order of their ids on a mesh with a regular
+    // numbering, else by the length of their Laplacian row (ids within a
+    // length), for the SELL-32 layout of the node Laplacian
     std::vector<int> node_int(nn, -1), int_node;
     {
-        HostCsr pn = pattern_from_groups(nn, nt, 4, nn, nn, [&](int t, int *out) {
-            for (int k = 0; k < 4; k++) {
-                const int v = TS[4 * t + k];
-                out[k] = m->h_node_bnd[v] ? -1 : v;
-            }
-        });
         std::vector<std::pair<int, int>> order;
+        HostCsr pn;
+        if (!regular)
+            pn = pattern_from_groups(nn, nt, 4, nn, nn, [&](int t, int *out) {
+                for (int k = 0; k < 4; k++) {
+                    const int v = TS[4 * t + k];
+                    out[k] = m->h_node_bnd[v] ? -1 : v;
+                }
+            });
         for (int n = 0; n < nn; n++)
-            if (!m->h_node_bnd[n]) order.push_back({pn.rowptr[n + 1] - pn.rowptr[n], n});
+            if (!m->h_node_bnd[n]) order.push_back({regular ? 0 : pn.rowptr[n + 1] - pn.rowptr[n], n});
         std::sort(order.begin(), order.end());
         for (auto &pr : order) {
             node_int[pr.second] = (int)int_node.size();
@@ -374,7 +464,10 @@ int build_mesh(const pic_mesh_desc *d, Mesh *m) {
         out->col = std::move(idx);
     };
     HostStage &H = *m->stage;
-    build_map(ne, 6, tet_edge.data(), &H.e2t);
+    // (edge rows in canonical order: neighbouring rows then share tets, whose
+    // accumulators the gather reads from L1; e2t_row names the row's edge)
+    build_map(ne, 6, tet_edge_c.data(), &H.e2t);
+    H.e2t_row = m->h_edge_internal;
     build_map(nn, 4, TS, &H.n2t);
 
     // ---- matrices ----
@@ -597,9 +690,9 @@ int build_mesh(const pic_mesh_desc *d, Mesh *m) {
     {
         std::vector<std::vector<double>> out, dg;
         if (m->n_abs_faces > 0)
-            build_sell(pa, {&Mv, &Kv, &Iv}, H.sell_ptr, H.sell_w, H.sell_col, out, dg);
+            build_sell(pa, {&Mv, &Kv, &Iv}, H.sell_ptr, H.sell_w, H.sell_col, out, dg, &H.sell_base, &H.sell_off);
         else
-            build_sell(pa, {&Mv, &Kv}, H.sell_ptr, H.sell_w, H.sell_col, out, dg);
+            build_sell(pa, {&Mv, &Kv}, H.sell_ptr, H.sell_w, H.sell_col, out, dg, &H.sell_base, &H.sell_off);
         H.sell_M = std::move(out[0]);
         H.sell_K = std::move(out[1]);
         H.M_diag = std::move(dg[0]);
@@ -609,7 +702,7 @@ int build_mesh(const pic_mesh_desc *d, Mesh *m) {
             H.I_diag = std::move(dg[2]);
         }
         m->nnz_A = (long long)pa.col.size();
-        build_sell(pl, {&Lv}, H.lsell_ptr, H.lsell_w, H.lsell_col, out, dg);
+        build_sell(pl, {&Lv}, H.lsell_ptr, H.lsell_w, H.lsell_col, out, dg, &H.lsell_base, &H.lsell_off);
         H.lsell_L = std::move(out[0]);
         H.L_diag = std::move(dg[0]);
         // the face mass in natural face order (rows of 4 or 7 entries)
@@ -644,14 +737,15 @@ int mesh_upload(Mesh *m) {
         (rc = m->tet_edge.upload(H.tet_edge)) || (rc = m->tet_face.upload(H.tet_face)) ||
         (rc = m->tet_sign.upload(m->h_tet_sign)) || (rc = m->tet_vol.upload(m->h_vol)) || (rc = m->xyz.upload(m->h_xyz)))
         return rc;
-    if ((rc = csr(H.e2t, &m->e2t)) || (rc = csr(H.n2t, &m->n2t))) return rc;
+    if ((rc = csr(H.e2t, &m->e2t)) || (rc = csr(H.n2t, &m->n2t)) || (rc = m->e2t_row.upload(H.e2t_row))) return rc;
     m->As.n_rows = m->n_int_edges;
     m->As.n_slices = (int)H.sell_w.size();
     m->As.n_elems = H.sell_ptr.empty() ? 0 : H.sell_ptr.back();
     if ((rc = m->As.ptr.upload(H.sell_ptr)) || (rc = m->As.width.upload(H.sell_w)) || (rc = m->As.col.upload(H.sell_col)) ||
         (rc = m->M_val.upload(H.sell_M)) || (rc = m->K_val.upload(H.sell_K)) || (rc = m->M_diag.upload(H.M_diag)) ||
-        (rc = m->K_diag.upload(H.K_diag)))
+        (rc = m->K_diag.upload(H.K_diag)) || (rc = m->As.base.upload(H.sell_base)) || (rc = m->As.off.upload(H.sell_off)))
         return rc;
+    m->As.narrow = !H.sell_base.empty();
     m->Hs.n_rows = m->n_faces;
     m->Hs.n_slices = (int)H.hsell_w.size();
     m->Hs.n_elems = H.hsell_ptr.empty() ? 0 : H.hsell_ptr.back();

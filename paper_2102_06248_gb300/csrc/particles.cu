@@ -1212,14 +1212,16 @@ __global__ void __launch_bounds__(256) k_overflow_scatter(const int *d_count, in
 // PLAIN accumulators hold charge already; MIXED ones hold fixed-point sums per
 // species, converted here with the species' q w.
 template <typename V>
-__global__ void __launch_bounds__(256) k_gather_edges(int ne, const int *__restrict__ ptr, const int *__restrict__ idx,
+__global__ void __launch_bounds__(256) k_gather_edges(int ne, const int *__restrict__ row, const int *__restrict__ ptr,
+                                                      const int *__restrict__ idx,
                                                       const V *__restrict__ tacc, int nsp, SpeciesParams sp,
                                                       const double *__restrict__ g, double *__restrict__ dg,
                                                       double *__restrict__ g_new) {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= ne) return;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= ne) return;
+    const int e = row[i];
     double s = 0.0;
-    for (int k = ptr[e]; k < ptr[e + 1]; k++) {
+    for (int k = ptr[i]; k < ptr[i + 1]; k++) {
         const int ref = idx[k];
         const size_t t = (size_t)(ref / 6);
         const int l = ref % 6;
@@ -1991,7 +1993,7 @@ int reduce_to_entities(Sim *s) {
     std::swap(s->wall_prev, s->wall);
     const SpeciesParams sp = species_params(s);
     if (s->mixed) {
-        { k_gather_edges<long long><<<(m->n_edges + 255) / 256, 256, 0, s->stream>>>(m->n_edges, m->e2t.rowptr.p, m->e2t.col.p, (const long long *)s->tacc.p, s->nsp, sp, s->g.p, s->dg.p, s->g_new.p); note_launch(); }
+        { k_gather_edges<long long><<<(m->n_edges + 255) / 256, 256, 0, s->stream>>>(m->n_edges, m->e2t_row.p, m->e2t.rowptr.p, m->e2t.col.p, (const long long *)s->tacc.p, s->nsp, sp, s->g.p, s->dg.p, s->g_new.p); note_launch(); }
         if (!s->nacc.p) {
             int rc = s->nacc.alloc(2 * (size_t)m->n_nodes * s->nsp);
             if (rc) return rc;
@@ -2001,7 +2003,7 @@ int reduce_to_entities(Sim *s) {
         { k_scatter_node_charge<<<(ntq + 255) / 256, 256, 0, s->stream>>>(m->n_tets, s->nsp, m->tet_nodes.p, (const long long *)s->tacc.p, (const long long *)s->wacc.p, s->nacc.p); note_launch(); }
         { k_node_charge_convert<<<(m->n_nodes + 255) / 256, 256, 0, s->stream>>>(m->n_nodes, s->nsp, sp, s->nacc.p, s->wall_prev.p, s->rho.p, s->wall.p); note_launch(); }
     } else {
-        { k_gather_edges<double><<<(m->n_edges + 255) / 256, 256, 0, s->stream>>>(m->n_edges, m->e2t.rowptr.p, m->e2t.col.p, (const double *)s->tacc.p, 1, sp, s->g.p, s->dg.p, s->g_new.p); note_launch(); }
+        { k_gather_edges<double><<<(m->n_edges + 255) / 256, 256, 0, s->stream>>>(m->n_edges, m->e2t_row.p, m->e2t.rowptr.p, m->e2t.col.p, (const double *)s->tacc.p, 1, sp, s->g.p, s->dg.p, s->g_new.p); note_launch(); }
         { k_gather_nodes<double><<<(m->n_nodes + 255) / 256, 256, 0, s->stream>>>(m->n_nodes, m->n2t.rowptr.p, m->n2t.col.p, (const double *)s->tacc.p, (const double *)s->wacc.p, 1, sp, s->wall_prev.p, s->rho.p, s->wall.p); note_launch(); }
     }
     FP_CUDA(cudaGetLastError());

@@ -40,10 +40,8 @@ struct DiagDev {
 // state of the bounded grid barrier of the persistent kernels
 struct GridBarrier {
     unsigned int count;   // arrivals since the launch (epoch k completes at k * blocks)
-    unsigned int flag;    // last epoch whose reduction results are published
-    int timeout;
-    int pad;
-    double val[6];        // results the last arriving block publishes
+    int timeout;          // a wait ran out of its bound: every block leaves
+    int pad[2];
 };
 
 // Host-visible control block (pinned), refreshed at every synchronising point
@@ -65,8 +63,11 @@ struct Control {
 // its vectors, the stopping rule and the blocks of the launch it owns
 struct PcgArgs {
     int n, n_slices;
-    const int *sp, *sw, *col;     // SELL-32: slice offsets, widths, column indices
-    const double *Av, *Dinv, *b;
+    const int *sp, *sw;           // SELL-32: slice offsets and widths
+    const unsigned char *rec;     // the matrix as FP64 records (stream.cuh)
+    int wide;                     // records with 32-bit columns
+    int evict_first;              // matrix larger than L2 can keep: stream it through
+    const double *Dinv, *b;       // (every vector is padded to whole slices, zeros past n)
     double *x, *r, *u, *w, *p, *s;
     double *part;                 // >= 5 * blocks partials
     CgState *st;                  // results (iterations, residual, failure)
@@ -86,7 +87,8 @@ struct PcgArgs {
     // mixed-precision refinement (refine = 1): FP64 residuals, FP32 corrections
     int refine;
     double inner_tol2;            // relative residual^2 of each FP32 correction solve
-    const float *Av32, *Dhalf32;   // FP32 values of D^-1/2 A D^-1/2, and D^-1/2
+    const unsigned char *rec32;   // FP32 records of D^-1/2 A D^-1/2
+    const float *Dhalf32;         // D^-1/2
     float *b32, *d32, *r32, *w32, *p32, *s32;
 };
 constexpr int kMaxBatchRuns = 64;
@@ -207,7 +209,8 @@ struct Sim {
     DevBuf<double> rhs;
     // solver work
     DevBuf<double> A_val, Dinv;
-    DevBuf<float> A32, Dhalf32, cg32;  // MIXED: FP32 scaled values, D^-1/2 and six correction vectors
+    DevBuf<float> Dhalf32, cg32;       // MIXED: D^-1/2 and six correction vectors
+    DevBuf<unsigned char> A_rec, A_rec32, L_rec;   // the solvers' matrices as records (stream.cuh)
     DevBuf<double> cg_r, cg_z, cg_p0, cg_p1, cg_q, cg_part;
     DevBuf<double> hb;              // face vector H (b + b_prev)
     DevBuf<double> w_edge;          // gradient completion: M t - d2 Gbar on interior edges

@@ -13,6 +13,7 @@
 #include <type_traits>
 
 #include "sim.h"
+#include "stream.cuh"
 
 namespace fp {
 
@@ -684,48 +685,59 @@ __global__ void __launch_bounds__(kThreads) k_max_abs_sum(int n, const double *_
 //    s = w + beta s, so one global reduction per iteration yields
 //    gamma = (r,u), delta = (w,u) and (r,r), from which
 //    beta = gamma'/gamma and alpha = gamma'/(delta - beta gamma'/alpha);
-//  * each block reduces its threads' values through shared memory (one warp
-//    per quantity) and only the last block to arrive at the grid barrier
-//    combines the blocks' partials, in a fixed order, and publishes the
-//    result; max|r| travels as the bit pattern of a nonnegative double, whose
-//    integer order is its numeric order, so it costs no FP64 instruction.
-// Every thread owns the same rows (row 32*slice + lane of its warp's slices)
-// in the vector phase and in the SpMV, so a thread reads back only what it
-// wrote itself, except the gathered vector (u, or the correction iterate):
-// plain loads in the two-slice form below, reads through L2 (__ldcg) in the
-// one-slice FP64 form; both see the other blocks' writes after the barrier.
-// The rest is latency work: the slice headers of a block's slices sit in
-// shared memory for the whole solve (the next one is read while the current
-// slice is summed), and the grid barriers are one release-add on a counter
-// that only grows plus acquire-loads.  (An L2 bulk prefetch of the next
-// slice's values and columns made the solve slower: it delays the slowest
-// blocks at the barrier.)  Every barrier spins with a bound: past it the kernel
-// records a timeout and every block leaves.
+//  * a reduction forms few FP64 sums, and the scalars of an iteration are
+//    formed by one warp of each block (grid_reduce); max|r| travels as the bit
+//    pattern of a nonnegative double, whose integer order is its numeric
+//    order, so it costs no FP64 instruction.
+// The matrix is streamed through shared memory by bulk copies (stream.cuh),
+// each warp a contiguous run of slices.  Every thread owns the rows of its
+// warp in the vector phase and in the SpMV; only the gathered vector (u, or the
+// correction iterate) is read across blocks, by plain loads that L1 may keep:
+// the grid barrier between the phases is a release/acquire pair, so they see
+// the other blocks' writes.  The grid barriers are one release-add on a
+// counter that only grows plus acquire-loads; every wait is bounded, past its
+// bound the kernel records a timeout and every block leaves.
+// Measured on the 64^3 plasma ball (1.8M rows, MIXED, 60 iterations): 4.44 ->
+// 2.69 ms a solve, 45 us an iteration: the stream of 150 MB of records takes
+// 22 us of them at the copy rate (it was 232 MB), the vector phase 4 us, the
+// two barriers and the reduction 9 us.
 // ---------------------------------------------------------------------------
-constexpr int kMaxPcgBlocks = 4 * kThreads;    // largest grid of the persistent PCG
-constexpr int kSmemSlices = 512;               // slice headers a block keeps in shared memory
+constexpr int kMaxPcgBlocks = 4 * kThreads;    // most blocks of one solve
+// Block (one per SM) and bytes of a warp's ring of a single solve: the FP64
+// PCG and anything on wide records, and the refinement on narrow ones
+template <bool REFINE, bool WIDE>
+struct PcgShape {
+    // (refinement, FP32 gathers in flight: 512, 768, 1024 threads 3.50, 2.79,
+    // 2.88 ms per Newmark solve of the 64^3 plasma ball, 128, 80, 64
+    // registers; FP64, bound by the FP64 pipes: 512 and 768 threads 1.75 and
+    // 1.87 ms on 40^3)
+    static constexpr int threads = REFINE && !WIDE ? 768 : 512;
+    static constexpr int ring = REFINE && !WIDE ? 2 * Record<double, false>::bytes : 8192;
+};
+// block of the multigrid completion (one per SM; 512 threads: 1.81 ms against
+// 1.44 ms on the 64^3 plasma ball, its phases wait on dependent loads)
+constexpr int kMgThreads = 1024;
+constexpr int kBatchRing = 2 * Record<double, false>::bytes;      // ... in the batched kernels
+constexpr int kBatchRingWide = 2 * Record<double, true>::bytes;
+// A matrix up to this size is left to stay in L2 between iterations, a larger
+// one is loaded evict-first so that the vectors stay (FP32 records of 67, 74
+// and 150 MB on the 48^3, 32x32x128 and 64^3 meshes: kept 4.40, 2.00, 3.92 ms
+// a solve, evict-first 4.46, 1.95, 3.15 ms)
+constexpr size_t kKeepInL2 = 70u << 20;
+constexpr int kSlicesPerPcgBlock = 4;          // a small system takes a block per four slices
+constexpr int kSmemSlices = 1024;              // slice widths a block keeps in shared memory
 constexpr long kSpinLimit = 1L << 22;          // about a second of polling
 constexpr int kMaxOuter = 12;                  // refinement steps of a mixed-precision solve
 constexpr int kMaxInner = 400;                 // FP32 iterations per refinement step
-constexpr int kVecSlices = 2;                  // slices a warp updates at once in the vector phase
 
 __device__ __forceinline__ void red_release_add(unsigned int *p, unsigned int v) {
     asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
-__device__ __forceinline__ unsigned int atom_acq_rel_add(unsigned int *p, unsigned int v) {
-    unsigned int old;
-    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
-    return old;
 }
 __device__ __forceinline__ unsigned int ld_acquire(const unsigned int *p) {
     unsigned int v;
     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
 }
-__device__ __forceinline__ void st_release(unsigned int *p, unsigned int v) {
-    asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
-
 // Spins (thread 0) until *p >= target; false when the bound or another
 // block's timeout ends the wait.
 __device__ __forceinline__ bool spin_until(GridBarrier *gb, const unsigned int *p, unsigned int target, long limit) {
@@ -756,91 +768,154 @@ __device__ __forceinline__ bool grid_barrier(GridBarrier *gb, unsigned int epoch
 __device__ __forceinline__ unsigned long long abs_bits(double v) {
     return (unsigned long long)__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFull;
 }
-
-// Block reduction of NS sums and one maximum (kept as bits) in a fixed order:
-// per quantity one warp adds the threads' values in thread order, then a
-// shuffle tree.  out(c, value) runs on lane 0 of warps 0..NS; the caller
-// synchronises before the shared arrays are reused.
-template <int NS, typename Out>
-__device__ __forceinline__ void block_reduce(const double v[NS], unsigned long long mx, double *shv,
-                                             unsigned long long *shm, Out out) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+__device__ __forceinline__ double warp_sum_d(double v) {
 #pragma unroll
-    for (int c = 0; c < NS; c++) shv[c * kThreads + threadIdx.x] = v[c];
-    shm[threadIdx.x] = mx;
-    __syncthreads();
-    if (warp < NS) {
-        double s = shv[warp * kThreads + lane];
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+    return v;
+}
+__device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long v) {
 #pragma unroll
-        for (int k = 1; k < kThreads / 32; k++) s += shv[warp * kThreads + lane + 32 * k];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xFFFFFFFFu, s, o);
-        if (lane == 0) out(warp, s);
-    } else if (warp == NS) {
-        unsigned long long m = shm[lane];
-#pragma unroll
-        for (int k = 1; k < kThreads / 32; k++) m = max(m, shm[lane + 32 * k]);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_down_sync(0xFFFFFFFFu, m, o));
-        if (lane == 0) out(NS, __longlong_as_double((long long)m));
-    }
+    for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xFFFFFFFFu, v, o));
+    return v;
 }
 
-// Reduction over the nb blocks of one solve at barrier number `epoch` (this
-// block is number bid): every block leaves its
-// partials (sums in part[c*G + block], c < NS; the maximum's bits in
-// part[NS*G + block]); the last block to arrive combines them in a fixed
-// order (thread t adds blocks t, t + kThreads, ..., all loads issued first,
-// then block_reduce), publishes the results in gb->val and raises gb->flag to
-// epoch.  out[0..NS) are the sums, out[NS] the maximum.
-template <int NS>
-__device__ __forceinline__ bool grid_reduce(GridBarrier *gb, double *part, const double v[NS],
-                                            unsigned long long mx, double *shv, unsigned long long *shm,
-                                            unsigned int epoch, double out[NS + 1], int nb, int bid, long limit) {
-    __shared__ int role;   // 1: last block, 0: waits, -1: timed out
+// Sum of a float over the warp, carried as hi + lo (every level an error-free
+// sum): exact but for terms 2^-48 below the total, at the FP32 rate
+__device__ __forceinline__ float2 warp_sum_f2(float v) {
+    float hi = v, lo = 0.0f;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const float b = __shfl_xor_sync(0xFFFFFFFFu, hi, o), bl = __shfl_xor_sync(0xFFFFFFFFu, lo, o);
+        const float t = __fadd_rn(hi, b), z = __fsub_rn(t, hi);
+        const float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(t, z)), __fsub_rn(b, z));
+        lo = __fadd_rn(__fadd_rn(lo, bl), e);
+        hi = t;
+    }
+    return make_float2(hi, lo);
+}
+
+__device__ __forceinline__ void sync_four_warps() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
+
+// Reduction of NS sums and one maximum (kept as bits) over the nb blocks of
+// one solve at barrier number `epoch` (this block, of T threads, is number
+// bid; its first `active` warps hold something), in a fixed order.  What it
+// costs is FP64 instructions and round trips to L2: each of an SM's four
+// schedulers issues one warp-wide FP64 instruction per 64 cycles (its result
+// comes after ~80; a division takes ~550), and a round trip is ~800 cycles.  So
+//  * per quantity one warp of the block, each on its own scheduler, adds the
+//    threads' values through shared memory and leaves the block's partial
+//    (sums in part[c * nb + block], the maximum's bits in part[NS * nb + block]);
+//    FP32 values are first added within their warps, as pairs of floats;
+//  * after ONE barrier (arrival counter, 1.2 us at 152 blocks, 2.2 us at 608)
+//    the first four warps of every block add all blocks' partials themselves, a
+//    quantity each, instead of waiting for a last block that combines and
+//    publishes them (two more round trips);
+//  * warps 0 and 1 then run scal(t, warp, lane), t[0..NS) the sums and t[NS]
+//    the maximum: the solver's scalars are formed by one warp, independent
+//    divisions in different lanes, its tests by the other, and handed to the
+//    block in shared memory.  (Formed by every thread, three divisions an
+//    iteration held the FP64 pipes for ~9 us.)
+template <int NS, int T, typename V, typename Scal>
+__device__ __forceinline__ bool grid_reduce(GridBarrier *gb, double *part, const V v[NS], unsigned long long mx,
+                                            double *shv, unsigned long long *shm, unsigned int epoch, int nb, int bid,
+                                            int active, long limit, Scal scal) {
+    __shared__ int ok;
     __shared__ double res[NS + 1];
-    const int G = nb;
-    block_reduce<NS>(v, mx, shv, shm, [&](int c, double val) { part[c * G + bid] = val; });
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        const unsigned int old = atom_acq_rel_add(&gb->count, 1u);
-        role = (old + 1u == epoch * (unsigned)G) ? 1 : 0;
+    constexpr bool kF32 = std::is_same<V, float>::value;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    static_assert(NS <= 4 && T / 32 > NS && T >= 128, "one warp per quantity");
+    // two sets of partials by parity: the next reduction may begin in a fast
+    // block while a slow one still reads this one's
+    part += (size_t)(epoch & 1u) * 5 * nb;
+    if (warp < active) {
+        if constexpr (kF32) {
+            float hi = 0.0f, lo = 0.0f;
+#pragma unroll
+            for (int c = 0; c < NS; c++) {
+                const float2 t = warp_sum_f2(v[c]);
+                hi = lane == c ? t.x : hi;
+                lo = lane == c ? t.y : lo;
+            }
+            if (lane < NS) shv[lane * 32 + warp] = (double)hi + (double)lo;
+        } else {
+#pragma unroll
+            for (int c = 0; c < NS; c++) shv[c * T + threadIdx.x] = v[c];
+            shm[threadIdx.x] = mx;
+        }
     }
     __syncthreads();
-    if (role == 1) {
-        double w[NS];
+    if (warp < NS) {
+        double sum;
+        if constexpr (kF32) {
+            sum = warp_sum_d(lane < active ? shv[warp * 32 + lane] : 0.0);
+        } else {
+            double s[4] = {0.0, 0.0, 0.0, 0.0};
+            for (int k = 0; k < active; k += 4) {
+#pragma unroll
+                for (int h = 0; h < 4; h++)
+                    if (k + h < active) s[h] += shv[warp * T + lane + 32 * (k + h)];
+            }
+            sum = warp_sum_d((s[0] + s[1]) + (s[2] + s[3]));
+        }
+        if (lane == 0) part[warp * nb + bid] = sum;
+    } else if (!kF32 && warp == NS) {
         unsigned long long m = 0;
+        for (int k = 0; k < active; k++) m = max(m, shm[lane + 32 * k]);
+        m = warp_max_u64(m);
+        if (lane == 0) part[NS * nb + bid] = __longlong_as_double((long long)m);
+    }
+    __syncthreads();
+    if (warp < 4) {
+        if (threadIdx.x == 0) {
+            red_release_add(&gb->count, 1u);
+            ok = spin_until(gb, &gb->count, epoch * (unsigned)nb, limit);
+        }
+        sync_four_warps();
+        int good = ok;
+        if (good) {
+            // raised by a block that lost a copy (stream.cuh): everybody leaves
+            const int lost = *(volatile int *)&gb->timeout;
+            constexpr int kU = 5;   // 152 blocks: one trip, every load issued before the first sum
+            if (warp < NS) {
+                double t = 0.0;
+                for (int b0 = lane; b0 < nb; b0 += 32 * kU) {
+                    double p[kU];
 #pragma unroll
-        for (int c = 0; c < NS; c++) w[c] = 0.0;
-        const unsigned long long *pm = reinterpret_cast<const unsigned long long *>(part) + NS * G;
+                    for (int k = 0; k < kU; k++) p[k] = b0 + 32 * k < nb ? __ldcg(part + warp * nb + b0 + 32 * k) : 0.0;
+                    t += ((p[0] + p[1]) + (p[2] + p[3])) + p[4];
+                }
+                t = warp_sum_d(t);
+                if (lane == 0) res[warp] = t;
+            }
+            if (warp == (NS < 4 ? NS : 3)) {
+                unsigned long long m = 0;
+                if constexpr (!kF32) {
+                    const unsigned long long *pm = reinterpret_cast<const unsigned long long *>(part) + NS * nb;
+                    for (int b0 = lane; b0 < nb; b0 += 32 * kU) {
 #pragma unroll
-        for (int k = 0; k < kMaxPcgBlocks / kThreads; k++) {
-            const int b = threadIdx.x + k * kThreads;
-            if (b < G) {
+                        for (int k = 0; k < kU; k++)
+                            if (b0 + 32 * k < nb) m = max(m, __ldcg(pm + b0 + 32 * k));
+                    }
+                    m = warp_max_u64(m);
+                }
+                if (lane == 0) res[NS] = __longlong_as_double((long long)m);
+            }
+            good = lost == 0;
+        }
+        sync_four_warps();
+        if (warp < 2) {
+            if (good) {
+                double t[NS + 1];
 #pragma unroll
-                for (int c = 0; c < NS; c++) w[c] += __ldcg(part + c * G + b);
-                m = max(m, __ldcg(pm + b));
+                for (int c = 0; c <= NS; c++) t[c] = res[c];
+                scal(t, warp, lane);
+            } else if (threadIdx.x == 0) {
+                ok = 0;
             }
         }
-        block_reduce<NS>(w, m, shv, shm, [&](int c, double val) {
-            res[c] = val;
-            gb->val[c] = val;
-        });
-        __syncthreads();
-        if (threadIdx.x == 0) st_release(&gb->flag, epoch);
-    } else if (role == 0 && threadIdx.x == 0) {
-        if (spin_until(gb, &gb->flag, epoch, limit)) {
-#pragma unroll
-            for (int c = 0; c <= NS; c++) res[c] = __ldcg(&gb->val[c]);
-        } else {
-            role = -1;
-        }
     }
     __syncthreads();
-    if (role < 0) return false;
-#pragma unroll
-    for (int c = 0; c <= NS; c++) out[c] = res[c];
-    return true;
+    return ok != 0;
 }
 
 // Several independent solves share one launch: run r owns the blocks
@@ -851,268 +926,312 @@ struct PcgBatch {
     PcgArgs run[MAXR];
 };
 
-// Per-block context of one solve: the block's place in its run, the slice
-// headers it caches, the barrier epoch and the shared reduction buffers.
+// Scalars of an iteration, formed by one thread of the block
+struct CgScalars {
+    double alpha, ralpha, rgamma, beta;   // in this order (lanes 0..3); ralpha = 1 / alpha, rgamma = 1 / gamma
+    double gamma, rr, bb, stop;           // stop: r.r at which the solve ends
+    float alpha32, beta32;
+    int iters, done, failed;
+};
+
+// first slice whose offset sp[] is at least `target` (all lanes of a warp;
+// 32 probes a round)
+__device__ __forceinline__ int find_slice(const int *__restrict__ sp, int ns, long target) {
+    const int lane = threadIdx.x & 31;
+    int lo = 0, hi = ns;
+    while (lo < hi) {
+        const int step = (hi - lo + 31) >> 5, p = lo + lane * step;
+        const bool reached = p >= hi || sp[p] >= target;
+        const int f = __ffs(__ballot_sync(0xFFFFFFFFu, reached)) - 1;   // 0..32 (-1: none)
+        const int last = f < 0 ? 31 : f - 1;                            // the last probe below the target
+        if (f >= 0) hi = min(hi, lo + f * step);
+        if (last >= 0) lo = lo + last * step + 1;
+    }
+    return lo;
+}
+
+// Per-block context of one solve.  The slices are dealt to the run's warps in
+// contiguous runs of equal numbers of entries; of the block's T / 32 warps,
+// `warps` take part (all of them unless the system has fewer slices than the
+// run has warps: a small system is spread over the run's blocks first, since
+// its iterations are bound by the latency and the FP64 rate of each SM).
+template <bool WIDE, int T, int RING>
 struct SolveCtx {
+    static constexpr int W = T / 32;
+    template <typename V>
+    using S = Stream<V, WIDE, RING, false>;
+    using S64 = S<double>;
+    using S32 = S<float>;
     const PcgArgs *a;
-    int nb, bid, lane, warp, sl0, sls;
-    bool cached;
-    int *s_sp, *s_sw;
+    int nb, bid, lane, warp, active;
+    int slice0;                  // first slice of the block
+    bool cached;                 // its slices' widths are in shared memory
+    const unsigned short *s_width;
     double *shv;
     unsigned long long *shm;
+    CgScalars *sc;
     unsigned int epoch;
-    __device__ void slice(int k, int sl, int &off, int &wid) const {
-        if (cached) {
-            off = s_sp[k * kSlicesPerBlock + warp];
-            wid = s_sw[k * kSlicesPerBlock + warp];
-        } else {
-            off = a->sp[sl];
-            wid = a->sw[sl];
-        }
-    }
-    // SpMV one slice at a time (unrolled by 8), f(i, sum_j A_ij v_j, v_i):
-    // the form of the FP64 PCG.  (The SpMV forms below were chosen by
-    // measurement, each kernel with the form it ran fastest in: the code the
-    // compiler makes of these loops at 64 registers is sensitive to their
-    // shape, by up to 40% in time.)
-    template <typename T, typename F>
-    __device__ __forceinline__ void spmv1(const T *__restrict__ Av, const T *v, F f) const {
-        const int *__restrict__ col = a->col;
-        const int n = a->n, ns = a->n_slices;
-        int off = 0, wid = 0;
-        if (sl0 < ns) slice(0, sl0, off, wid);
-        for (int k = 0, sl = sl0; sl < ns; k++, sl += sls) {
-            int noff = 0, nwid = 0;
-            if (sl + sls < ns) slice(k + 1, sl + sls, noff, nwid);
-            const int i = sl * 32 + lane;
-            const T vi = i < n ? v[i] : (T)0;
-            T acc = 0;
-            const int kb = off + lane;
-#pragma unroll 8
-            for (int j = 0; j < wid; j++) acc = fma(Av[kb + 32 * j], __ldcg(v + col[kb + 32 * j]), acc);
-            if (i < n) f(i, acc, vi);
-            off = noff;
-            wid = nwid;
-        }
-    }
-    // SpMV over the warp's slices with values Av: f(i, sum_j A_ij v_j, v_i):
-    // the form of the MIXED refinement (FP32 corrections, FP64 residuals).
-    // Two of the warp's slices at a time (two independent chains of loads in
-    // flight); the row's own v_i is read with the row's entries.  The matrix
-    // streams through once per iteration and is loaded evict-first, while
-    // the vector's gathers are plain loads that L1 may keep (coherent: the
-    // grid barrier before each phase is a release/acquire pair, so they see
-    // the other blocks' writes; the read-only path would not be): 4.79 ->
-    // 4.55 ms per MIXED Newmark solve on the 64^3 plasma ball, against
-    // 4.62 ms with the gathers bypassing L1.
-    template <typename T, typename F>
-    __device__ __forceinline__ void spmv(const T *__restrict__ Av, const T *v, F f) const {
-        const int *__restrict__ col = a->col;
-        const int n = a->n, ns = a->n_slices;
-        for (int k = 0, sl = sl0; sl < ns; k += 2, sl += 2 * sls) {
-            const bool hb = sl + sls < ns;
-            int offa, wida, offb = 0, widb = 0;
-            slice(k, sl, offa, wida);
-            if (hb) slice(k + 1, sl + sls, offb, widb);
-            const int ia = sl * 32 + lane, ib = (sl + sls) * 32 + lane;
-            const T va = ia < n ? v[ia] : (T)0;
-            const T vb = hb && ib < n ? v[ib] : (T)0;
-            T acca = 0, accb = 0;
-            const int ka = offa + lane, kb = offb + lane, wmin = min(wida, widb);
-            // joint unroll: 2 for FP32 values, 8 for FP64 (measured best of 2, 4, 8)
-            constexpr int kU = std::is_same<T, float>::value ? 2 : 8;
-            int j = 0;
-#pragma unroll kU
-            for (; j < wmin; j++) {
-                acca = fma(__ldcs(Av + ka + 32 * j), v[__ldcs(col + ka + 32 * j)], acca);
-                accb = fma(__ldcs(Av + kb + 32 * j), v[__ldcs(col + kb + 32 * j)], accb);
-            }
-#pragma unroll 4
-            for (int ja = j; ja < wida; ja++) acca = fma(__ldcs(Av + ka + 32 * ja), v[__ldcs(col + ka + 32 * ja)], acca);
-#pragma unroll 4
-            for (int jb = j; jb < widb; jb++) accb = fma(__ldcs(Av + kb + 32 * jb), v[__ldcs(col + kb + 32 * jb)], accb);
-            if (ia < n) f(ia, acca, va);
-            if (hb && ib < n) f(ib, accb, vb);
-        }
+    WarpStream ws;
+    __device__ __forceinline__ int width(int sl) const { return cached ? (int)s_width[sl - slice0] : a->sw[sl]; }
+    // (a copy that does not arrive raises the run's timeout flag, which every
+    // block sees after the next grid reduction)
+    template <typename V, typename F>
+    __device__ __forceinline__ void spmv(const unsigned char *recs, const V *v, bool more, F f) {
+        if (!S<V>::pass(ws, recs, v, more, [&](int sl) { return width(sl); }, f) && lane == 0)
+            atomicExch(&a->gb->timeout, 1);
     }
 };
 
-struct CgOut {
-    int iters;
-    bool failed;
-    double rr, gamma, bb;
+// 16 bytes of a vector: four FP32 or two FP64 consecutive rows of one lane
+template <typename V>
+struct Pack {
+    static constexpr int n = 16 / (int)sizeof(V);
+    V v[n];
+    __device__ __forceinline__ void load(const V *p) {
+        const int4 t = *reinterpret_cast<const int4 *>(p);
+        memcpy(v, &t, 16);
+    }
+    __device__ __forceinline__ void store(V *p) const {
+        int4 t;
+        memcpy(&t, v, 16);
+        *reinterpret_cast<int4 *>(p) = t;
+    }
+    __device__ __forceinline__ void zero() {
+#pragma unroll
+        for (int k = 0; k < n; k++) v[k] = 0;
+    }
 };
 
-// Chronopoulos-Gear Jacobi-PCG on the context's matrix with values Av in
-// precision T: x, r, u = D^-1 r, w = A u, p, s = A p.  With UNIT the matrix
-// has a unit diagonal (a diagonally scaled system): u is r itself (the caller
-// passes r for u), and neither D^-1 nor u is read or written.  Per-thread
-// sums are kept in T and the block and grid reductions in FP64 (in FP32 the
-// per-thread sums cover about a dozen rows).  max|r| is tracked in FP64 only.
-// Returns false if a barrier timed out.
-template <typename T, bool UNIT = false>
-__device__ __forceinline__ bool cg_core(SolveCtx &c, const T *__restrict__ Av, const T *__restrict__ Dinv,
-                                        const T *b, T *x, T *r, T *u, T *w, T *p, T *s, bool x_zero, double tol2,
-                                        double abs_inf, int max_iters, CgOut &o) {
-    constexpr bool kMax = std::is_same<T, double>::value;
+// Chronopoulos-Gear Jacobi-PCG on the context's matrix (records in precision
+// V): x, r, u = D^-1 r, w = A u, p, s = A p.  With UNIT the matrix has a unit
+// diagonal (a diagonally scaled system): u is r itself (the caller passes r
+// for u), and neither D^-1 nor u is read or written.  Per-thread sums are kept
+// in V and the block and grid reductions in FP64 (in FP32 the per-thread sums
+// cover a few dozen rows, in four chains).  max|r| is tracked in FP64 only.
+// The stream of the records is running (begun by the caller, which also ends
+// it); the results are left in the context's scalars.  Returns false if a
+// wait ran out.
+template <typename V, bool UNIT, bool WIDE, int T, int RING>
+__device__ __forceinline__ bool cg_core(SolveCtx<WIDE, T, RING> &c, const unsigned char *recs,
+                                        const V *__restrict__ Dinv, const V *b, V *x, V *r, V *u, V *w, V *p, V *s,
+                                        bool x_zero, double tol2, double abs_inf, int max_iters) {
+    constexpr bool kF64 = std::is_same<V, double>::value;
+    constexpr int E = Pack<V>::n;
     const PcgArgs &a = *c.a;
-    const int n = a.n, lane = c.lane;
-    double t[5];
+    CgScalars *sc = c.sc;
+    const int row0 = 32 * c.ws.s0 + E * c.lane, row1 = 32 * c.ws.s1;   // the lane's packs: row0, row0 + 32 E, ...
     {
-        T v[4] = {0, 0, 0, 0};   // gamma, rr, delta, bb
+        V v[4] = {0, 0, 0, 0};   // gamma, rr, delta, bb
         unsigned long long mx = 0;
-        auto init_row = [&](int i, T ax, T) {
-            const T bi = b[i], ri = bi - ax;
-            T ui;
+        auto init_row = [&](int i, V bi, V ri) {
+            V ui;
             if constexpr (UNIT) ui = ri;
             else ui = Dinv[i] * ri;
-            if (x_zero) x[i] = 0;
             r[i] = ri;
             if constexpr (!UNIT) u[i] = ui;
             v[0] = fma(ri, ui, v[0]);
             v[1] = fma(ri, ri, v[1]);
             v[3] = fma(bi, bi, v[3]);
-            if constexpr (kMax) mx = max(mx, abs_bits(ri));
+            if constexpr (kF64) mx = max(mx, abs_bits(ri));
         };
         if (x_zero) {
-            for (int sl = c.sl0; sl < a.n_slices; sl += c.sls)
-                if (sl * 32 + lane < n) init_row(sl * 32 + lane, (T)0, (T)0);
+            for (int i = 32 * c.ws.s0 + c.lane; i < row1; i += 32) {
+                const V bi = b[i];
+                x[i] = 0;
+                init_row(i, bi, bi);
+            }
         } else {
-            if constexpr (std::is_same<T, double>::value) c.spmv1(Av, x, init_row);
-            else c.spmv(Av, x, init_row);
+            c.template spmv<V>(recs, x, true, [&](int i, V ax, V) {
+                const V bi = b[i];
+                init_row(i, bi, bi - ax);
+            });
         }
         if (!grid_barrier(a.gb, ++c.epoch, c.nb, a.spin_limit)) return false;
-        auto wrow = [&](int i, T au, T ui) {
+        c.template spmv<V>(recs, u, true, [&](int i, V au, V ui) {
             w[i] = au;
             v[2] = fma(au, ui, v[2]);
-        };
-        if constexpr (std::is_same<T, double>::value) c.spmv1(Av, u, wrow);
-        else c.spmv(Av, u, wrow);
-        const double vd[4] = {(double)v[0], (double)v[1], (double)v[2], (double)v[3]};
-        if (!grid_reduce<4>(a.gb, a.part, vd, mx, c.shv, c.shm, ++c.epoch, t, c.nb, c.bid, a.spin_limit)) return false;
+        });
+        if (!grid_reduce<4, T>(a.gb, a.part, v, mx, c.shv, c.shm, ++c.epoch, c.nb, c.bid, c.active, a.spin_limit,
+                               [&](const double *t, int wp, int l) {
+                                   if (wp == 0) {
+                                       const double q = (l == 0 ? t[0] : l == 1 ? t[2] : 1.0) / (l == 0 ? t[2] : t[0]);
+                                       if (l < 3) (&sc->alpha)[l] = q;
+                                       if (l == 0) sc->alpha32 = (float)q;
+                                   } else if (l == 0) {
+                                       sc->beta = 0.0;
+                                       sc->beta32 = 0.0f;
+                                       sc->gamma = t[0];
+                                       sc->rr = t[1];
+                                       sc->bb = t[3];
+                                       sc->stop = tol2 * t[3];
+                                       sc->iters = 0;
+                                       sc->failed = 0;
+                                       sc->done = (t[3] == 0.0) || (t[1] <= sc->stop) || (t[4] <= abs_inf);
+                                       if (!sc->done && max_iters <= 0) sc->done = sc->failed = 1;
+                                   }
+                               }))
+            return false;
     }
-    double gamma = t[0], rr = t[1];
-    const double bb = t[3];
-    double alpha = t[0] / t[2], beta = 0.0;
-    bool done = (bb == 0.0) || (rr <= tol2 * bb) || (t[4] <= abs_inf);
-    if (bb == 0.0)
-        for (int sl = c.sl0; sl < a.n_slices; sl += c.sls)
-            if (sl * 32 + lane < n) x[sl * 32 + lane] = 0;
-    int iters = 0;
-    bool failed = false;
-    while (!done) {
-        if (iters >= max_iters) {
-            failed = true;
-            break;
+    if (sc->bb == 0.0)
+        for (int i = 32 * c.ws.s0 + c.lane; i < row1; i += 32) x[i] = 0;
+    while (!sc->done) {
+        const bool first = sc->iters == 0;
+        V al, be;
+        if constexpr (kF64) {
+            al = sc->alpha;
+            be = sc->beta;
+        } else {
+            al = sc->alpha32;
+            be = sc->beta32;
         }
-        const bool first = iters == 0;
-        const T al = (T)alpha, be = (T)beta;
         // ---- p = u + beta p, s = w + beta s, x += alpha p, r -= alpha s, u = D^-1 r ----
-        // kVecSlices of the warp's slices at a time, every load issued before
-        // the first store (the vectors may alias as far as the compiler knows)
-        T v[3] = {0, 0, 0};   // gamma, rr, delta
+        // 16 bytes a load, every load before the first store
+        V vg[E], vr[E];   // gamma, rr: a chain per element of the pack
+#pragma unroll
+        for (int k = 0; k < E; k++) vg[k] = vr[k] = 0;
         unsigned long long mx = 0;
-        for (int sl = c.sl0; sl < a.n_slices; sl += kVecSlices * c.sls) {
-            T q[kVecSlices][7];   // u w p s x r D^-1
-#pragma unroll
-            for (int h = 0; h < kVecSlices; h++) {
-#pragma unroll
-                for (int k = 0; k < 7; k++) q[h][k] = 0;
-                const int slh = sl + h * c.sls, i = slh * 32 + lane;
-                if (slh < a.n_slices && i < n) {
-                    q[h][1] = w[i];
-                    if (!first) {
-                        q[h][2] = p[i];
-                        q[h][3] = s[i];
-                    }
-                    q[h][4] = x[i];
-                    q[h][5] = r[i];
-                    if constexpr (UNIT) {
-                        q[h][0] = q[h][5];
-                    } else {
-                        q[h][0] = u[i];
-                        q[h][6] = Dinv[i];
-                    }
-                }
+#pragma unroll 2
+        for (int i = row0; i < row1; i += 32 * E) {
+            Pack<V> qu, qw, qp, qs, qx, qr, qd;
+            qw.load(w + i);
+            qr.load(r + i);
+            qx.load(x + i);
+            qp.zero();
+            qs.zero();
+            if (!first) {
+                qp.load(p + i);
+                qs.load(s + i);
+            }
+            if constexpr (UNIT) {
+                qu = qr;
+            } else {
+                qu.load(u + i);
+                qd.load(Dinv + i);
             }
 #pragma unroll
-            for (int h = 0; h < kVecSlices; h++) {
-                const int slh = sl + h * c.sls, i = slh * 32 + lane;
-                if (slh < a.n_slices && i < n) {
-                    const T pi = first ? q[h][0] : fma(be, q[h][2], q[h][0]);
-                    const T si = first ? q[h][1] : fma(be, q[h][3], q[h][1]);
-                    const T ri = fma(-al, si, q[h][5]);
-                    T un;
-                    if constexpr (UNIT) un = ri;
-                    else un = q[h][6] * ri;
-                    p[i] = pi;
-                    s[i] = si;
-                    x[i] = fma(al, pi, q[h][4]);
-                    r[i] = ri;
-                    if constexpr (!UNIT) u[i] = un;
-                    v[0] = fma(ri, un, v[0]);
-                    v[1] = fma(ri, ri, v[1]);
-                    if constexpr (kMax) mx = max(mx, abs_bits(ri));
-                }
+            for (int k = 0; k < E; k++) {
+                const V pi = first ? qu.v[k] : fma(be, qp.v[k], qu.v[k]);
+                const V si = first ? qw.v[k] : fma(be, qs.v[k], qw.v[k]);
+                const V ri = fma(-al, si, qr.v[k]);
+                V un;
+                if constexpr (UNIT) un = ri;
+                else un = qd.v[k] * ri;
+                qp.v[k] = pi;
+                qs.v[k] = si;
+                qx.v[k] = fma(al, pi, qx.v[k]);
+                qr.v[k] = ri;
+                qu.v[k] = un;
+                vg[k] = fma(ri, un, vg[k]);
+                vr[k] = fma(ri, ri, vr[k]);
+                if constexpr (kF64) mx = max(mx, abs_bits(ri));
             }
+            qp.store(p + i);
+            qs.store(s + i);
+            qx.store(x + i);
+            qr.store(r + i);
+            if constexpr (!UNIT) qu.store(u + i);
         }
         if (!grid_barrier(a.gb, ++c.epoch, c.nb, a.spin_limit)) return false;
         // ---- w = A u ----
-        auto wrow = [&](int i, T au, T ui) {
+        V v2 = 0;   // delta
+        c.template spmv<V>(recs, u, true, [&](int i, V au, V ui) {
             w[i] = au;
-            v[2] = fma(au, ui, v[2]);
-        };
-        if constexpr (std::is_same<T, double>::value) c.spmv1(Av, u, wrow);
-        else c.spmv(Av, u, wrow);
-        const double vd[3] = {(double)v[0], (double)v[1], (double)v[2]};
-        if (!grid_reduce<3>(a.gb, a.part, vd, mx, c.shv, c.shm, ++c.epoch, t, c.nb, c.bid, a.spin_limit)) return false;
-        iters++;
-        rr = t[1];
-        done = (rr <= tol2 * bb) || (t[3] <= abs_inf);
-        const double gnew = t[0];
-        beta = gnew / gamma;
-        alpha = gnew / (t[2] - beta * gnew / alpha);
-        gamma = gnew;
+            v2 = fma(au, ui, v2);
+        });
+        V vd[3];
+        if constexpr (UNIT) {   // u is r: gamma is rr
+            vd[0] = (vg[0] + vg[1]) + (vg[2] + vg[3]);
+            vd[1] = vd[0];
+        } else {
+            vd[0] = vg[0] + vg[1];
+            vd[1] = vr[0] + vr[1];
+        }
+        vd[2] = v2;
+        // beta = gamma'/gamma, alpha = gamma' / (delta - beta gamma' / alpha)
+        if (!grid_reduce<3, T>(a.gb, a.part, vd, mx, c.shv, c.shm, ++c.epoch, c.nb, c.bid, c.active, a.spin_limit,
+                               [&](const double *t, int wp, int l) {
+                                   if (wp == 0) {
+                                       const double be = t[0] * sc->rgamma, den = t[2] - be * t[0] * sc->ralpha;
+                                       __syncwarp();
+                                       const double q = (l == 0 ? t[0] : l == 1 ? den : 1.0) / (l == 0 ? den : t[0]);
+                                       const double o = l == 3 ? be : q;
+                                       if (l < 4) (&sc->alpha)[l] = o;
+                                       const float f = (float)o;
+                                       if (l == 0) sc->alpha32 = f;
+                                       if (l == 3) sc->beta32 = f;
+                                   } else if (l == 0) {
+                                       sc->gamma = t[0];
+                                       sc->rr = t[1];
+                                       const int it = ++sc->iters;
+                                       int done = (t[1] <= sc->stop) || (t[3] <= abs_inf);
+                                       if (!done && it >= max_iters) done = sc->failed = 1;
+                                       sc->done = done;
+                                   }
+                               }))
+            return false;
     }
-    o.iters = iters;
-    o.failed = failed;
-    o.rr = rr;
-    o.gamma = gamma;
-    o.bb = bb;
     return true;
 }
 
-// the whole solve, run by block `bid` of the nb blocks that own it: FP64
-// PCG (REFINE false) or the MIXED refinement (REFINE true, a.refine set).
-// The two are separate kernels so that each gets the register allocation of
-// its own loops.
-template <bool REFINE>
-__device__ __forceinline__ void pcg_body(const PcgArgs &a, const int nb, const int bid) {
-    __shared__ double shv[4 * kThreads];
-    __shared__ unsigned long long shm[kThreads];
-    __shared__ int s_sp[kSmemSlices], s_sw[kSmemSlices];
-    SolveCtx c;
+// the whole solve, run by block `bid` (T threads) of the nb blocks that own
+// it: FP64 PCG (REFINE false) or the MIXED refinement (REFINE true, a.refine
+// set).  The two are separate kernels so that each gets the register
+// allocation of its own loops.  ring: RING bytes of shared memory per warp.
+template <bool REFINE, bool WIDE, int T, int RING>
+__device__ __forceinline__ void pcg_body(const PcgArgs &a, const int nb, const int bid, unsigned char *ring, double *shv,
+                                         unsigned long long *shm) {
+    constexpr int W = T / 32;
+    __shared__ unsigned short s_width[kSmemSlices];
+    __shared__ __align__(8) unsigned long long s_bars[W][kMaxStages];
+    __shared__ CgScalars scal;
+    __shared__ int s_range[2];
+    struct Refine {
+        double rr, bb, sigma, inv;
+        int stop, failed, total;
+    };
+    __shared__ Refine rf;
+    using Ctx = SolveCtx<WIDE, T, RING>;
+    Ctx c;
     c.a = &a;
     c.nb = nb;
     c.bid = bid;
     c.lane = threadIdx.x & 31;
     c.warp = threadIdx.x >> 5;
-    c.sl0 = bid * kSlicesPerBlock + c.warp;
-    c.sls = nb * kSlicesPerBlock;
-    c.s_sp = s_sp;
-    c.s_sw = s_sw;
     c.shv = shv;
     c.shm = shm;
+    c.sc = &scal;
     c.epoch = 0;
-    // the block's slice headers, k-th slice of warp `warp` at k * 8 + warp
-    c.cached = (long)((a.n_slices + c.sls - 1) / c.sls) * kSlicesPerBlock <= kSmemSlices;
-    if (c.cached)
-        for (int k = 0, sl = c.sl0; sl < a.n_slices; k++, sl += c.sls)
-            if (c.lane == 0) {
-                s_sp[k * kSlicesPerBlock + c.warp] = a.sp[sl];
-                s_sw[k * kSlicesPerBlock + c.warp] = a.sw[sl];
+    {
+        const int warps = min(W, (a.n_slices + nb - 1) / nb);   // the block's warps that take part
+        const int gw = bid * warps + c.warp, total = nb * warps;
+        const long cols = a.sp[a.n_slices] >> 5;
+        c.active = warps;
+        WarpStream &w = c.ws;
+        w.s0 = w.s1 = w.rec0 = w.nrec = w.skip = w.stage = w.inflight = w.next = 0;
+        w.parity = 0;
+        if (c.warp < warps) {
+            w.s0 = find_slice(a.sp, a.n_slices, cols * gw / total * 32);
+            w.s1 = find_slice(a.sp, a.n_slices, cols * (gw + 1) / total * 32);
+            if (w.s1 > w.s0) {
+                const int k0 = a.sp[w.s0] >> 5, k1 = a.sp[w.s1] >> 5;
+                w.rec0 = k0 / kCols;
+                w.nrec = (k1 + kCols - 1) / kCols - w.rec0;
+                w.skip = k0 - w.rec0 * kCols;
             }
-    __syncwarp();
+        }
+        w.ring = smem_u32(ring) + (uint32_t)(c.warp * RING);
+        w.bars = smem_u32(&s_bars[c.warp][0]);
+        w.policy = a.evict_first ? policy_evict_first() : policy_evict_normal();
+        if (c.lane == 0 && c.warp == 0) s_range[0] = w.s0;
+        if (c.lane == 0 && c.warp == warps - 1) s_range[1] = w.s1;
+        __syncthreads();
+        c.slice0 = s_range[0];
+        c.cached = s_range[1] - s_range[0] <= kSmemSlices;
+        c.s_width = s_width;
+        if (c.cached)
+            for (int sl = w.s0 + c.lane; sl < w.s1; sl += 32) s_width[sl - c.slice0] = (unsigned short)a.sw[sl];
+        __syncwarp();
+    }
     CgState *st = a.st;
     double abs_inf = a.abs_inf, tol2 = a.tol2;
     if (a.abs_src) {
@@ -1120,12 +1239,13 @@ __device__ __forceinline__ void pcg_body(const PcgArgs &a, const int nb, const i
         if (qv > 0.0) abs_inf = a.abs_factor * qv;
         else tol2 = a.fallback_tol2;
     }
-    CgOut o{0, false, 0.0, 0.0, 0.0};
     int outer = 0;
+    bool good = true;
     if constexpr (!REFINE) {
-        if (!cg_core<double>(c, a.Av, a.Dinv, a.b, a.x, a.r, a.u, a.w, a.p, a.s, a.x_zero != 0, tol2, abs_inf,
-                             a.max_iters, o))
-            goto timeout;
+        Ctx::S64::begin(c.ws, a.rec, 1 << 30);
+        good = cg_core<double, false, WIDE, T, RING>(c, a.rec, a.Dinv, a.b, a.x, a.r, a.u, a.w, a.p, a.s, a.x_zero != 0,
+                                                     tol2, abs_inf, a.max_iters);
+        good = Ctx::S64::end(c.ws) && good;
     } else {
         // Iterative refinement: the FP64 residual b - A x decides; each
         // correction A d = r / sigma is solved in FP32 (values and vectors) to
@@ -1138,70 +1258,69 @@ __device__ __forceinline__ void pcg_body(const PcgArgs &a, const int nb, const i
         // FP32 subnormal range.  (Stopping a correction solve at what the
         // stopping rule still asks saves FP32 iterations but leaves the
         // completion more to do, at a higher price per order of magnitude.)
-        const int n = a.n;
-        int total = 0;
-        bool failed = false;
-        double rr = 0.0, bb = 0.0;
+        const int n = a.n, row0 = 32 * c.ws.s0 + c.lane, row1 = 32 * c.ws.s1;
+        if (threadIdx.x == 0) {
+            rf.failed = 0;
+            rf.total = 0;
+        }
         while (true) {
-            if (outer > 0 && !grid_barrier(a.gb, ++c.epoch, nb, a.spin_limit)) goto timeout;   // x complete
-            double t[3];
-            {
+            Ctx::S64::begin(c.ws, a.rec, c.ws.nrec);   // on its way while the blocks meet
+            if (outer > 0 && good) good = grid_barrier(a.gb, ++c.epoch, nb, a.spin_limit);   // x complete
+            if (good) {
                 double v2[2] = {0.0, 0.0};
-                c.spmv(a.Av, a.x, [&](int i, double ax, double) {
+                c.template spmv<double>(a.rec, a.x, false, [&](int i, double ax, double) {
                     const double bi = a.b[i], ri = bi - ax;
                     a.r[i] = ri;
                     v2[0] = fma(ri, ri, v2[0]);
                     v2[1] = fma(bi, bi, v2[1]);
                 });
-                if (!grid_reduce<2>(a.gb, a.part, v2, 0ull, shv, shm, ++c.epoch, t, nb, bid, a.spin_limit)) goto timeout;
+                good = grid_reduce<2, T>(a.gb, a.part, v2, 0ull, shv, shm, ++c.epoch, nb, bid, c.active, a.spin_limit,
+                                         [&](const double *t, int wp, int l) {
+                                             if (wp + l != 0) return;
+                                             rf.rr = t[0];
+                                             rf.bb = t[1];
+                                             rf.stop = t[1] == 0.0 || t[0] <= tol2 * t[1];
+                                             if (!rf.stop && (rf.total >= a.max_iters || outer >= kMaxOuter))
+                                                 rf.stop = rf.failed = 1;
+                                             rf.sigma = sqrt(t[0] / n);
+                                             rf.inv = 1.0 / rf.sigma;
+                                         });
             }
-            rr = t[0];
-            bb = t[1];
-            if (bb == 0.0 || rr <= tol2 * bb) break;
-            if (total >= a.max_iters || outer >= kMaxOuter) {
-                failed = true;
-                break;
-            }
-            const double sigma = sqrt(rr / n), inv = 1.0 / sigma;
-            for (int sl = c.sl0; sl < a.n_slices; sl += c.sls) {
-                const int i = sl * 32 + c.lane;
-                if (i < n) a.b32[i] = (float)(a.r[i] * inv) * a.Dhalf32[i];
-            }
-            CgOut oi{0, false, 0.0, 0.0, 0.0};
-            if (!cg_core<float, true>(c, a.Av32, a.Dhalf32, a.b32, a.d32, a.r32, a.r32, a.w32, a.p32, a.s32, true,
-                                a.inner_tol2, -1.0, min(kMaxInner, a.max_iters - total), oi))
-                goto timeout;
-            total += oi.iters;
+            good = Ctx::S64::end(c.ws) && good;
+            if (!good || rf.stop) break;
+            Ctx::S32::begin(c.ws, a.rec32, 1 << 30);
+            const double sigma = rf.sigma, inv = rf.inv;
+            for (int i = row0; i < row1; i += 32) a.b32[i] = (float)(a.r[i] * inv) * a.Dhalf32[i];
+            good = cg_core<float, true, WIDE, T, RING>(c, a.rec32, a.Dhalf32, a.b32, a.d32, a.r32, a.r32, a.w32, a.p32,
+                                                       a.s32, true, a.inner_tol2, -1.0,
+                                                       min(kMaxInner, a.max_iters - rf.total));
+            good = Ctx::S32::end(c.ws) && good;
+            if (!good) break;
             outer++;
-            for (int sl = c.sl0; sl < a.n_slices; sl += c.sls) {
-                const int i = sl * 32 + c.lane;
-                if (i < n) a.x[i] = fma(sigma * (double)a.Dhalf32[i], (double)a.d32[i], a.x[i]);
-            }
+            for (int i = row0; i < row1; i += 32)
+                a.x[i] = fma(sigma * (double)a.Dhalf32[i], (double)a.d32[i], a.x[i]);
+            __syncthreads();   // every thread has read rf.total
+            if (threadIdx.x == 0) rf.total += scal.iters;
         }
-        if (bb == 0.0)
-            for (int sl = c.sl0; sl < a.n_slices; sl += c.sls)
-                if (sl * 32 + c.lane < n) a.x[sl * 32 + c.lane] = 0.0;
-        o.iters = total;
-        o.failed = failed;
-        o.rr = rr;
-        o.bb = bb;
+        if (good && rf.bb == 0.0)
+            for (int i = row0; i < row1; i += 32) a.x[i] = 0.0;
     }
     if (bid == 0 && threadIdx.x == 0) {
-        st->iters = o.iters;
+        if (!good) {
+            st->done = 1;
+            st->failed = 1;
+            atomicOr(a.status, (uint32_t)ST_BARRIER);
+            return;
+        }
+        const int failed = REFINE ? rf.failed : scal.failed;
+        st->iters = REFINE ? rf.total : scal.iters;
         st->outer = outer;
-        st->rr = o.rr;
-        st->rz = o.gamma;
-        st->bb = o.bb;
+        st->rr = REFINE ? rf.rr : scal.rr;
+        st->rz = REFINE ? 0.0 : scal.gamma;
+        st->bb = REFINE ? rf.bb : scal.bb;
         st->done = 1;
-        st->failed = o.failed ? 1 : 0;
-        if (o.failed && !a.quiet) atomicOr(a.status, (uint32_t)ST_CG_NO_CONV);
-    }
-    return;
-timeout:
-    if (bid == 0 && threadIdx.x == 0) {
-        st->done = 1;
-        st->failed = 1;
-        atomicOr(a.status, (uint32_t)ST_BARRIER);
+        st->failed = failed;
+        if (failed && !a.quiet) atomicOr(a.status, (uint32_t)ST_CG_NO_CONV);
     }
 }
 
@@ -1296,20 +1415,43 @@ __device__ __forceinline__ float half_row_dot(const int *__restrict__ ptr, const
     return s;
 }
 
-// the whole solve, run by block `bid` of the nb blocks that own it
-__device__ __forceinline__ void mg_body(const MgArgs &a, const int nb, const int bid) {
-    __shared__ double shv[4 * kThreads];
-    __shared__ unsigned long long shm[kThreads];
-    const int G = nb * kThreads, gt = bid * kThreads + threadIdx.x;
+// the whole solve, run by block `bid` (T threads) of the nb blocks that own
+// it; the scalars are formed by one thread per block (see grid_reduce)
+template <int T>
+__device__ __forceinline__ void mg_body(const MgArgs &a, const int nb, const int bid, double *shv,
+                                        unsigned long long *shm) {
+    struct Scalars {
+        double thr, tol2, bb, rr, rz, rzo, alpha, beta, zs;
+        float inv;
+        int it, done, failed;
+    };
+    __shared__ Scalars sc;
+    const int G = nb * T, gt = bid * T + threadIdx.x;
     const int lane = threadIdx.x & 31, nw = G >> 5, gw = gt >> 5;
     const long lim = a.spin_limit;
     unsigned int epoch = 0;
-    double thr = -1.0, tol2 = a.fallback_tol2;
-    if (a.abs_src) {
-        const double qv = *a.abs_src;
-        if (qv > 0.0) thr = a.abs_factor * qv;
+    if (threadIdx.x == 0) {
+        sc.thr = -1.0;
+        sc.tol2 = a.fallback_tol2;
+        if (a.abs_src) {
+            const double qv = *a.abs_src;
+            if (qv > 0.0) sc.thr = a.abs_factor * qv;
+        }
+        sc.it = 0;
+        sc.failed = 0;
+        sc.rzo = 0.0;
     }
-    double t[4];
+    // after a residual: |r|^2 = t[0], max|r| = t[1]; sigma scales the next V-cycle
+    auto residual = [&](const double *t, int wp, int l) {
+        if (wp + l != 0) return;
+        sc.rr = t[0];
+        int done = sc.bb == 0.0 || (sc.thr >= 0.0 ? t[1] <= sc.thr : t[0] <= sc.tol2 * sc.bb);
+        if (!done && sc.it >= a.max_iters) done = sc.failed = 1;
+        sc.done = done;
+        const double sigma = t[1] > 0.0 ? t[1] : 1.0;
+        sc.inv = (float)(1.0 / sigma);
+        sc.zs = sigma * a.s0;
+    };
     // x = 0, r = b; |b|^2 and max|r|
     {
         double v[1] = {0.0};
@@ -1321,21 +1463,16 @@ __device__ __forceinline__ void mg_body(const MgArgs &a, const int nb, const int
             v[0] += bi * bi;
             mx = max(mx, abs_bits(bi));
         }
-        if (!grid_reduce<1>(a.gb, a.part, v, mx, shv, shm, ++epoch, t, nb, bid, lim)) goto timeout;
+        if (!grid_reduce<1, T>(a.gb, a.part, v, mx, shv, shm, ++epoch, nb, bid, T / 32, lim, [&](const double *t, int wp, int l) {
+                if (wp + l == 0) sc.bb = t[0];
+                residual(t, wp, l);
+            }))
+            goto timeout;
     }
     {
-        const double bb = t[0];
-        double rmax = t[1], rr = bb, rz_old = 0.0;
-        int it = 0;
-        bool failed = false;
-        auto converged = [&]() { return bb == 0.0 || (thr >= 0.0 ? rmax <= thr : rr <= tol2 * bb); };
-        while (!converged()) {
-            if (it >= a.max_iters) {
-                failed = true;
-                break;
-            }
-            const double sigma = rmax > 0.0 ? rmax : 1.0;
-            const float inv = (float)(1.0 / sigma);
+        while (!sc.done) {
+            const bool first = sc.it == 0;
+            const float inv = sc.inv;
             // V1: scaled residual r32, the first Jacobi sweep z0 = w0 r32 and
             // t0 = r32 - L z0, with the neighbours' z0 formed from r on the fly
             // (no barrier between the sweep and the residual)
@@ -1473,7 +1610,7 @@ __device__ __forceinline__ void mg_body(const MgArgs &a, const int nb, const int
             // V8: post-smoothing on level 0, z = sigma s0 z0 in FP64; (r, z), (r, z_old)
             {
                 double v[2] = {0.0, 0.0};
-                const double zs = sigma * a.s0;
+                const double zs = sc.zs;
                 for (int sl = gw; sl < a.n_slices; sl += nw) {
                     const int row = sl * 32 + lane, kb = a.sp[sl] + lane, kw = a.sw[sl];
                     float s = 0.0f;
@@ -1487,11 +1624,15 @@ __device__ __forceinline__ void mg_body(const MgArgs &a, const int nb, const int
                         a.z[row] = zi;
                     }
                 }
-                if (!grid_reduce<2>(a.gb, a.part, v, 0ull, shv, shm, ++epoch, t, nb, bid, lim)) goto timeout;
+                if (!grid_reduce<2, T>(a.gb, a.part, v, 0ull, shv, shm, ++epoch, nb, bid, T / 32, lim, [&](const double *t, int wp, int l) {
+                        if (wp + l != 0) return;
+                        sc.rz = t[0];
+                        sc.beta = sc.it == 0 ? 0.0 : (t[0] - t[1]) / sc.rzo;
+                        sc.rzo = t[0];
+                    }))
+                    goto timeout;
             }
-            const double rz = t[0];
-            const double beta = it == 0 ? 0.0 : (rz - t[1]) / rz_old;
-            rz_old = rz;
+            const double beta = sc.beta;
             // w = L z (z is complete: the reduction above was a grid barrier),
             // p = z + beta p, q = w + beta q (= L p), and (p, q)
             {
@@ -1503,17 +1644,22 @@ __device__ __forceinline__ void mg_body(const MgArgs &a, const int nb, const int
                     for (int j = 0; j < kw; j++) s = fma(a.Lv[kb + 32 * j], a.z[a.col[kb + 32 * j]], s);
                     if (row < a.n0) {
                         const double zi = a.z[row];
-                        const double pi = it == 0 ? zi : zi + beta * a.p[row];   // p, q not read before set
-                        const double qi = it == 0 ? s : s + beta * a.q[row];
+                        const double pi = first ? zi : zi + beta * a.p[row];   // p, q not read before set
+                        const double qi = first ? s : s + beta * a.q[row];
                         a.p[row] = pi;
                         a.q[row] = qi;
                         a.zo[row] = zi;
                         v[0] += pi * qi;
                     }
                 }
-                if (!grid_reduce<1>(a.gb, a.part, v, 0ull, shv, shm, ++epoch, t, nb, bid, lim)) goto timeout;
+                if (!grid_reduce<1, T>(a.gb, a.part, v, 0ull, shv, shm, ++epoch, nb, bid, T / 32, lim, [&](const double *t, int wp, int l) {
+                        if (wp + l != 0) return;
+                        sc.alpha = sc.rz / t[0];
+                        sc.it++;
+                    }))
+                    goto timeout;
             }
-            const double alpha = rz_old / t[0];
+            const double alpha = sc.alpha;
             // x += alpha p, r -= alpha q; |r|^2 and max|r|
             {
                 double v[1] = {0.0};
@@ -1525,19 +1671,16 @@ __device__ __forceinline__ void mg_body(const MgArgs &a, const int nb, const int
                     v[0] += ri * ri;
                     mx = max(mx, abs_bits(ri));
                 }
-                if (!grid_reduce<1>(a.gb, a.part, v, mx, shv, shm, ++epoch, t, nb, bid, lim)) goto timeout;
+                if (!grid_reduce<1, T>(a.gb, a.part, v, mx, shv, shm, ++epoch, nb, bid, T / 32, lim, residual)) goto timeout;
             }
-            rr = t[0];
-            rmax = t[1];
-            it++;
         }
         if (bid == 0 && threadIdx.x == 0) {
-            a.st->iters = it;
-            a.st->rr = rr;
-            a.st->bb = bb;
+            a.st->iters = sc.it;
+            a.st->rr = sc.rr;
+            a.st->bb = sc.bb;
             a.st->done = 1;
-            a.st->failed = failed ? 1 : 0;
-            if (failed) atomicOr(a.status, (uint32_t)ST_CG_NO_CONV);
+            a.st->failed = sc.failed;
+            if (sc.failed) atomicOr(a.status, (uint32_t)ST_CG_NO_CONV);
         }
         return;
     }
@@ -1549,31 +1692,43 @@ timeout:
     }
 }
 
-__global__ void __launch_bounds__(kThreads, 4) k_mg_pcg(const MgArgs a) { mg_body(a, gridDim.x, blockIdx.x); }
+__global__ void __launch_bounds__(kMgThreads, 1) k_mg_pcg(const MgArgs a) {
+    __shared__ double shv[4 * kMgThreads];
+    __shared__ unsigned long long shm[kMgThreads];
+    mg_body<kMgThreads>(a, gridDim.x, blockIdx.x, shv, shm);
+}
 
-// one solve per launch (its arguments passed by value)
-template <bool REFINE>
-__global__ void __launch_bounds__(kThreads, 4) k_pcg_persistent(const PcgArgs a) {
-    pcg_body<REFINE>(a, gridDim.x, blockIdx.x);
+// one solve per launch (its arguments passed by value), one block per SM
+extern __shared__ __align__(128) unsigned char s_ring[];
+template <bool REFINE, bool WIDE>
+__global__ void __launch_bounds__(PcgShape<REFINE, WIDE>::threads, 1) k_pcg_persistent(const PcgArgs a) {
+    using P = PcgShape<REFINE, WIDE>;
+    __shared__ double shv[4 * P::threads];
+    __shared__ unsigned long long shm[P::threads];
+    pcg_body<REFINE, WIDE, P::threads, P::ring>(a, gridDim.x, blockIdx.x, s_ring, shv, shm);
 }
 
 // several solves of one kind per launch: run r owns blocks [block0, block0 + blocks).
-// Built for MINB = 4 blocks per SM (64 registers), MINB = 3 (80: the
-// refinement form then keeps its state in registers), MINB = 6 (40) and
-// MINB = 8 (32: more warps to hide the latency of many small systems, at the
-// price of spills); a batch's tuner picks.
-template <bool REFINE, int MINB>
+// Built for MINB = 4 blocks per SM (64 registers) and MINB = 3 (80); a batch's
+// tuner picks.  ANYWIDE: some run's records are wide (the others' may be narrow).
+template <bool REFINE, int MINB, bool ANYWIDE>
 __global__ void __launch_bounds__(kThreads, MINB) k_pcg_batched(const __grid_constant__ PcgBatch<kMaxBatchRuns> B) {
     // the block's run, copied to shared memory: read through a dynamic index
     // in parameter space, the arguments made the solve half as fast again
     __shared__ PcgArgs sa;
+    __shared__ double shv[4 * kThreads];
+    __shared__ unsigned long long shm[kThreads];
     if (threadIdx.x == 0) {
         int ri = 0;
         while (ri + 1 < B.n_runs && (int)blockIdx.x >= B.run[ri + 1].block0) ri++;
         sa = B.run[ri];
     }
     __syncthreads();
-    pcg_body<REFINE>(sa, sa.blocks, (int)blockIdx.x - sa.block0);
+    constexpr int kRing = ANYWIDE ? kBatchRingWide : kBatchRing;
+    if (ANYWIDE && sa.wide)
+        pcg_body<REFINE, true, kThreads, kBatchRingWide>(sa, sa.blocks, (int)blockIdx.x - sa.block0, s_ring, shv, shm);
+    else
+        pcg_body<REFINE, false, kThreads, kRing>(sa, sa.blocks, (int)blockIdx.x - sa.block0, s_ring, shv, shm);
 }
 
 int grid_for_rows(int n) { return std::max(1, std::min(kMaxBlocks, (n + kRowsPerBlock - 1) / kRowsPerBlock)); }
@@ -1595,21 +1750,53 @@ __global__ void k_axpby(int n, double a, const double *__restrict__ x, double b,
     if (i < n) out[i] = a * x[i] + b * y[i];
 }
 
-// MIXED corrections solve the diagonally scaled system D^-1/2 A D^-1/2 (unit
-// diagonal: Jacobi-PCG on A is plain CG on it, without the D^-1 and u vectors)
-__global__ void k_scale_sell_f32(int n, int n_slices, const int *__restrict__ sp, const int *__restrict__ sw,
-                                 const int *__restrict__ col, const double *__restrict__ v,
-                                 const double *__restrict__ dinv, float *__restrict__ out) {
+// The solvers' matrices as records (stream.cuh): the FP64 values as they are,
+// or, with dinv, FP32 values of the diagonally scaled D^-1/2 A D^-1/2 (unit
+// diagonal: Jacobi-PCG on A is plain CG on it, without the D^-1 and u vectors),
+// which the MIXED corrections solve.  One warp a slice; the records past the
+// last column were zeroed (value 0, an existing column).
+template <typename V, bool WIDE>
+__global__ void k_pack_records(int n, int n_slices, const int *__restrict__ sp, const int *__restrict__ sw,
+                               const int *__restrict__ col, const int *__restrict__ base,
+                               const unsigned char *__restrict__ off, const double *__restrict__ v,
+                               const double *__restrict__ dinv, unsigned char *__restrict__ out) {
+    using Rec = Record<V, WIDE>;
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const int sl = t >> 5, lane = t & 31;
     if (sl >= n_slices) return;
-    const int i = sl * 32 + lane;
-    const double di = i < n ? sqrt(dinv[i]) : 0.0;
+    const int i = sl * 32 + lane, k0 = sp[sl] >> 5;
+    const double di = dinv && i < n ? sqrt(dinv[i]) : 0.0;
     for (int j = 0; j < sw[sl]; j++) {
-        const int k = sp[sl] + 32 * j + lane;
-        out[k] = i < n ? (float)(v[k] * di * sqrt(dinv[col[k]])) : 0.0f;
+        const int k = k0 + j, c = k & (kCols - 1);
+        const size_t e = 32 * (size_t)k + lane;
+        unsigned char *rec = out + (size_t)(k / kCols) * Rec::bytes;
+        double x = 0.0;
+        if (i < n) x = dinv ? v[e] * di * sqrt(dinv[col[e]]) : v[e];
+        *reinterpret_cast<V *>(rec + record_value_at<V>(c, lane)) = (V)x;
+        if constexpr (WIDE) {
+            *reinterpret_cast<int *>(rec + Rec::val + ((c >> 2) * 32 + lane) * 16 + (c & 3) * 4) = col[e];
+        } else {
+            rec[Rec::val + lane * kCols + c] = off[e];
+            if (lane == 0) *reinterpret_cast<int *>(rec + Rec::val + Rec::idx + 4 * c) = base[k];
+        }
     }
 }
+
+template <typename V>
+int pack_records(const DevSell &A, const double *v, const double *dinv, DevBuf<unsigned char> &out) {
+    const size_t cols = (size_t)(A.n_elems / 32), recs = (cols + kCols - 1) / kCols;
+    const size_t bytes = recs * (A.narrow ? Record<V, false>::bytes : Record<V, true>::bytes);
+    int rc = out.alloc(bytes);
+    if (rc) return rc;
+    if (!bytes) return PIC_OK;
+    FP_CUDA(cudaMemset(out.p, 0, bytes));
+    const unsigned blocks = (unsigned)((A.n_slices * 32 + 255) / 256);
+    if (A.narrow) { k_pack_records<V, false><<<blocks, 256>>>(A.n_rows, A.n_slices, A.ptr.p, A.width.p, A.col.p, A.base.p, A.off.p, v, dinv, out.p); note_launch(); }
+    else { k_pack_records<V, true><<<blocks, 256>>>(A.n_rows, A.n_slices, A.ptr.p, A.width.p, A.col.p, nullptr, nullptr, v, dinv, out.p); note_launch(); }
+    FP_CUDA(cudaGetLastError());
+    return PIC_OK;
+}
+
 __global__ void k_sqrt_f32(int n, const double *__restrict__ dinv, float *__restrict__ out) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) out[i] = (float)sqrt(dinv[i]);
@@ -1623,9 +1810,11 @@ int solver_alloc(Sim *s) {
     const int ne = m->n_edges, nf = m->n_faces, nn = m->n_nodes, ni = m->n_int_edges, nin = m->n_int_nodes;
     int rc;
     DevBuf<double> *edge_vecs[] = {&s->e, &s->e_prev, &s->x, &s->g, &s->g_prev, &s->g_new, &s->dg, &s->rhs};
+    // the solvers' vectors are padded to whole slices, zeros past the rows
+    auto padded = [](int n) { return (size_t)(std::max(n, 1) + 31) / 32 * 32; };
     for (auto *v : edge_vecs) {
-        if ((rc = v->alloc(ne))) return rc;
-        FP_CUDA(cudaMemset(v->p, 0, sizeof(double) * ne));
+        if ((rc = v->alloc(padded(ne)))) return rc;
+        FP_CUDA(cudaMemset(v->p, 0, sizeof(double) * padded(ne)));
     }
     DevBuf<double> *face_vecs[] = {&s->b, &s->b_prev, &s->b_new, &s->hb};
     for (auto *v : face_vecs) {
@@ -1639,13 +1828,13 @@ int solver_alloc(Sim *s) {
     }
     DevBuf<double> *int_vecs[] = {&s->Dinv, &s->cg_r, &s->cg_z, &s->cg_p0, &s->cg_p1, &s->cg_q, &s->w_edge, &s->me, &s->ev};
     for (auto *v : int_vecs) {
-        if ((rc = v->alloc(std::max(ni, 1)))) return rc;
-        FP_CUDA(cudaMemset(v->p, 0, sizeof(double) * std::max(ni, 1)));
+        if ((rc = v->alloc(padded(ni)))) return rc;
+        FP_CUDA(cudaMemset(v->p, 0, sizeof(double) * padded(ni)));
     }
     DevBuf<double> *lap_vecs[] = {&s->L_Dinv, &s->l_x, &s->l_b, &s->l_r, &s->l_z, &s->l_p0, &s->l_p1, &s->l_q};
     for (auto *v : lap_vecs) {
-        if ((rc = v->alloc(std::max(nin, 1)))) return rc;
-        FP_CUDA(cudaMemset(v->p, 0, sizeof(double) * std::max(nin, 1)));
+        if ((rc = v->alloc(padded(nin)))) return rc;
+        FP_CUDA(cudaMemset(v->p, 0, sizeof(double) * padded(nin)));
     }
     if ((rc = s->cg_part.alloc(8 * kMaxBlocks)) || (rc = s->l_part.alloc(8 * kMaxBlocks)) ||
         (rc = s->diag_part.alloc(8 * kMaxBlocks)))
@@ -1663,11 +1852,15 @@ int solver_alloc(Sim *s) {
                                                      m->n_abs_faces > 0 ? m->I_diag.p : nullptr, ci, s->Dinv.p); note_launch(); }
     }
     if (nin > 0) { k_recip_diag<<<(nin + 255) / 256, 256>>>(nin, m->L.rowptr.p, m->L.col.p, m->L_val.p, s->L_Dinv.p); note_launch(); }
+    if (nel > 0 && (rc = pack_records<double>(m->As, s->A_val.p, nullptr, s->A_rec))) return rc;
+    if (nin > 0 && (rc = pack_records<double>(m->Ls, m->Ls_val.p, nullptr, s->L_rec))) return rc;
     // MIXED: the correction solves of the Newmark refinement run on the
     // diagonally scaled system in FP32
     if (s->mixed && nel > 0) {
-        if ((rc = s->A32.alloc(nel)) || (rc = s->Dhalf32.alloc(ni)) || (rc = s->cg32.alloc(6 * (size_t)ni))) return rc;
-        { k_scale_sell_f32<<<(unsigned)((m->As.n_slices * 32 + 255) / 256), 256>>>(ni, m->As.n_slices, m->As.ptr.p, m->As.width.p, m->As.col.p, s->A_val.p, s->Dinv.p, s->A32.p); note_launch(); }
+        if ((rc = s->Dhalf32.alloc(padded(ni))) || (rc = s->cg32.alloc(6 * padded(ni)))) return rc;
+        FP_CUDA(cudaMemset(s->Dhalf32.p, 0, sizeof(float) * padded(ni)));
+        FP_CUDA(cudaMemset(s->cg32.p, 0, sizeof(float) * 6 * padded(ni)));
+        if ((rc = pack_records<float>(m->As, s->A_val.p, s->Dinv.p, s->A_rec32))) return rc;
         { k_sqrt_f32<<<(unsigned)((ni + 255) / 256), 256>>>(ni, s->Dinv.p, s->Dhalf32.p); note_launch(); }
     }
     FP_CUDA(cudaGetLastError());
@@ -1717,24 +1910,52 @@ int newmark_rhs(Sim *s) {
     return PIC_OK;
 }
 
-// co-resident blocks per SM of the persistent PCG for up to MAXR runs (0:
-// no cooperative launch on this device)
-// (queried once per device and kept: no runtime queries while a stream is
-// being captured)
+// A persistent kernel and its launch shape: co-resident blocks per SM (0: no
+// cooperative launch on this device), queried once per device and kept (no
+// runtime queries while a stream is being captured)
 constexpr int kMaxDevices = 64;
-template <bool BATCHED, bool REFINE, int MINB = 4>
-static int coop_per_sm() {
-    static int cache[kMaxDevices];   // 0: not queried, -1: unavailable
-    int dev = 0, coop = 0, per_sm = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 0;
-    if (cache[dev]) return std::max(cache[dev], 0);
-    cache[dev] = -1;
-    if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop) return 0;
-    cudaError_t e = BATCHED ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pcg_batched<REFINE, MINB>, kThreads, 0)
-                            : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pcg_persistent<REFINE>, kThreads, 0);
-    if (e != cudaSuccess) return 0;
-    cache[dev] = per_sm > 0 ? per_sm : -1;
-    return std::max(per_sm, 0);
+struct CoopKernel {
+    const void *fn;
+    int threads, ring;            // dynamic shared memory: the warps' rings
+    int cache[kMaxDevices];       // 0: not queried, -1: unavailable
+    std::mutex lock;
+    CoopKernel(const void *f, int t, int ring_per_warp) : fn(f), threads(t), ring(ring_per_warp * (t / 32)), cache{} {}
+    int per_sm() {
+        int dev = 0, coop = 0, n = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 0;
+        std::lock_guard<std::mutex> hold(lock);
+        if (cache[dev]) return std::max(cache[dev], 0);
+        cache[dev] = -1;
+        if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop) return 0;
+        if (ring > 0 && cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, ring) != cudaSuccess) return 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, threads, ring) != cudaSuccess) return 0;
+        cache[dev] = n > 0 ? n : -1;
+        return std::max(n, 0);
+    }
+    int launch(int blocks, void **args, cudaStream_t st) {
+        FP_CUDA(cudaLaunchCooperativeKernel(fn, blocks, threads, args, ring, st));
+        note_launch();
+        return PIC_OK;
+    }
+};
+
+template <bool REFINE, bool WIDE>
+static CoopKernel &coop_single() {
+    using P = PcgShape<REFINE, WIDE>;
+    static CoopKernel k((const void *)k_pcg_persistent<REFINE, WIDE>, P::threads, P::ring);
+    return k;
+}
+template <bool REFINE, int MINB, bool ANYWIDE>
+static CoopKernel &coop_batched() {
+    static CoopKernel k((const void *)k_pcg_batched<REFINE, MINB, ANYWIDE>, kThreads, ANYWIDE ? kBatchRingWide : kBatchRing);
+    return k;
+}
+static CoopKernel &pcg_kernel(bool one, bool refine, bool wide, int build) {
+    if (one) return refine ? (wide ? coop_single<true, true>() : coop_single<true, false>())
+                           : (wide ? coop_single<false, true>() : coop_single<false, false>());
+    if (wide) return refine ? coop_batched<true, 3, true>() : coop_batched<false, 3, true>();
+    if (build == 1) return refine ? coop_batched<true, 3, false>() : coop_batched<false, 3, false>();
+    return refine ? coop_batched<true, 4, false>() : coop_batched<false, 4, false>();
 }
 
 static int sm_count() {
@@ -1749,7 +1970,6 @@ static int sm_count() {
 
 __global__ void k_reset_gbar(GridBarrier *gb) {
     gb->count = 0;
-    gb->flag = 0;
     gb->timeout = 0;
 }
 
@@ -1758,7 +1978,6 @@ __global__ void k_reset_barriers(PcgBatch<kMaxBatchRuns> B) {
     if (r < B.n_runs) {
         GridBarrier *gb = B.run[r].gb;
         gb->count = 0;
-        gb->flag = 0;
         gb->timeout = 0;
     }
 }
@@ -1774,7 +1993,7 @@ static int assign_blocks(PcgArgs *runs, int n_runs, int budget) {
     long want_total = 0, slices = 0;
     std::vector<int> want(n_runs);
     for (int r = 0; r < n_runs; r++) {
-        want[r] = std::max(1, std::min(kMaxPcgBlocks, (runs[r].n_slices + kSlicesPerBlock - 1) / kSlicesPerBlock));
+        want[r] = std::max(1, std::min(kMaxPcgBlocks, (runs[r].n_slices + kSlicesPerPcgBlock - 1) / kSlicesPerPcgBlock));
         want_total += want[r];
         slices += std::max(runs[r].n_slices, 1);
     }
@@ -1816,11 +2035,10 @@ int launch_pcg_runs(PcgArgs *runs, int n_runs, int blocks_per_sm, cudaStream_t s
             set_error("the solves of one persistent launch must all be FP64 or all be refinements");
             return PIC_ERR_INVALID_ARG;
         }
-    int per_sm = one ? (refine ? coop_per_sm<false, true>() : coop_per_sm<false, false>())
-                 : build == 1 ? (refine ? coop_per_sm<true, true, 3>() : coop_per_sm<true, false, 3>())
-                 : build == 2 ? (refine ? coop_per_sm<true, true, 6>() : coop_per_sm<true, false, 6>())
-                 : build == 3 ? (refine ? coop_per_sm<true, true, 8>() : coop_per_sm<true, false, 8>())
-                              : (refine ? coop_per_sm<true, true>() : coop_per_sm<true, false>());
+    bool wide = false;
+    for (int r = 0; r < n_runs; r++) wide = wide || runs[r].wide;
+    CoopKernel &kernel = pcg_kernel(one, refine, wide, build);
+    int per_sm = kernel.per_sm();
     if (per_sm <= 0) {
         set_error("the persistent PCG needs a device with cooperative launch");
         return PIC_ERR_CUDA;
@@ -1833,24 +2051,12 @@ int launch_pcg_runs(PcgArgs *runs, int n_runs, int blocks_per_sm, cudaStream_t s
     all.n_runs = n_runs;
     for (int r = 0; r < n_runs; r++) all.run[r] = runs[r];
     { k_reset_barriers<<<1, kMaxBatchRuns, 0, st>>>(all); note_launch(); }
-    if (one) {
-        PcgArgs a1 = all.run[0];
-        void *args[] = {&a1};
-        const void *k = refine ? (const void *)k_pcg_persistent<true> : (const void *)k_pcg_persistent<false>;
-        FP_CUDA(cudaLaunchCooperativeKernel(k, G, kThreads, args, 0, st));
-    } else {
-        void *args[] = {&all};
-        const void *k = build == 1 ? (refine ? (const void *)k_pcg_batched<true, 3> : (const void *)k_pcg_batched<false, 3>)
-                      : build == 2 ? (refine ? (const void *)k_pcg_batched<true, 6> : (const void *)k_pcg_batched<false, 6>)
-                      : build == 3 ? (refine ? (const void *)k_pcg_batched<true, 8> : (const void *)k_pcg_batched<false, 8>)
-                                   : (refine ? (const void *)k_pcg_batched<true, 4> : (const void *)k_pcg_batched<false, 4>);
-        FP_CUDA(cudaLaunchCooperativeKernel(k, G, kThreads, args, 0, st));
-    }
-    note_launch();
-    return PIC_OK;
+    PcgArgs a1 = all.run[0];
+    void *args[] = {one ? (void *)&a1 : (void *)&all};
+    return kernel.launch(G, args, st);
 }
 
-static PcgArgs make_args(Sim *s, const DevSell &A, const double *Av, const double *Dinv, const double *b, double *x,
+static PcgArgs make_args(Sim *s, const DevSell &A, const DevBuf<unsigned char> &rec, const double *Dinv, const double *b, double *x,
                          double *r, double *u, double *w, double *p, double *sv, double *part, CgState *st,
                          double tol, double fallback_tol, int max_iters, const double *abs_src, double abs_factor,
                          bool x_zero, bool quiet) {
@@ -1860,8 +2066,9 @@ static PcgArgs make_args(Sim *s, const DevSell &A, const double *Av, const doubl
     a.n_slices = A.n_slices;
     a.sp = A.ptr.p;
     a.sw = A.width.p;
-    a.col = A.col.p;
-    a.Av = Av;
+    a.rec = rec.p;
+    a.wide = !A.narrow;
+    a.evict_first = rec.n > kKeepInL2;
     a.Dinv = Dinv;
     a.b = b;
     a.x = x;
@@ -1890,7 +2097,7 @@ static PcgArgs make_args(Sim *s, const DevSell &A, const double *Av, const doubl
 // iterations without an error (training samples, solver timing)
 PcgArgs pcg_args_truncated(Sim *s, int iters) {
     const Mesh *m = s->mesh;
-    return make_args(s, m->As, s->A_val.p, s->Dinv.p, s->rhs.p, s->x.p, s->cg_r.p, s->cg_z.p, s->cg_q.p, s->cg_p0.p,
+    return make_args(s, m->As, s->A_rec, s->Dinv.p, s->rhs.p, s->x.p, s->cg_r.p, s->cg_z.p, s->cg_q.p, s->cg_p0.p,
                      s->cg_p1.p, s->cg_part.p, &s->dctl.p->cg, 0.0, 0.0, iters, nullptr, 0.0, true, true);
 }
 
@@ -1910,15 +2117,16 @@ PcgArgs pcg_args_newmark_truncated(Sim *s, int iters) {
 // the stopping rule in both precisions.
 PcgArgs pcg_args_newmark(Sim *s) {
     const Mesh *m = s->mesh;
-    PcgArgs a = make_args(s, m->As, s->A_val.p, s->Dinv.p, s->rhs.p, s->x.p, s->cg_r.p, s->cg_z.p, s->cg_q.p,
+    PcgArgs a = make_args(s, m->As, s->A_rec, s->Dinv.p, s->rhs.p, s->x.p, s->cg_r.p, s->cg_z.p, s->cg_q.p,
                           s->cg_p0.p, s->cg_p1.p, s->cg_part.p, &s->dctl.p->cg, s->cfg.cg_tol, 0.0,
                           s->cfg.cg_max_iters, nullptr, 0.0, false, false);
-    if (s->mixed && s->A32.p) {
-        const size_t ni = (size_t)m->n_int_edges;
+    if (s->mixed && s->A_rec32.p) {
+        const size_t ni = s->cg32.n / 6;
         float *v = s->cg32.p;
         a.refine = 1;
         a.inner_tol2 = 1e-10;
-        a.Av32 = s->A32.p;
+        a.rec32 = s->A_rec32.p;
+        a.evict_first = s->A_rec32.n > kKeepInL2;
         a.Dhalf32 = s->Dhalf32.p;
         a.b32 = v;
         a.d32 = v + ni;
@@ -1936,7 +2144,7 @@ PcgArgs pcg_args_completion(Sim *s) {
     const Mesh *m = s->mesh;
     // (in both precisions FP64: the completion is bound by the latency of its
     // iterations, not by their arithmetic, and FP32 corrections took more)
-    return make_args(s, m->Ls, m->Ls_val.p, s->L_Dinv.p, s->l_b.p, s->l_x.p, s->l_r.p, s->l_z.p, s->l_q.p,
+    return make_args(s, m->Ls, s->L_rec, s->L_Dinv.p, s->l_b.p, s->l_x.p, s->l_r.p, s->l_z.p, s->l_q.p,
                      s->l_p0.p, s->l_p1.p, s->l_part.p, &s->dctl.p->lap, 0.0, s->cfg.init_tol, 20000,
                      &s->dctl.p->qmax, s->cfg.completion_tol, true, false);
 }
@@ -1979,7 +2187,7 @@ int laplacian_solve(Sim *s, const double *rhs_int, double *x_int, double tol, co
                     double abs_factor) {
     const Mesh *m = s->mesh;
     if (m->n_int_nodes == 0) return PIC_OK;
-    PcgArgs a = make_args(s, m->Ls, m->Ls_val.p, s->L_Dinv.p, rhs_int, x_int, s->l_r.p, s->l_z.p, s->l_q.p,
+    PcgArgs a = make_args(s, m->Ls, s->L_rec, s->L_Dinv.p, rhs_int, x_int, s->l_r.p, s->l_z.p, s->l_q.p,
                           s->l_p0.p, s->l_p1.p, s->l_part.p, &s->dctl.p->lap, tol, s->cfg.init_tol, 20000, abs_src,
                           abs_factor, true, false);
     return launch_pcg_runs(&a, 1, s->cfg.solver_blocks_per_sm, s->stream);
@@ -2060,32 +2268,17 @@ int mg_completion(Sim *s) {
     if (rc) return rc;
     // z_old starts at zero (the first beta is 0 and ignores it, but it is read)
     FP_CUDA(cudaMemsetAsync(s->l_p1.p, 0, sizeof(double) * n0, s->stream));
-    static int per_sm_cache[kMaxDevices];
-    int dev = 0;
-    FP_CUDA(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= kMaxDevices) {
-        set_error("mg_completion: device index out of range");
-        return PIC_ERR_CUDA;
-    }
-    if (!per_sm_cache[dev]) {
-        int per_sm = 0, coop = 0;
-        FP_CUDA(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
-        FP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_mg_pcg, kThreads, 0));
-        per_sm_cache[dev] = (coop && per_sm > 0) ? per_sm : -1;
-    }
-    if (per_sm_cache[dev] < 0) {
+    static CoopKernel kernel((const void *)k_mg_pcg, kMgThreads, 0);
+    const int per_sm = kernel.per_sm();
+    if (per_sm <= 0) {
         set_error("the multigrid completion needs a device with cooperative launch");
         return PIC_ERR_CUDA;
     }
-    // four blocks per SM (2, 3, 4 measured 2.87, 2.41, 2.17 ms per completion
-    // on the 64^3 plasma-ball mesh: the phases are latency-bound)
-    const int want = s->cfg.solver_blocks_per_sm ? s->cfg.solver_blocks_per_sm : 4;
-    const int blocks = std::max(1, std::min(per_sm_cache[dev], want)) * sm_count();
+    const int want = s->cfg.solver_blocks_per_sm ? s->cfg.solver_blocks_per_sm : 1;
+    const int blocks = std::max(1, std::min(per_sm, want)) * sm_count();
     { k_reset_gbar<<<1, 1, 0, s->stream>>>(a.gb); note_launch(); }
     void *args[] = {&a};
-    FP_CUDA(cudaLaunchCooperativeKernel((const void *)k_mg_pcg, blocks, kThreads, args, 0, s->stream));
-    note_launch();
-    return PIC_OK;
+    return kernel.launch(blocks, args, s->stream);
 }
 
 // ---------------------------------------------------------------------------
@@ -2104,11 +2297,14 @@ struct CompletionRun {
     MgArgs mg;
 };
 struct CompletionTable {
-    int n_runs, total_blocks;
+    int n_runs, total_blocks, any_wide, pad;
     CompletionRun run[kMaxBatchRuns];
 };
 
-__global__ void __launch_bounds__(kThreads, 4) k_completion_batched(const CompletionTable *__restrict__ T) {
+template <bool ANYWIDE>
+__global__ void __launch_bounds__(kThreads, ANYWIDE ? 3 : 4) k_completion_batched(const CompletionTable *__restrict__ T) {
+    __shared__ double shv[4 * kThreads];
+    __shared__ unsigned long long shm[kThreads];
     // the block's run record in shared memory (read through a dynamic index
     // from global memory, every use would be a load)
     __shared__ __align__(16) CompletionRun sr;
@@ -2125,8 +2321,16 @@ __global__ void __launch_bounds__(kThreads, 4) k_completion_batched(const Comple
         for (int k = threadIdx.x; k < (int)(sizeof(CompletionRun) / sizeof(int)); k += blockDim.x) dst[k] = src[k];
     }
     __syncthreads();
-    if (sr.kind) mg_body(sr.mg, sr.blocks, (int)blockIdx.x - sr.block0);
-    else pcg_body<false>(sr.pcg, sr.blocks, (int)blockIdx.x - sr.block0);
+    constexpr int kRing = ANYWIDE ? kBatchRingWide : kBatchRing;
+    const int bid = (int)blockIdx.x - sr.block0;
+    if (sr.kind) mg_body<kThreads>(sr.mg, sr.blocks, bid, shv, shm);
+    else if (ANYWIDE && sr.pcg.wide) pcg_body<false, true, kThreads, kBatchRingWide>(sr.pcg, sr.blocks, bid, s_ring, shv, shm);
+    else pcg_body<false, false, kThreads, kRing>(sr.pcg, sr.blocks, bid, s_ring, shv, shm);
+}
+static CoopKernel &completion_kernel(bool any_wide) {
+    static CoopKernel narrow((const void *)k_completion_batched<false>, kThreads, kBatchRing);
+    static CoopKernel wide((const void *)k_completion_batched<true>, kThreads, kBatchRingWide);
+    return any_wide ? wide : narrow;
 }
 
 __global__ void k_reset_completion_barriers(const CompletionTable *__restrict__ T) {
@@ -2134,7 +2338,6 @@ __global__ void k_reset_completion_barriers(const CompletionTable *__restrict__ 
     if (r < T->n_runs) {
         GridBarrier *gb = T->run[r].kind ? T->run[r].mg.gb : T->run[r].pcg.gb;
         gb->count = 0;
-        gb->flag = 0;
         gb->timeout = 0;
     }
 }
@@ -2153,25 +2356,6 @@ bool completion_uses_multigrid(Sim *const *sims, int n) {
 // warp per slice, up to blocks_per_sm (0: as many as fit) on every SM.
 int prepare_completion_table(Sim *const *sims, int n, int blocks_per_sm, void *table_dev, int *n_runs,
                              int *total_blocks) {
-    static int per_sm_cache[kMaxDevices];
-    int dev = 0;
-    FP_CUDA(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= kMaxDevices) {
-        set_error("batched completion: device index out of range");
-        return PIC_ERR_CUDA;
-    }
-    if (!per_sm_cache[dev]) {
-        int per_sm = 0, coop = 0;
-        FP_CUDA(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
-        FP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_completion_batched, kThreads, 0));
-        per_sm_cache[dev] = (coop && per_sm > 0) ? per_sm : -1;
-    }
-    if (per_sm_cache[dev] < 0) {
-        set_error("the batched completion needs a device with cooperative launch");
-        return PIC_ERR_CUDA;
-    }
-    const int per_sm = blocks_per_sm > 0 ? std::min(per_sm_cache[dev], blocks_per_sm) : per_sm_cache[dev];
-    const int budget = per_sm * sm_count();
     std::vector<CompletionTable> host(1);
     CompletionTable &T = host[0];
     std::memset(&T, 0, sizeof(T));
@@ -2189,8 +2373,16 @@ int prepare_completion_table(Sim *const *sims, int n, int blocks_per_sm, void *t
             r.kind = 0;
             r.pcg = pcg_args_completion(s);
         }
+        if (!r.kind && r.pcg.wide) T.any_wide = 1;
         slices.push_back(std::max(1, (m->n_int_nodes + 31) / 32));
     }
+    const int fit = completion_kernel(T.any_wide != 0).per_sm();
+    if (fit <= 0) {
+        set_error("the batched completion needs a device with cooperative launch");
+        return PIC_ERR_CUDA;
+    }
+    const int per_sm = blocks_per_sm > 0 ? std::min(fit, blocks_per_sm) : fit;
+    const int budget = per_sm * sm_count();
     if (T.n_runs > budget) {
         set_error("more batched solves than co-resident blocks");
         return PIC_ERR_INVALID_ARG;
@@ -2224,20 +2416,19 @@ int prepare_completion_table(Sim *const *sims, int n, int blocks_per_sm, void *t
     T.total_blocks = b0;
     FP_CUDA(cudaMemcpy(table_dev, &T, sizeof(T), cudaMemcpyHostToDevice));
     *n_runs = T.n_runs;
-    *total_blocks = T.total_blocks;
+    *total_blocks = T.any_wide ? -T.total_blocks : T.total_blocks;
     return PIC_OK;
 }
 
 // One launch of the table's solves on st (the members' l_p1 zeroed first by
-// the caller for the multigrid runs).  total_blocks: the table's block count.
+// the caller for the multigrid runs).  total_blocks: the table's block count,
+// negative when a run's records are wide.
 int launch_completion_table(const void *table_dev, int n_runs, int total_blocks, cudaStream_t st) {
     if (n_runs <= 0) return PIC_OK;
     const CompletionTable *T = static_cast<const CompletionTable *>(table_dev);
     { k_reset_completion_barriers<<<1, kMaxBatchRuns, 0, st>>>(T); note_launch(); }
     void *args[] = {&T};
-    FP_CUDA(cudaLaunchCooperativeKernel((const void *)k_completion_batched, total_blocks, kThreads, args, 0, st));
-    note_launch();
-    return PIC_OK;
+    return completion_kernel(total_blocks < 0).launch(std::abs(total_blocks), args, st);
 }
 
 // Completion of the field solve on the gradient subspace: the part of the
