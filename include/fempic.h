@@ -430,12 +430,12 @@ int64_t pic_launch_count(void);
  * when they need the solve: runtimes that hand out all device memory from
  * their own pool and forbid libraries to allocate, or services whose memory
  * budget is fixed at start-up.  Solves (G^T M G) phi = rho on the interior nodes
- * (phi = 0 on wall nodes) with the Jacobi-PCG of pic_sim_init, to the relative
- * residual tol, on `stream`.
+ * (phi = 0 on wall nodes) to the relative residual tol, on `stream`, with the
+ * library's persistent solvers of the node Laplacian.
  *   rho_nodes [n_nodes], phi_nodes [n_nodes]: device arrays of the current
  *   device, read / written during the call (phi is fully overwritten).
  * It allocates nothing: its working vectors live in one fixed device array of
- * the library (33.7 MB on every GPU that loads the solver, held until exit),
+ * the library (37.9 MB on every GPU that loads the solver, held until exit),
  * which limits the mesh to 524,288 interior nodes (PIC_ERR_INVALID_ARG above
  * that).  The mesh must already have its device copy, made by a
  * pic_sim_create on it (PIC_ERR_STATE otherwise), and the current device
@@ -443,7 +443,7 @@ int64_t pic_launch_count(void);
  * first call on each device looks up the array's device address.  All calls
  * share the array and it keeps the last call's contents (the call sets
  * everything it reads); calls that overlap on the GPU, from two streams or
- * two threads, race on it.  Synchronises `stream` for its convergence checks
+ * two threads, race on it.  Synchronises `stream` for its result
  * (PIC_ERR_STATE when `stream` is being captured). */
 int pic_electrostatic_solve_noalloc(const pic_mesh *mesh, const double *rho_nodes, double *phi_nodes, double tol,
                                     void *stream);

@@ -182,12 +182,10 @@ struct Mesh {
     // face mass [*mu^-1] on all faces (SELL-32, natural face order)
     DevSell Hs;
     DevBuf<double> Hs_val;
-    // node Laplacian G^T M G on interior nodes (compact numbering, ordered by
-    // row length): CSR and SELL-32 copies
-    DevCsr L;
-    DevBuf<double> L_val;
+    // node Laplacian G^T M G on interior nodes (compact numbering)
     DevSell Ls;
     DevBuf<double> Ls_val, L_diag;
+    DevBuf<unsigned char> L_rec;     // as records of the streamed solves (stream.cuh)
     // smoothed-aggregation hierarchy preconditioning the completion (3 levels;
     // mg_levels = 0 when the mesh is small or the set-up declined)
     int mg_levels = 0, mg_n1 = 0, mg_n2 = 0;

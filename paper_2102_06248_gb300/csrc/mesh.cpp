@@ -752,7 +752,6 @@ int mesh_upload(Mesh *m) {
     if ((rc = m->Hs.ptr.upload(H.hsell_ptr)) || (rc = m->Hs.width.upload(H.hsell_w)) ||
         (rc = m->Hs.col.upload(H.hsell_col)) || (rc = m->Hs_val.upload(H.hsell_H)))
         return rc;
-    if ((rc = csr(H.L, &m->L)) || (rc = m->L_val.upload(H.L_val))) return rc;
     m->Ls.n_rows = m->n_int_nodes;
     m->Ls.n_slices = (int)H.lsell_w.size();
     m->Ls.n_elems = H.lsell_ptr.empty() ? 0 : H.lsell_ptr.back();

@@ -210,7 +210,7 @@ struct Sim {
     // solver work
     DevBuf<double> A_val, Dinv;
     DevBuf<float> Dhalf32, cg32;       // MIXED: D^-1/2 and six correction vectors
-    DevBuf<unsigned char> A_rec, A_rec32, L_rec;   // the solvers' matrices as records (stream.cuh)
+    DevBuf<unsigned char> A_rec, A_rec32;   // the system matrix as records (stream.cuh)
     DevBuf<double> cg_r, cg_z, cg_p0, cg_p1, cg_q, cg_part;
     DevBuf<double> hb;              // face vector H (b + b_prev)
     DevBuf<double> w_edge;          // gradient completion: M t - d2 Gbar on interior edges
