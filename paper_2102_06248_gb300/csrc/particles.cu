@@ -455,17 +455,14 @@ __device__ __forceinline__ void push_record(const PushArgs<R, V> &a, uint32_t ai
     for (int c = 0; c < kNV; c++) o[c] = v[c];
 }
 
-__device__ __forceinline__ double shfl_up_v(double v, int off) { return __shfl_up_sync(0xFFFFFFFFu, v, off); }
-__device__ __forceinline__ long long shfl_up_v(long long v, int off) { return __shfl_up_sync(0xFFFFFFFFu, v, off); }
-
 // Deterministic reduction of the first-piece deposits of a block of sorted
 // particles into the per-tet accumulators: a warp-segmented inclusive scan by
 // key, runs inside a warp stored directly (sole writer), the warps' boundary
 // pieces merged in warp order, and the block's own boundary runs handed to
 // k_fixup through the carry slots.
-template <typename R, typename V, typename KE>
-__device__ __forceinline__ void reduce_block(const PushArgs<R, V> &a, uint32_t rkey, V vals[kNV], KE ke,
-                                             int alive_out, int n_alive) {
+__device__ __forceinline__ void reduce_block(const PushArgs<double, double> &a, uint32_t rkey, double vals[kNV],
+                                             double ke, int alive_out, int n_alive) {
+    using V = double;
     __shared__ uint32_t s_key[kPushBlock / 32][2];
     __shared__ V s_val[kPushBlock / 32][2][kNV];
     __shared__ double s_ke[kPushBlock / 32];
@@ -473,44 +470,18 @@ __device__ __forceinline__ void reduce_block(const PushArgs<R, V> &a, uint32_t r
     {
         const unsigned ball = __ballot_sync(0xFFFFFFFFu, alive_out);
         if (lane == 0 && ball) atomicAdd(a.n_alive_next, __popc(ball));
-        KE k2 = ke;   // kinetic energy: FP32 per warp in MIXED, FP64 across warps
+        double k2 = ke;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) k2 += __shfl_down_sync(0xFFFFFFFFu, k2, o);
-        if (lane == 0) s_ke[warp] = (double)k2;
+        if (lane == 0) s_ke[warp] = k2;
     }
-    if constexpr (std::is_same<V, long long>::value) {
-        // MIXED: the four node charges are integers in [0, 2^24]; a warp's run
-        // sums at most 32 of them (< 2^29), so two share one 64-bit lane of
-        // the scan without carries: 8 scanned channels instead of 10
-        long long w[8];
 #pragma unroll
-        for (int c = 0; c < 6; c++) w[c] = vals[c];
-        w[6] = vals[6] | (vals[7] << 32);
-        w[7] = vals[8] | (vals[9] << 32);
+    for (int off = 1; off < 32; off <<= 1) {
+        const uint32_t ko = __shfl_up_sync(0xFFFFFFFFu, rkey, off);
 #pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const uint32_t ko = __shfl_up_sync(0xFFFFFFFFu, rkey, off);
-#pragma unroll
-            for (int c = 0; c < 8; c++) {
-                const long long vo = shfl_up_v(w[c], off);
-                if (lane >= off && ko == rkey) w[c] += vo;
-            }
-        }
-#pragma unroll
-        for (int c = 0; c < 6; c++) vals[c] = w[c];
-        vals[6] = w[6] & 0xFFFFFFFFll;
-        vals[7] = (long long)((unsigned long long)w[6] >> 32);
-        vals[8] = w[7] & 0xFFFFFFFFll;
-        vals[9] = (long long)((unsigned long long)w[7] >> 32);
-    } else {
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const uint32_t ko = __shfl_up_sync(0xFFFFFFFFu, rkey, off);
-#pragma unroll
-            for (int c = 0; c < kNV; c++) {
-                const V vo = shfl_up_v(vals[c], off);
-                if (lane >= off && ko == rkey) vals[c] += vo;
-            }
+        for (int c = 0; c < kNV; c++) {
+            const V vo = __shfl_up_sync(0xFFFFFFFFu, vals[c], off);
+            if (lane >= off && ko == rkey) vals[c] += vo;
         }
     }
     const uint32_t knext = __shfl_down_sync(0xFFFFFFFFu, rkey, 1);
@@ -598,9 +569,15 @@ template <typename R, int MODE>
 __device__ __forceinline__ void gather_push(const PushArgs<R, typename std::conditional<std::is_same<R, double>::value, double, long long>::type> &a,
                                             const R *cf, const R P[3], const R V[3], R d0, R d1, R d2, int spc,
                                             long src, long i, R Q[3], R Vn[3]) {
+    // (records of 10: 40 or 80 bytes, so pairs are aligned)
+    using R2 = typename std::conditional<std::is_same<R, double>::value, double2, float2>::type;
     R c[10];
 #pragma unroll
-    for (int k = 0; k < 10; k++) c[k] = cf[k];
+    for (int k = 0; k < 5; k++) {
+        const R2 t = reinterpret_cast<const R2 *>(cf)[k];
+        c[2 * k] = t.x;
+        c[2 * k + 1] = t.y;
+    }
     // Whitney fields in the tet (Sec. II.A): E = E0 + Omega x d, B = B0 + beta d
     const R E[3] = {c[0] + c[4] * d2 - c[5] * d1, c[1] + c[5] * d0 - c[3] * d2, c[2] + c[3] * d1 - c[4] * d0};
     const R B[3] = {c[6] + c[9] * d0, c[7] + c[9] * d1, c[8] + c[9] * d2};
@@ -995,153 +972,329 @@ __global__ void __launch_bounds__(kPushBlock) k_push_plain(const PushArgs<double
         rkey = (uint32_t)tet;
         }
     }
-    reduce_block<double, double, double>(a, rkey, vals, ke, alive_out, n_alive);
+    reduce_block(a, rkey, vals, ke, alive_out, n_alive);
 }
 
 // ---------------------------------------------------------------------------
 // MIXED: FP32 state, gather, push and walk; fixed-point barycentrics and an
-// integer deposit (exact), accumulators per (tet, species)
+// integer deposit (exact), accumulators per (tet, species).
+//
+// The kernel is bound by instruction issue, and a third of its instructions
+// used to sum the deposits of equal keys: a segmented scan of eight 64-bit
+// channels over the warp for every 32 particles, then a merge of the block's
+// warps behind a block barrier and a second kernel for runs that span blocks.
+// Sums of integers do not depend on their order, so a warp now takes `rounds`
+// times 32 consecutive sorted particles and
+//  * while all its lanes hold the key of the round before -- the common case
+//    where a tet has more than a few dozen particles -- adds each lane's deposit
+//    to the lane's own accumulators (a multiply-add per product, no shuffle);
+//  * when the key changes between rounds, sums the lanes' accumulators once,
+//    with the 32-bit warp reduction on limbs;
+//  * scans only the rounds with several keys.
+// A run that lies inside the warp's particles is stored; the first and last
+// runs, which neighbouring warps may share, are added with 64-bit atomics to
+// the cleared accumulators.  No block barrier, no second kernel.
+// Measured (33.5M particles, 64^3 plasma ball): 1.72 -> 1.22 ms; 4M in 23x25x21
+// cells 0.25 -> 0.19 ms.  4, 8, 16 rounds: 1.37, 1.22, 1.24 ms; three blocks per SM
+// (80 registers, no spills) 1.27 ms; reading the next round's key and place,
+// or its whole state, a round ahead 1.31 and 1.40 ms.
 // ---------------------------------------------------------------------------
+constexpr int kMaxRounds = 8;          // rounds of a warp (a lane's charges stay < 2^30, its currents < 2^54)
+
+// sum over the warp of v, |v| < 2^58: three limbs of 22 bits and a signed top
+__device__ __forceinline__ long long warp_sum_i64(long long v) {
+    constexpr unsigned kMask = (1u << 22) - 1;
+    const unsigned l0 = __reduce_add_sync(0xFFFFFFFFu, (unsigned)v & kMask);
+    const unsigned l1 = __reduce_add_sync(0xFFFFFFFFu, (unsigned)(v >> 22) & kMask);
+    const int l2 = __reduce_add_sync(0xFFFFFFFFu, (int)(v >> 44));
+    return (long long)l0 + ((long long)l1 << 22) + ((long long)l2 << 44);
+}
+// sum over the warp of q (any 32-bit value: two halves)
+__device__ __forceinline__ long long warp_sum_charge(unsigned q) {
+    const unsigned lo = __reduce_add_sync(0xFFFFFFFFu, q & 0xFFFFu), hi = __reduce_add_sync(0xFFFFFFFFu, q >> 16);
+    return (long long)lo + ((long long)hi << 16);
+}
+
+// the sum of a run by one lane: stored, or added where another warp shares the run
+__device__ __forceinline__ void put_run(long long *tacc, uint32_t key, bool shared, const long long v[kNV]) {
+    long long *dst = tacc + (size_t)key * kNV;
+    if (shared) {
+#pragma unroll
+        for (int c = 0; c < kNV; c++)
+            if (v[c]) atomicAdd(reinterpret_cast<unsigned long long *>(dst + c), (unsigned long long)v[c]);
+    } else {
+#pragma unroll
+        for (int c = 0; c < kNV / 2; c++) reinterpret_cast<longlong2 *>(dst)[c] = make_longlong2(v[2 * c], v[2 * c + 1]);
+    }
+}
+
 template <int MODE>
-__global__ void __launch_bounds__(kPushBlock, 4) k_push_mixed(const PushArgs<float, long long> a) {
-    const long i = (long)blockIdx.x * kPushBlock + threadIdx.x;
-    const int n_alive = *a.d_n_alive;
-    const bool active = i < n_alive;
-    uint32_t rkey = kInvalid;
-    long long vals[kNV];
+__global__ void __launch_bounds__(kPushBlock, 4) k_push_mixed(const PushArgs<float, long long> a, int rounds) {
+    const int lane = threadIdx.x & 31, n_alive = *a.d_n_alive;
+    const long gw = (long)blockIdx.x * (kPushBlock / 32) + (threadIdx.x >> 5);
+    const long base = gw * 32 * rounds;
+    if (base >= n_alive) {
+        if (lane == 0) a.ke_part[gw] = 0.0;
+        return;
+    }
+    const long end = min(base + 32L * rounds, (long)n_alive);
+    const uint32_t prevk = base > 0 ? acc_index<long long>(a.skey[base - 1], a.nsp) : kInvalid;
+    const uint32_t nextk = end < n_alive ? acc_index<long long>(a.skey[end], a.nsp) : kInvalid;
+    // the run being summed: its key, the lanes' parts, and whether they are
+    // spread over the lanes (else lane 31 holds it all)
+    uint32_t ckey = kInvalid;
+    bool spread = false;
+    long long acc[6] = {0, 0, 0, 0, 0, 0};
+    unsigned accq[4] = {0, 0, 0, 0};
+    float ke_hi = 0.0f, ke_lo = 0.0f;
+    int alive = 0;
+    // the whole run's sums, in every lane
+    auto total = [&](long long t[kNV]) {
+        if (spread) {
 #pragma unroll
-    for (int c = 0; c < kNV; c++) vals[c] = 0;
-    float ke = 0.0f;
-    int alive_out = 0;
-    if (active) {
-        const uint32_t key = a.skey[i];
-        const int tet = (int)(key >> 2), spc = (int)(key & 3u);
-        const long src = a.perm[i];
-        const float P[3] = {a.sx0[src], a.sx1[src], a.sx2[src]};
-        const float V[3] = {a.sv0[src], a.sv1[src], a.sv2[src]};
-        float gp[12];
-        load_geo32(a.geo32, tet, gp);
-        float Q[3], Vn[3];
-        gather_push<float, MODE>(a, a.coef + 10 * (size_t)tet, P, V, P[0] - gp[0], P[1] - gp[1], P[2] - gp[2], spc,
-                                 src, i, Q, Vn);
-        float lf[4];
-        int LS[4], LE[4];
-        bary32(gp, P[0], P[1], P[2], lf);
-        quantize(lf, -1, LS);
-        int T = tet;
-        int4 tn = a.tnodes[T];
-        int entry = -1;
-        bool done = false, absorbed = false;
-        int endT = tet;
-        for (int seg = 0; seg < a.walk_cap; seg++) {
-            if (seg > 0) load_geo32(a.geo32, T, gp);
-            float le[4];
-            bary32(gp, Q[0], Q[1], Q[2], le);
-            int kmin = -1;
-            float smin = 2.0f;
-            float ls[4];
+            for (int c = 0; c < 6; c++) t[c] = warp_sum_i64(acc[c]);
 #pragma unroll
-            for (int k = 0; k < 4; k++) ls[k] = (float)LS[k] * (1.0f / 16777216.0f);
+            for (int k = 0; k < 4; k++) t[6 + k] = warp_sum_charge(accq[k]);
+        } else {
 #pragma unroll
-            for (int k = 0; k < 4; k++) {
-                if (k == entry || !(le[k] < 0.0f)) continue;
-                float s = ls[k] / (ls[k] - le[k]);
-                s = s < 0.0f ? 0.0f : s;
-                if (s < smin) {
-                    smin = s;
-                    kmin = k;
+            for (int c = 0; c < 6; c++) t[c] = __shfl_sync(0xFFFFFFFFu, acc[c], 31);
+#pragma unroll
+            for (int k = 0; k < 4; k++) t[6 + k] = __shfl_sync(0xFFFFFFFFu, accq[k], 31);
+        }
+    };
+    auto flush = [&]() {
+        if (ckey == kInvalid) return;
+        long long t[kNV];
+        total(t);
+        if (lane == 0) put_run(a.tacc, ckey, ckey == prevk || ckey == nextk, t);
+    };
+    for (long r0 = base; r0 < end; r0 += 32) {
+        const long i = r0 + lane;
+        const bool active = i < end;
+        uint32_t rkey = kInvalid;
+        int S0[4] = {0, 0, 0, 0}, E0[4] = {0, 0, 0, 0};   // first piece of the path, and (ends) whether it is the whole
+        bool ends = false;
+        if (active) {
+            const uint32_t key = a.skey[i];
+            const int tet = (int)(key >> 2), spc = (int)(key & 3u);
+            const long src = a.perm[i];
+            const float P[3] = {a.sx0[src], a.sx1[src], a.sx2[src]};
+            const float V[3] = {a.sv0[src], a.sv1[src], a.sv2[src]};
+            rkey = (uint32_t)(tet * a.nsp + spc);
+            float gp[12];
+            load_geo32(a.geo32, tet, gp);
+            float Q[3], Vn[3];
+            gather_push<float, MODE>(a, a.coef + 10 * (size_t)tet, P, V, P[0] - gp[0], P[1] - gp[1], P[2] - gp[2], spc,
+                                     src, i, Q, Vn);
+            float lf[4];
+            int LS[4], LE[4];
+            bary32(gp, P[0], P[1], P[2], lf);
+            quantize(lf, -1, LS);
+#pragma unroll
+            for (int k = 0; k < 4; k++) S0[k] = LS[k];
+            int T = tet;
+            int4 tn = a.tnodes[T];
+            int entry = -1;
+            bool done = false, absorbed = false;
+            int endT = tet;
+            for (int seg = 0; seg < a.walk_cap; seg++) {
+                if (seg > 0) load_geo32(a.geo32, T, gp);
+                float le[4];
+                bary32(gp, Q[0], Q[1], Q[2], le);
+                int kmin = -1;
+                float smin = 2.0f;
+                float ls[4];
+#pragma unroll
+                for (int k = 0; k < 4; k++) ls[k] = (float)LS[k] * (1.0f / 16777216.0f);
+#pragma unroll
+                for (int k = 0; k < 4; k++) {
+                    if (k == entry || !(le[k] < 0.0f)) continue;
+                    float s = ls[k] / (ls[k] - le[k]);
+                    s = s < 0.0f ? 0.0f : s;
+                    if (s < smin) {
+                        smin = s;
+                        kmin = k;
+                    }
                 }
-            }
-            long long rec[kNV];
-            if (kmin < 0) {
-                quantize(le, -1, LE);
-                segment_current_fix(LS, LE, rec);
+                if (kmin < 0) {
+                    quantize(le, -1, LE);
+                    if (seg == 0) {
 #pragma unroll
-                for (int k = 0; k < 4; k++) rec[6 + k] = LE[k];
+                        for (int k = 0; k < 4; k++) E0[k] = LE[k];
+                        ends = true;
+                    } else {
+                        long long rec[kNV];
+                        segment_current_fix(LS, LE, rec);
+#pragma unroll
+                        for (int k = 0; k < 4; k++) rec[6 + k] = LE[k];
+                        push_record(a, (uint32_t)(T * a.nsp + spc), 0, i, seg, rec);
+                    }
+                    endT = T;
+                    done = true;
+                    break;
+                }
+                float lx[4];
+                int LX[4];
+#pragma unroll
+                for (int k = 0; k < 4; k++) lx[k] = ls[k] + smin * (le[k] - ls[k]);
+                quantize(lx, kmin, LX);
                 if (seg == 0) {
 #pragma unroll
-                    for (int c = 0; c < kNV; c++) vals[c] = rec[c];
+                    for (int k = 0; k < 4; k++) E0[k] = LX[k];
                 } else {
+                    long long rec[kNV];
+                    segment_current_fix(LS, LX, rec);
+#pragma unroll
+                    for (int k = 0; k < 4; k++) rec[6 + k] = 0;
                     push_record(a, (uint32_t)(T * a.nsp + spc), 0, i, seg, rec);
                 }
-                endT = T;
-                done = true;
-                break;
+                const int nb = (&a.tnbr[T].x)[kmin];
+                if (nb < 0) {
+                    long long wrec[kNV];
+#pragma unroll
+                    for (int k = 0; k < 6; k++) wrec[k] = 0;
+#pragma unroll
+                    for (int k = 0; k < 4; k++) wrec[6 + k] = LX[k];
+                    push_record(a, (uint32_t)(T * a.nsp + spc), 1, i, kMaxWalk, wrec);
+                    absorbed = true;
+                    done = true;
+                    break;
+                }
+                const int4 nn = a.tnodes[nb];
+                const int tv[4] = {tn.x, tn.y, tn.z, tn.w};
+                const int nv[4] = {nn.x, nn.y, nn.z, nn.w};
+#pragma unroll
+                for (int j = 0; j < 4; j++) {
+                    int l = 0;
+                    bool shared = false;
+#pragma unroll
+                    for (int k = 0; k < 4; k++)
+                        if (nv[j] == tv[k]) {
+                            l = LX[k];
+                            shared = true;
+                        }
+                    LS[j] = l;
+                    if (!shared) entry = j;
+                }
+                T = nb;
+                tn = nn;
             }
-            float lx[4];
-            int LX[4];
-#pragma unroll
-            for (int k = 0; k < 4; k++) lx[k] = ls[k] + smin * (le[k] - ls[k]);
-            quantize(lx, kmin, LX);
-            segment_current_fix(LS, LX, rec);
-#pragma unroll
-            for (int k = 0; k < 4; k++) rec[6 + k] = 0;
-            if (seg == 0) {
-#pragma unroll
-                for (int c = 0; c < kNV; c++) vals[c] = rec[c];
-            } else {
-                push_record(a, (uint32_t)(T * a.nsp + spc), 0, i, seg, rec);
-            }
-            const int nb = (&a.tnbr[T].x)[kmin];
-            if (nb < 0) {
-                long long wrec[kNV];
-#pragma unroll
-                for (int k = 0; k < 6; k++) wrec[k] = 0;
-#pragma unroll
-                for (int k = 0; k < 4; k++) wrec[6 + k] = LX[k];
-                push_record(a, (uint32_t)(T * a.nsp + spc), 1, i, kMaxWalk, wrec);
+            if (!done) {
+                atomicOr(a.status, (uint32_t)ST_WALK_CAP);
                 absorbed = true;
-                done = true;
-                break;
             }
-            const int4 nn = a.tnodes[nb];
-            const int tv[4] = {tn.x, tn.y, tn.z, tn.w};
-            const int nv[4] = {nn.x, nn.y, nn.z, nn.w};
-#pragma unroll
-            for (int j = 0; j < 4; j++) {
-                int l = 0;
-                bool shared = false;
-#pragma unroll
-                for (int k = 0; k < 4; k++)
-                    if (nv[j] == tv[k]) {
-                        l = LX[k];
-                        shared = true;
-                    }
-                LS[j] = l;
-                if (!shared) entry = j;
+            a.dx0[i] = Q[0];
+            a.dx1[i] = Q[1];
+            a.dx2[i] = Q[2];
+            a.dv0[i] = Vn[0];
+            a.dv1[i] = Vn[1];
+            a.dv2[i] = Vn[2];
+            a.did[i] = a.sid[src];
+            a.dkey[i] = absorbed ? a.dead_key : (((uint32_t)endT << 2) | (uint32_t)spc);
+            if (!absorbed) {
+                alive++;
+                const float ke = 0.5f * a.mw32[spc] * (Vn[0] * Vn[0] + Vn[1] * Vn[1] + Vn[2] * Vn[2]);
+                if (!(ke == ke) || !(Q[0] == Q[0])) atomicOr(a.status, (uint32_t)ST_NAN);
+                // error-free sum over the lane's particles
+                const float t = __fadd_rn(ke_hi, ke), z = __fsub_rn(t, ke_hi);
+                ke_lo = __fadd_rn(ke_lo, __fadd_rn(__fsub_rn(ke_hi, __fsub_rn(t, z)), __fsub_rn(ke, z)));
+                ke_hi = t;
             }
-            T = nb;
-            tn = nn;
         }
-        if (!done) {
-            atomicOr(a.status, (uint32_t)ST_WALK_CAP);
-            absorbed = true;
+        // ---- the deposit of the first pieces ----
+        const uint32_t k0 = __shfl_sync(0xFFFFFFFFu, rkey, 0);
+        if (__all_sync(0xFFFFFFFFu, rkey == k0)) {
+            if (k0 != ckey) {
+                flush();
+                ckey = k0;
+#pragma unroll
+                for (int c = 0; c < 6; c++) acc[c] = 0;
+#pragma unroll
+                for (int k = 0; k < 4; k++) accq[k] = 0;
+            }
+            spread = true;
+            acc[0] += (long long)S0[0] * E0[1] - (long long)E0[0] * S0[1];
+            acc[1] += (long long)S0[0] * E0[2] - (long long)E0[0] * S0[2];
+            acc[2] += (long long)S0[0] * E0[3] - (long long)E0[0] * S0[3];
+            acc[3] += (long long)S0[1] * E0[2] - (long long)E0[1] * S0[2];
+            acc[4] += (long long)S0[1] * E0[3] - (long long)E0[1] * S0[3];
+            acc[5] += (long long)S0[2] * E0[3] - (long long)E0[2] * S0[3];
+#pragma unroll
+            for (int k = 0; k < 4; k++) accq[k] += ends ? (unsigned)E0[k] : 0u;
+            continue;
         }
-        a.dx0[i] = Q[0];
-        a.dx1[i] = Q[1];
-        a.dx2[i] = Q[2];
-        a.dv0[i] = Vn[0];
-        a.dv1[i] = Vn[1];
-        a.dv2[i] = Vn[2];
-        a.did[i] = a.sid[src];
-        a.dkey[i] = absorbed ? a.dead_key : (((uint32_t)endT << 2) | (uint32_t)spc);
-        if (!absorbed) {
-            alive_out = 1;
-            ke = 0.5f * a.mw32[spc] * (Vn[0] * Vn[0] + Vn[1] * Vn[1] + Vn[2] * Vn[2]);
-            if (!(ke == ke) || !(Q[0] == Q[0])) atomicOr(a.status, (uint32_t)ST_NAN);
+        // several keys: a segmented inclusive scan (the four charges, < 2^29 for
+        // the 32 particles of a round, two per 64-bit channel); the carried run
+        // is kept out of it and added to its tail
+        long long w[8];
+        segment_current_fix(S0, E0, w);
+        {
+            const long long q0 = ends ? E0[0] : 0, q1 = ends ? E0[1] : 0, q2 = ends ? E0[2] : 0, q3 = ends ? E0[3] : 0;
+            w[6] = q0 | (q1 << 32);
+            w[7] = q2 | (q3 << 32);
         }
-        rkey = (uint32_t)(tet * a.nsp + spc);
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const uint32_t ko = __shfl_up_sync(0xFFFFFFFFu, rkey, off);
+#pragma unroll
+            for (int c = 0; c < 8; c++) {
+                const long long vo = __shfl_up_sync(0xFFFFFFFFu, w[c], off);
+                if (lane >= off && ko == rkey) w[c] += vo;
+            }
+        }
+        long long vals[kNV];
+#pragma unroll
+        for (int c = 0; c < 6; c++) vals[c] = w[c];
+        vals[6] = w[6] & 0xFFFFFFFFll;
+        vals[7] = (long long)((unsigned long long)w[6] >> 32);
+        vals[8] = w[7] & 0xFFFFFFFFll;
+        vals[9] = (long long)((unsigned long long)w[7] >> 32);
+        const uint32_t knext = __shfl_down_sync(0xFFFFFFFFu, rkey, 1);
+        if (ckey != kInvalid) {
+            long long t[kNV];
+            total(t);
+            if (ckey == k0) {
+                if (rkey == k0 && knext != rkey) {   // the first run's tail (it is not lane 31: there are several keys)
+#pragma unroll
+                    for (int c = 0; c < kNV; c++) vals[c] += t[c];
+                }
+            } else if (lane == 0) {
+                put_run(a.tacc, ckey, ckey == prevk || ckey == nextk, t);
+            }
+        }
+        if (lane < 31 && knext != rkey && rkey != kInvalid)
+            put_run(a.tacc, rkey, rkey == prevk || rkey == nextk, vals);
+        // the last run goes on: lane 31 holds its sum so far
+        ckey = __shfl_sync(0xFFFFFFFFu, rkey, 31);
+        spread = false;
+        const bool holds = lane == 31;
+#pragma unroll
+        for (int c = 0; c < 6; c++) acc[c] = holds ? vals[c] : 0;
+#pragma unroll
+        for (int k = 0; k < 4; k++) accq[k] = holds ? (unsigned)vals[6 + k] : 0u;
     }
-    reduce_block<float, long long, float>(a, rkey, vals, ke, alive_out, n_alive);
+    flush();
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const float b = __shfl_xor_sync(0xFFFFFFFFu, ke_hi, o), bl = __shfl_xor_sync(0xFFFFFFFFu, ke_lo, o);
+        const float t = __fadd_rn(ke_hi, b), z = __fsub_rn(t, ke_hi);
+        const float e = __fadd_rn(__fsub_rn(ke_hi, __fsub_rn(t, z)), __fsub_rn(b, z));
+        ke_lo = __fadd_rn(__fadd_rn(ke_lo, bl), e);
+        ke_hi = t;
+    }
+    alive = __reduce_add_sync(0xFFFFFFFFu, alive);
+    if (lane == 0) {
+        a.ke_part[gw] = (double)ke_hi + (double)ke_lo;
+        if (alive) atomicAdd(a.n_alive_next, alive);
+    }
 }
 
 // spanning runs: a head piece (the last run of a block, or a block's first run
 // that does not continue from the previous block) adds the following blocks'
 // first-run pieces of the same key in block order
-template <typename V>
-__global__ void __launch_bounds__(256) k_fixup(int n_blocks, int nsp, const uint32_t *__restrict__ skey,
+__global__ void __launch_bounds__(256) k_fixup(int n_blocks, const uint32_t *__restrict__ skey,
                                                const int *d_n_alive, const uint32_t *__restrict__ bkey,
-                                               const V *__restrict__ bval, V *__restrict__ tacc) {
+                                               const double *__restrict__ bval, double *__restrict__ tacc) {
     const long j = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= 2L * n_blocks) return;
     const uint32_t k = bkey[j];
@@ -1151,9 +1304,9 @@ __global__ void __launch_bounds__(256) k_fixup(int n_blocks, int nsp, const uint
     if (slot == 0) {
         const long p = blk * kPushBlock - 1;
         const int n_alive = *d_n_alive;
-        if (blk > 0 && p < n_alive && acc_index<V>(skey[p], nsp) == k) return;
+        if (blk > 0 && p < n_alive && acc_index<double>(skey[p], 1) == k) return;
     }
-    V sum[kNV];
+    double sum[kNV];
     for (int c = 0; c < kNV; c++) sum[c] = bval[j * kNV + c];
     for (long b = blk + 1; b < n_blocks && bkey[2 * b] == k; b++)
         for (int c = 0; c < kNV; c++) sum[c] += bval[2 * b * kNV + c];
@@ -1191,8 +1344,9 @@ __global__ void __launch_bounds__(256) k_overflow_reduce(const int *d_count, int
 // the records is needed, unlike the FP64 records of the PLAIN path.
 __global__ void __launch_bounds__(256) k_overflow_scatter(const int *d_count, int cap,
                                                           const unsigned long long *__restrict__ okey,
-                                                          const long long *__restrict__ oval, int oshift,
-                                                          unsigned long long *tacc, unsigned long long *wacc) {
+                                                          const long long *__restrict__ oval, int oshift, int nsp,
+                                                          const int4 *__restrict__ tnodes, unsigned long long *tacc,
+                                                          unsigned long long *nacc) {
     const int n = min(*d_count, cap);
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= n) return;
@@ -1200,8 +1354,13 @@ __global__ void __launch_bounds__(256) k_overflow_scatter(const int *d_count, in
     const size_t idx = (size_t)(tw >> 1);
     const long long *v = oval + (size_t)j * kNV;
     if (tw & 1ull) {
+        // a wall charge: to its nodes' wall sums (k_scatter_node_charge)
+        const size_t t = idx / nsp, q = idx - t * nsp;
+        const int4 tn = tnodes[t];
+        const int nd[4] = {tn.x, tn.y, tn.z, tn.w};
+#pragma unroll
         for (int c = 0; c < 4; c++)
-            if (v[6 + c]) atomicAdd(wacc + idx * 4 + c, (unsigned long long)v[6 + c]);
+            if (v[6 + c]) atomicAdd(nacc + 2 * ((size_t)nd[c] * nsp + q) + 1, (unsigned long long)v[6 + c]);
     } else {
         for (int c = 0; c < kNV; c++)
             if (v[c]) atomicAdd(tacc + idx * kNV + c, (unsigned long long)v[c]);
@@ -1363,29 +1522,26 @@ __global__ void k_load_particles(int n, int start, const double *__restrict__ x,
 }
 
 // MIXED node charges, tet by tet: each (tet, species) reads its four node
-// charges and four wall charges once (contiguous) and adds them to per-(node,
-// species) integer sums.  Integer additions commute, so the sums do not depend
+// charges once (contiguous) and adds them to per-(node, species) integer sums
+// (wall charges go there straight from their records).  Integer additions commute, so the sums do not depend
 // on the order of the atomics; a node gather would read one 8-byte value from
 // a different tet record per reference instead (7x the bytes, measured).
 __global__ void __launch_bounds__(256) k_scatter_node_charge(int nt, int nsp, const int4 *__restrict__ tnodes,
                                                              const long long *__restrict__ tacc,
-                                                             const long long *__restrict__ wacc,
                                                              unsigned long long *__restrict__ nacc) {
     const int tq = blockIdx.x * blockDim.x + threadIdx.x;
     if (tq >= nt * nsp) return;
     const int t = tq / nsp, q = tq - t * nsp;
     const longlong2 *a2 = reinterpret_cast<const longlong2 *>(tacc + (size_t)tq * kNV + 6);
-    const longlong2 *w2 = reinterpret_cast<const longlong2 *>(wacc + (size_t)tq * 4);
-    const longlong2 a01 = a2[0], a23 = a2[1], w01 = w2[0], w23 = w2[1];
-    const long long ca[4] = {a01.x, a01.y, a23.x, a23.y}, cw[4] = {w01.x, w01.y, w23.x, w23.y};
-    if ((ca[0] | ca[1] | ca[2] | ca[3] | cw[0] | cw[1] | cw[2] | cw[3]) == 0) return;
+    const longlong2 a01 = a2[0], a23 = a2[1];
+    const long long ca[4] = {a01.x, a01.y, a23.x, a23.y};
+    if ((ca[0] | ca[1] | ca[2] | ca[3]) == 0) return;
     const int4 tn = tnodes[t];
     const int nd[4] = {tn.x, tn.y, tn.z, tn.w};
 #pragma unroll
     for (int k = 0; k < 4; k++) {
         unsigned long long *o = nacc + 2 * ((size_t)nd[k] * nsp + q);
         if (ca[k]) atomicAdd(o, (unsigned long long)ca[k]);
-        if (cw[k]) atomicAdd(o + 1, (unsigned long long)cw[k]);
     }
 }
 
@@ -1518,7 +1674,7 @@ int particles_alloc(Sim *s, size_t cap) {
         return rc;
     const size_t blocks = std::max<size_t>(1, (cap + kPushBlock - 1) / kPushBlock);
     if ((rc = s->bcar.alloc(2 * blocks * kNV)) || (rc = s->bcar_key.alloc(2 * blocks)) ||
-        (rc = s->ke_part.alloc(blocks)))
+        (rc = s->ke_part.alloc(blocks * (kPushBlock / 32))))
         return rc;
     s->push_blocks_cap = blocks;
     s->cap = cap;
@@ -1576,9 +1732,11 @@ int upload_particles(Sim *s) {
     if (rc) return rc;
     // per-tet accumulators: one set per species in MIXED (fixed point is per unit charge)
     s->nsp = s->mixed ? std::max(1, s->n_species) : 1;
-    if ((rc = s->tacc.alloc((size_t)kNV * s->mesh->n_tets * s->nsp)) ||
-        (rc = s->wacc.alloc((size_t)4 * s->mesh->n_tets * s->nsp)))
-        return rc;
+    if ((rc = s->tacc.alloc((size_t)kNV * s->mesh->n_tets * s->nsp))) return rc;
+    if (s->mixed) {
+        if ((rc = s->nacc.alloc(2 * (size_t)s->mesh->n_nodes * s->nsp))) return rc;
+        FP_CUDA(cudaMemsetAsync(s->nacc.p, 0, sizeof(unsigned long long) * s->nacc.n, s->stream));
+    }
     PartBank &k = s->bank[0];
     for (const Sim::LoadRun &r : s->load_runs) {
         const int blocks = (r.n + 255) / 256;
@@ -1767,6 +1925,13 @@ static void fill_push_args(Sim *s, PushArgs<R, V> &a) {
     a.ke_part = s->ke_part.p;
 }
 
+// Particles of a MIXED push warp: kMaxRounds times 32 where that leaves every
+// SM its full 32 warps, fewer for fewer particles (152 SMs)
+static int push_rounds(long n) {
+    const long warps = 152L * 32;
+    return (int)std::min<long>(kMaxRounds, std::max<long>(1, n / (32 * warps)));
+}
+
 template <typename R, typename V>
 static int launch_push(Sim *s, int mode) {
     PushArgs<R, V> a;
@@ -1775,14 +1940,15 @@ static int launch_push(Sim *s, int mode) {
     // the live particles of this step are the first n_alive sorted entries
     // (in a batch the grid covers all n_total and the kernel reads n_alive)
     const int live = s->batch_mode ? s->n_total : s->hctl->n_alive;
-    const int blocks = std::max(1, (live + kPushBlock - 1) / kPushBlock);
+    const int rounds = s->mixed ? push_rounds(live) : 1;
+    const int blocks = std::max(1, (int)((live + (long)kPushBlock * rounds - 1) / ((long)kPushBlock * rounds)));
     FP_CUDA(cudaMemsetAsync(&dc->pad, 0, sizeof(int), s->stream));
     prof_begin(s, PH_PUSH);
     if (std::is_same<R, float>::value) {
         const PushArgs<float, long long> &am = reinterpret_cast<const PushArgs<float, long long> &>(a);
-        if (mode == 2) { k_push_mixed<2><<<blocks, kPushBlock, 0, s->stream>>>(am); note_launch(); }
-        else if (mode == 1) { k_push_mixed<1><<<blocks, kPushBlock, 0, s->stream>>>(am); note_launch(); }
-        else { k_push_mixed<0><<<blocks, kPushBlock, 0, s->stream>>>(am); note_launch(); }
+        if (mode == 2) { k_push_mixed<2><<<blocks, kPushBlock, 0, s->stream>>>(am, rounds); note_launch(); }
+        else if (mode == 1) { k_push_mixed<1><<<blocks, kPushBlock, 0, s->stream>>>(am, rounds); note_launch(); }
+        else { k_push_mixed<0><<<blocks, kPushBlock, 0, s->stream>>>(am, rounds); note_launch(); }
     } else {
         const PushArgs<double, double> &ap = reinterpret_cast<const PushArgs<double, double> &>(a);
         if (mode == 2) { k_push_plain<2><<<blocks, kPushBlock, 0, s->stream>>>(ap); note_launch(); }
@@ -1792,9 +1958,9 @@ static int launch_push(Sim *s, int mode) {
     prof_end(s, PH_PUSH);
     prof_begin(s, PH_DEPOSIT);
     FP_CUDA(cudaGetLastError());
-    // runs that span blocks are added in block order
-    { k_fixup<V><<<(2 * blocks + 255) / 256, 256, 0, s->stream>>>(blocks, s->nsp, s->skey.p, &dc->n_alive, s->bcar_key.p, (const V *)s->bcar.p, (V *)s->tacc.p); note_launch(); }
-    s->n_ke_parts = blocks;
+    // PLAIN: runs that span blocks are added in block order
+    if (!s->mixed) { k_fixup<<<(2 * blocks + 255) / 256, 256, 0, s->stream>>>(blocks, s->skey.p, &dc->n_alive, s->bcar_key.p, s->bcar.p, s->tacc.p); note_launch(); }
+    s->n_ke_parts = s->mixed ? blocks * (kPushBlock / 32) : blocks;
     FP_CUDA(cudaGetLastError());
     return PIC_OK;
 }
@@ -1804,7 +1970,7 @@ int particle_push(Sim *s, int charge_only) {
     const size_t vsz = 8;   // double or int64 accumulators
     for (int attempt = 0;; attempt++) {
         FP_CUDA(cudaMemsetAsync(s->tacc.p, 0, vsz * kNV * (size_t)m->n_tets * s->nsp, s->stream));
-        FP_CUDA(cudaMemsetAsync(s->wacc.p, 0, vsz * 4 * (size_t)m->n_tets * s->nsp, s->stream));
+        if (!s->mixed) FP_CUDA(cudaMemsetAsync(s->wacc.p, 0, vsz * 4 * (size_t)m->n_tets, s->stream));
         FP_CUDA(cudaMemsetAsync(&s->dctl.p->n_over, 0, sizeof(int), s->stream));
         if (s->n_total == 0) break;
         const int mode = charge_only ? 2 : (s->ab ? 1 : 0);
@@ -1838,7 +2004,7 @@ int particle_push(Sim *s, int charge_only) {
         // known on the host since the push, or (batch) a device count bounded by the buffer
         const int nover = s->batch_mode ? s->ocap : s->hctl->n_over;
         if (nover > 0 && s->mixed) {
-            { k_overflow_scatter<<<(nover + 255) / 256, 256, 0, s->stream>>>(&s->dctl.p->n_over, nover, s->okey.p, (const long long *)s->oval.p, oshift, (unsigned long long *)s->tacc.p, (unsigned long long *)s->wacc.p); note_launch(); }
+            { k_overflow_scatter<<<(nover + 255) / 256, 256, 0, s->stream>>>(&s->dctl.p->n_over, nover, s->okey.p, (const long long *)s->oval.p, oshift, s->nsp, m->tet_nodes.p, (unsigned long long *)s->tacc.p, s->nacc.p); note_launch(); }
             FP_CUDA(cudaGetLastError());
         } else if (nover > 0) {
             unsigned long long *ok;
@@ -1908,7 +2074,7 @@ static int particles_grow(Sim *s, size_t cap, size_t keep) {
         return rc;
     const size_t blocks = std::max<size_t>(1, (cap + kPushBlock - 1) / kPushBlock);
     if ((rc = s->bcar.alloc(2 * blocks * kNV)) || (rc = s->bcar_key.alloc(2 * blocks)) ||
-        (rc = s->ke_part.alloc(blocks)))
+        (rc = s->ke_part.alloc(blocks * (kPushBlock / 32))))
         return rc;
     s->push_blocks_cap = blocks;
     s->cap = cap;
@@ -1994,13 +2160,8 @@ int reduce_to_entities(Sim *s) {
     const SpeciesParams sp = species_params(s);
     if (s->mixed) {
         { k_gather_edges<long long><<<(m->n_edges + 255) / 256, 256, 0, s->stream>>>(m->n_edges, m->e2t_row.p, m->e2t.rowptr.p, m->e2t.col.p, (const long long *)s->tacc.p, s->nsp, sp, s->g.p, s->dg.p, s->g_new.p); note_launch(); }
-        if (!s->nacc.p) {
-            int rc = s->nacc.alloc(2 * (size_t)m->n_nodes * s->nsp);
-            if (rc) return rc;
-            FP_CUDA(cudaMemsetAsync(s->nacc.p, 0, sizeof(unsigned long long) * s->nacc.n, s->stream));
-        }
         const int ntq = m->n_tets * s->nsp;
-        { k_scatter_node_charge<<<(ntq + 255) / 256, 256, 0, s->stream>>>(m->n_tets, s->nsp, m->tet_nodes.p, (const long long *)s->tacc.p, (const long long *)s->wacc.p, s->nacc.p); note_launch(); }
+        { k_scatter_node_charge<<<(ntq + 255) / 256, 256, 0, s->stream>>>(m->n_tets, s->nsp, m->tet_nodes.p, (const long long *)s->tacc.p, s->nacc.p); note_launch(); }
         { k_node_charge_convert<<<(m->n_nodes + 255) / 256, 256, 0, s->stream>>>(m->n_nodes, s->nsp, sp, s->nacc.p, s->wall_prev.p, s->rho.p, s->wall.p); note_launch(); }
     } else {
         { k_gather_edges<double><<<(m->n_edges + 255) / 256, 256, 0, s->stream>>>(m->n_edges, m->e2t_row.p, m->e2t.rowptr.p, m->e2t.col.p, (const double *)s->tacc.p, 1, sp, s->g.p, s->dg.p, s->g_new.p); note_launch(); }
