@@ -101,7 +101,7 @@ struct DevCsr {
 struct DevSell {
     int n_rows = 0, n_slices = 0;
     long long n_elems = 0;
-    int narrow = 0;
+    int narrow = 0, max_width = 0;
     DevBuf<int> ptr, width, col, base;
     DevBuf<unsigned char> off;
 };

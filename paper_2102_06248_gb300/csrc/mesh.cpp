@@ -746,6 +746,7 @@ int mesh_upload(Mesh *m) {
         (rc = m->K_diag.upload(H.K_diag)) || (rc = m->As.base.upload(H.sell_base)) || (rc = m->As.off.upload(H.sell_off)))
         return rc;
     m->As.narrow = !H.sell_base.empty();
+    for (int w : H.sell_w) m->As.max_width = std::max(m->As.max_width, w);
     m->Hs.n_rows = m->n_faces;
     m->Hs.n_slices = (int)H.hsell_w.size();
     m->Hs.n_elems = H.hsell_ptr.empty() ? 0 : H.hsell_ptr.back();
@@ -756,8 +757,11 @@ int mesh_upload(Mesh *m) {
     m->Ls.n_slices = (int)H.lsell_w.size();
     m->Ls.n_elems = H.lsell_ptr.empty() ? 0 : H.lsell_ptr.back();
     if ((rc = m->Ls.ptr.upload(H.lsell_ptr)) || (rc = m->Ls.width.upload(H.lsell_w)) ||
-        (rc = m->Ls.col.upload(H.lsell_col)) || (rc = m->Ls_val.upload(H.lsell_L)) || (rc = m->L_diag.upload(H.L_diag)))
+        (rc = m->Ls.col.upload(H.lsell_col)) || (rc = m->Ls_val.upload(H.lsell_L)) || (rc = m->L_diag.upload(H.L_diag)) ||
+        (rc = m->Ls.base.upload(H.lsell_base)) || (rc = m->Ls.off.upload(H.lsell_off)))
         return rc;
+    m->Ls.narrow = !H.lsell_base.empty();
+    for (int w : H.lsell_w) m->Ls.max_width = std::max(m->Ls.max_width, w);
     if ((rc = m->node_int.upload(H.node_int)) || (rc = m->int_node.upload(H.int_node))) return rc;
     if ((rc = csr(H.e2f, &m->e2f)) || (rc = m->e2f_sgn.upload(H.e2f_sgn))) return rc;
     if ((rc = csr(H.n2e, &m->n2e)) || (rc = m->n2e_sgn.upload(H.n2e_sgn))) return rc;

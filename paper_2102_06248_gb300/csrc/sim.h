@@ -64,6 +64,9 @@ struct Control {
 struct PcgArgs {
     int n, n_slices;
     const int *sp, *sw;           // SELL-32: slice offsets and widths
+    const int *col;               // ... columns and FP64 values (k_pcg_small)
+    const double *Av;
+    int max_width;
     const unsigned char *rec;     // the matrix as FP64 records (stream.cuh)
     int wide;                     // records with 32-bit columns
     int evict_first;              // matrix larger than L2 can keep: stream it through

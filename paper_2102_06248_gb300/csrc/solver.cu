@@ -791,6 +791,8 @@ __device__ __forceinline__ int find_slice(const int *__restrict__ sp, int ns, lo
     return lo;
 }
 
+extern __shared__ __align__(128) unsigned char s_ring[];   // dynamic shared memory of the persistent kernels
+
 // Per-block context of one solve.  The slices are dealt to the run's warps in
 // contiguous runs of equal numbers of entries; of the block's T / 32 warps,
 // `warps` take part (all of them unless the system has fewer slices than the
@@ -1162,6 +1164,260 @@ __device__ __forceinline__ void pcg_body(const PcgArgs &a, const int nb, const i
         st->done = 1;
         st->failed = failed;
         if (failed && !a.quiet) atomicOr(a.status, (uint32_t)ST_CG_NO_CONV);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// FP64 PCG on a system small enough for one SELL slice per warp (the fields of
+// small meshes, their node Laplacians).  Such an iteration is a chain of
+// latencies: two meetings of the blocks, the FP64 instructions of the
+// reduction and of the scalars, loads of vectors from L2.  So
+//  * a lane keeps its row of every vector in registers and the warp its
+//    slice's entries in shared memory for the whole solve; only the vector the
+//    product gathers goes through L2;
+//  * the recurrence is the pipelined one (Ghysels and Vanroose, "Hiding global
+//    synchronization latency in the preconditioned Conjugate Gradient
+//    algorithm", 2014): with m = D^-1 w and n = A m it needs one meeting of
+//    the blocks per iteration, and n does not wait for the scalars, so the
+//    product runs while four more warps of the block add the partials and form
+//    the scalars;
+//  * the iterates are those of PCG up to rounding, which the longer recurrence
+//    amplifies: the solution is checked against b - A x and continued from,
+//    twice at most, if it misses the stopping rule by more than 2%.
+// Per iteration, streamed form and this: 20^3 (52,460 rows) 12.2 and 7.5 us,
+// 16^3 (26,416 rows) 10.7 and 7.1 us, 6^3 (1,206 rows) 9.6 and 6.2 us.
+// ---------------------------------------------------------------------------
+constexpr int kSmallWarps = 12;               // slices of a block; four more warps reduce
+constexpr int kSmallThreads = 32 * (kSmallWarps + 4);
+constexpr int kSmallWidth = 32;               // columns of a slice held in shared memory
+constexpr int kSmallSlice = kSmallWidth * 32 * 12;
+constexpr int kSmallRestarts = 2;
+constexpr double kSmallTol2 = 0.9e-26;        // smallest relative tolerance (squared) of the pipelined recurrence
+constexpr int kSmallBlocks = 160;             // partials a warp adds with five loads a lane
+
+// the whole solve, run by block `bid` of the nb blocks that own it
+__device__ __forceinline__ void small_body(const PcgArgs &a, const int nb, const int bid) {
+    __shared__ double shv[3][kSmallWarps * 32];
+    __shared__ unsigned long long shm[kSmallWarps * 32];
+    __shared__ double res[4];
+    struct Scalars {
+        double alpha, ralpha, rgamma, beta;   // in this order (lanes 0..3)
+        double gamma, rr, bb, stop, abs_inf, tol2;
+        int iters, fresh, done, failed, ok, checked;
+    };
+    __shared__ Scalars sc;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int per = (a.n_slices + nb - 1) / nb;              // slices of a block
+    const int sl = bid * per + warp;
+    const bool holds = warp < per && sl < a.n_slices;        // this warp has a slice
+    const int active = min(per, a.n_slices - bid * per);     // warps of the block that have one
+    const int i = sl * 32 + lane;
+    double *sv = reinterpret_cast<double *>(s_ring + (size_t)warp * kSmallSlice);
+    int *scol = reinterpret_cast<int *>(sv + kSmallWidth * 32);
+    int width = 0;
+    double x = 0, r = 0, u = 0, w = 0, m = 0, p = 0, s = 0, q = 0, z = 0, d = 0, b = 0;
+    if (holds) {
+        const int k0 = a.sp[sl];
+        width = a.sw[sl];
+        for (int j = 0; j < width; j++) {
+            sv[32 * j + lane] = a.Av[k0 + 32 * j + lane];
+            scol[32 * j + lane] = a.col[k0 + 32 * j + lane];
+        }
+        b = a.b[i];
+        d = a.Dinv[i];
+        if (!a.x_zero) x = a.x[i];
+    }
+    if (threadIdx.x == 0) {
+        sc.abs_inf = a.abs_inf;
+        sc.tol2 = a.tol2;
+        if (a.abs_src) {
+            const double qv = *a.abs_src;
+            if (qv > 0.0) sc.abs_inf = a.abs_factor * qv;
+            else sc.tol2 = a.fallback_tol2;
+        }
+        sc.iters = sc.done = sc.failed = sc.checked = 0;
+        sc.fresh = 1;
+    }
+    unsigned int epoch = 0;
+    // row of A v: two chains, every gather of 24 columns in flight at once
+    auto spmv = [&](const double *v) -> double {
+        double s0 = 0, s1 = 0;
+        for (int j0 = 0; j0 < width; j0 += 24) {
+            double g[24];
+#pragma unroll
+            for (int j = 0; j < 24; j++) g[j] = j0 + j < width ? v[scol[32 * (j0 + j) + lane]] : 0.0;
+#pragma unroll
+            for (int j = 0; j < 24; j += 2) {
+                if (j0 + j < width) s0 = fma(sv[32 * (j0 + j) + lane], g[j], s0);
+                if (j0 + j + 1 < width) s1 = fma(sv[32 * (j0 + j + 1) + lane], g[j + 1], s1);
+            }
+        }
+        return s0 + s1;
+    };
+    // meets the other blocks (all threads of the block; the reducing warps wait for them)
+    auto meet = [&]() -> bool {
+        __syncthreads();
+        epoch++;
+        if (threadIdx.x == 32 * kSmallWarps) {
+            red_release_add(&a.gb->count, 1u);
+            sc.ok = spin_until(a.gb, &a.gb->count, epoch * (unsigned)nb, a.spin_limit);
+        }
+        __syncthreads();
+        return sc.ok != 0;
+    };
+    // meets the other blocks with three sums and a maximum; work() runs in the
+    // slices' warps while the others add the partials and run scal(t, warp, lane)
+    auto reduce = [&](double v0, double v1, double v2, double vm, auto work, auto scal) -> bool {
+        if (warp < kSmallWarps) {
+            const int t = threadIdx.x;
+            shv[0][t] = v0;
+            shv[1][t] = v1;
+            shv[2][t] = v2;
+            shm[t] = abs_bits(vm);
+        }
+        __syncthreads();
+        epoch++;
+        double *part = a.part + (size_t)(epoch & 1u) * 4 * nb;
+        const int dw = warp - kSmallWarps;
+        if (dw >= 0) {
+            if (dw < 3) {
+                double c[4] = {0, 0, 0, 0};
+#pragma unroll
+                for (int k = 0; k < kSmallWarps; k++)
+                    if (k < active) c[k & 3] += shv[dw][32 * k + lane];
+                const double t = warp_sum_d((c[0] + c[1]) + (c[2] + c[3]));
+                if (lane == 0) part[dw * nb + bid] = t;
+            } else {
+                unsigned long long t = 0;
+                for (int k = 0; k < active; k++) t = max(t, shm[32 * k + lane]);
+                t = warp_max_u64(t);
+                if (lane == 0) part[3 * nb + bid] = __longlong_as_double((long long)t);
+            }
+            sync_four_warps();
+            if (threadIdx.x == 32 * kSmallWarps) {
+                red_release_add(&a.gb->count, 1u);
+                sc.ok = spin_until(a.gb, &a.gb->count, epoch * (unsigned)nb, a.spin_limit);
+            }
+            sync_four_warps();
+        }
+        __syncthreads();
+        if (!sc.ok) return false;
+        if (dw < 0) {
+            work();
+        } else {
+            double c[5];
+#pragma unroll
+            for (int k = 0; k < 5; k++) c[k] = lane + 32 * k < nb ? __ldcg(part + dw * nb + lane + 32 * k) : 0.0;
+            if (dw < 3) {
+                const double t = warp_sum_d(((c[0] + c[1]) + (c[2] + c[3])) + c[4]);
+                if (lane == 0) res[dw] = t;
+            } else {
+                unsigned long long t = 0;
+#pragma unroll
+                for (int k = 0; k < 5; k++) t = max(t, (unsigned long long)__double_as_longlong(c[k]));
+                t = warp_max_u64(t);
+                if (lane == 0) res[3] = __longlong_as_double((long long)t);
+            }
+            sync_four_warps();
+            if (dw < 2) {
+                const double t[4] = {res[0], res[1], res[2], res[3]};
+                scal(t, dw, lane);
+            }
+        }
+        __syncthreads();
+        return true;
+    };
+    double *buf[2] = {a.u, a.w};
+    int turn = 0;
+    bool good = true;
+    // r = b - A x (x in memory, complete in every block)
+    if (holds) r = a.x_zero ? b : b - spmv(a.x);
+    while (true) {
+        // from r: u = D^-1 r, w = A u, m = D^-1 w, no directions yet
+        u = d * r;
+        p = s = q = z = 0;
+        if (holds) buf[turn][i] = u;
+        good = reduce(b * b, 0.0, 0.0, 0.0, [&]() { if (holds) w = spmv(buf[turn]); },
+                      [&](const double *t, int wp, int l) {
+                          if (wp + l == 0) {
+                              sc.bb = t[0];
+                              sc.stop = sc.tol2 * t[0];
+                          }
+                      });
+        if (!good) break;
+        turn ^= 1;
+        m = d * w;
+        while (true) {
+            if (holds) buf[turn][i] = m;
+            double n = 0;
+            good = reduce(r * u, r * r, w * u, r, [&]() { if (holds) n = spmv(buf[turn]); },
+                          [&](const double *t, int wp, int l) {
+                              if (wp == 0) {
+                                  const double be = sc.fresh ? 0.0 : t[0] * sc.rgamma;
+                                  const double den = sc.fresh ? t[2] : t[2] - be * t[0] * sc.ralpha;
+                                  __syncwarp();
+                                  const double o = (l == 0 ? t[0] : l == 1 ? den : 1.0) / (l == 0 ? den : t[0]);
+                                  if (l < 4) (&sc.alpha)[l] = l == 3 ? be : o;
+                              } else if (l == 0) {
+                                  sc.gamma = t[0];
+                                  sc.rr = t[1];
+                                  int done = sc.bb == 0.0 || t[1] <= sc.stop || t[3] <= sc.abs_inf;
+                                  if (!done && sc.iters >= a.max_iters) done = sc.failed = 1;
+                                  sc.done = done;
+                              }
+                          });
+            if (!good || sc.done) break;
+            turn ^= 1;
+            const double al = sc.alpha, be = sc.beta;
+            z = fma(be, z, n);
+            q = fma(be, q, m);
+            s = fma(be, s, w);
+            p = fma(be, p, u);
+            x = fma(al, p, x);
+            r = fma(-al, s, r);
+            u = fma(-al, q, u);
+            w = fma(-al, z, w);
+            m = d * w;
+            if (threadIdx.x == 0) {
+                sc.iters++;
+                sc.fresh = 0;
+            }
+        }
+        if (!good) break;
+        if (sc.bb == 0.0) x = 0.0;
+        if (holds) {
+            a.x[i] = x;
+            a.r[i] = r;
+        }
+        if (sc.failed || sc.bb == 0.0 || sc.checked >= kSmallRestarts) break;
+        // the residual of x itself
+        if (!(good = meet())) break;
+        double t = 0;
+        if (holds) t = b - spmv(a.x);
+        good = reduce(t * t, 0.0, 0.0, t, []() {}, [&](const double *v, int wp, int l) {
+            if (wp + l == 0) {
+                sc.done = v[0] <= 1.04 * sc.stop || v[3] <= 1.02 * sc.abs_inf;
+                sc.checked++;
+                sc.fresh = 1;
+            }
+        });
+        if (!good || sc.done) break;
+        r = t;
+    }
+    if (bid == 0 && threadIdx.x == 0) {
+        CgState *st = a.st;
+        st->done = 1;
+        st->failed = good ? sc.failed : 1;
+        if (!good) {
+            atomicOr(a.status, (uint32_t)ST_BARRIER);
+            return;
+        }
+        st->iters = sc.iters;
+        st->outer = 0;
+        st->rr = sc.rr;
+        st->rz = sc.gamma;
+        st->bb = sc.bb;
+        if (sc.failed && !a.quiet) atomicOr(a.status, (uint32_t)ST_CG_NO_CONV);
     }
 }
 
@@ -1571,13 +1827,26 @@ __global__ void __launch_bounds__(kMgThreads, 1) k_mg_pcg(const MgArgs a) {
 }
 
 // one solve per launch (its arguments passed by value), one block per SM
-extern __shared__ __align__(128) unsigned char s_ring[];
 template <bool REFINE, bool WIDE>
 __global__ void __launch_bounds__(PcgShape<REFINE, WIDE>::threads, 1) k_pcg_persistent(const PcgArgs a) {
     using P = PcgShape<REFINE, WIDE>;
     __shared__ double shv[4 * P::threads];
     __shared__ unsigned long long shm[P::threads];
     pcg_body<REFINE, WIDE, P::threads, P::ring>(a, gridDim.x, blockIdx.x, s_ring, shv, shm);
+}
+
+__global__ void __launch_bounds__(kSmallThreads, 1) k_pcg_small(const PcgArgs a) {
+    small_body(a, gridDim.x, blockIdx.x);
+}
+__global__ void __launch_bounds__(kSmallThreads, 1) k_pcg_small_batched(const __grid_constant__ PcgBatch<kMaxBatchRuns> B) {
+    __shared__ PcgArgs sa;
+    if (threadIdx.x == 0) {
+        int ri = 0;
+        while (ri + 1 < B.n_runs && (int)blockIdx.x >= B.run[ri + 1].block0) ri++;
+        sa = B.run[ri];
+    }
+    __syncthreads();
+    small_body(sa, sa.blocks, (int)blockIdx.x - sa.block0);
 }
 
 // several solves of one kind per launch: run r owns blocks [block0, block0 + blocks).
@@ -1888,6 +2157,45 @@ static int assign_blocks(PcgArgs *runs, int n_runs, int budget) {
     return PIC_OK;
 }
 
+// FP64 systems whose slices all find a warp (one block per SM): one slice a
+// warp for the whole solve, whatever the launch shape asked for.  20^3 (52,460
+// rows, 1,640 slices, 227 iterations) 2.77 -> 1.70 ms; systems beyond take the streamed
+// form, whose iteration is bound by the FP64 pipes rather than by latency.  So
+// do relative tolerances below 1e-13, which the pipelined recurrence reaches
+// only with restarts (20^3 Laplacian, 1e-14: 3.0 ms against 1.3 ms).  A run
+// gets the same blocks alone and in a batch, so its results are the same
+// bits.
+static int launch_small(PcgArgs *runs, int n_runs, cudaStream_t st, bool *launched) {
+    const int most = std::min(sm_count(), kSmallBlocks);
+    int G = 0;
+    for (int r = 0; r < n_runs; r++) {
+        PcgArgs &a = runs[r];
+        if (a.max_width > kSmallWidth || a.n_slices > kSmallWarps * most || (!a.abs_src && a.tol2 < kSmallTol2))
+            return PIC_OK;
+        int blocks = std::min(most, std::max(1, (a.n_slices + kSlicesPerPcgBlock - 1) / kSlicesPerPcgBlock));
+        const int per = (a.n_slices + blocks - 1) / blocks;
+        blocks = (a.n_slices + per - 1) / per;   // no block without a slice
+        a.block0 = G;
+        a.blocks = blocks;
+        G += blocks;
+    }
+    if (G > sm_count()) return PIC_OK;
+    static CoopKernel one((const void *)k_pcg_small, kSmallThreads, kSmallSlice * kSmallWarps / (kSmallThreads / 32));
+    static CoopKernel many((const void *)k_pcg_small_batched, kSmallThreads, kSmallSlice * kSmallWarps / (kSmallThreads / 32));
+    CoopKernel &kernel = n_runs == 1 ? one : many;
+    if (kernel.per_sm() <= 0) {
+        set_error("the persistent PCG needs a device with cooperative launch");
+        return PIC_ERR_CUDA;
+    }
+    PcgBatch<kMaxBatchRuns> all;
+    all.n_runs = n_runs;
+    for (int r = 0; r < n_runs; r++) all.run[r] = runs[r];
+    { k_reset_barriers<<<1, kMaxBatchRuns, 0, st>>>(all); note_launch(); }
+    void *args[] = {n_runs == 1 ? (void *)&all.run[0] : (void *)&all};
+    *launched = true;
+    return kernel.launch(G, args, st);
+}
+
 // One cooperative launch of the persistent PCG over n_runs solves on stream
 // st.  Results and failures reach the host through each run's CgState and
 // status word at the next synchronisation.
@@ -1903,6 +2211,11 @@ int launch_pcg_runs(PcgArgs *runs, int n_runs, int blocks_per_sm, cudaStream_t s
             set_error("the solves of one persistent launch must all be FP64 or all be refinements");
             return PIC_ERR_INVALID_ARG;
         }
+    if (!refine) {
+        bool launched = false;
+        int rc = launch_small(runs, n_runs, st, &launched);
+        if (rc || launched) return rc;
+    }
     bool wide = false;
     for (int r = 0; r < n_runs; r++) wide = wide || runs[r].wide;
     CoopKernel &kernel = pcg_kernel(one, refine, wide, build);
@@ -1924,8 +2237,11 @@ int launch_pcg_runs(PcgArgs *runs, int n_runs, int blocks_per_sm, cudaStream_t s
     return kernel.launch(G, args, st);
 }
 
-static PcgArgs matrix_args(const DevSell &A, const DevBuf<unsigned char> &rec) {
+static PcgArgs matrix_args(const DevSell &A, const double *Av, const DevBuf<unsigned char> &rec) {
     PcgArgs a{};
+    a.col = A.col.p;
+    a.Av = Av;
+    a.max_width = A.max_width;
     a.n = A.n_rows;
     a.n_slices = A.n_slices;
     a.sp = A.ptr.p;
@@ -1936,12 +2252,12 @@ static PcgArgs matrix_args(const DevSell &A, const DevBuf<unsigned char> &rec) {
     return a;
 }
 
-static PcgArgs make_args(Sim *s, const DevSell &A, const DevBuf<unsigned char> &rec, const double *Dinv, const double *b, double *x,
+static PcgArgs make_args(Sim *s, const DevSell &A, const double *Av, const DevBuf<unsigned char> &rec, const double *Dinv, const double *b, double *x,
                          double *r, double *u, double *w, double *p, double *sv, double *part, CgState *st,
                          double tol, double fallback_tol, int max_iters, const double *abs_src, double abs_factor,
                          bool x_zero, bool quiet) {
     Control *dc = s->dctl.p;
-    PcgArgs a = matrix_args(A, rec);
+    PcgArgs a = matrix_args(A, Av, rec);
     a.Dinv = Dinv;
     a.b = b;
     a.x = x;
@@ -1970,7 +2286,7 @@ static PcgArgs make_args(Sim *s, const DevSell &A, const DevBuf<unsigned char> &
 // iterations without an error (training samples, solver timing)
 PcgArgs pcg_args_truncated(Sim *s, int iters) {
     const Mesh *m = s->mesh;
-    return make_args(s, m->As, s->A_rec, s->Dinv.p, s->rhs.p, s->x.p, s->cg_r.p, s->cg_z.p, s->cg_q.p, s->cg_p0.p,
+    return make_args(s, m->As, s->A_val.p, s->A_rec, s->Dinv.p, s->rhs.p, s->x.p, s->cg_r.p, s->cg_z.p, s->cg_q.p, s->cg_p0.p,
                      s->cg_p1.p, s->cg_part.p, &s->dctl.p->cg, 0.0, 0.0, iters, nullptr, 0.0, true, true);
 }
 
@@ -1990,7 +2306,7 @@ PcgArgs pcg_args_newmark_truncated(Sim *s, int iters) {
 // the stopping rule in both precisions.
 PcgArgs pcg_args_newmark(Sim *s) {
     const Mesh *m = s->mesh;
-    PcgArgs a = make_args(s, m->As, s->A_rec, s->Dinv.p, s->rhs.p, s->x.p, s->cg_r.p, s->cg_z.p, s->cg_q.p,
+    PcgArgs a = make_args(s, m->As, s->A_val.p, s->A_rec, s->Dinv.p, s->rhs.p, s->x.p, s->cg_r.p, s->cg_z.p, s->cg_q.p,
                           s->cg_p0.p, s->cg_p1.p, s->cg_part.p, &s->dctl.p->cg, s->cfg.cg_tol, 0.0,
                           s->cfg.cg_max_iters, nullptr, 0.0, false, false);
     if (s->mixed && s->A_rec32.p) {
@@ -2017,7 +2333,7 @@ PcgArgs pcg_args_completion(Sim *s) {
     const Mesh *m = s->mesh;
     // (in both precisions FP64: the completion is bound by the latency of its
     // iterations, not by their arithmetic, and FP32 corrections took more)
-    return make_args(s, m->Ls, m->L_rec, s->L_Dinv.p, s->l_b.p, s->l_x.p, s->l_r.p, s->l_z.p, s->l_q.p,
+    return make_args(s, m->Ls, m->Ls_val.p, m->L_rec, s->L_Dinv.p, s->l_b.p, s->l_x.p, s->l_r.p, s->l_z.p, s->l_q.p,
                      s->l_p0.p, s->l_p1.p, s->l_part.p, &s->dctl.p->lap, 0.0, s->cfg.init_tol, 20000,
                      &s->dctl.p->qmax, s->cfg.completion_tol, true, false);
 }
@@ -2060,7 +2376,7 @@ int laplacian_solve(Sim *s, const double *rhs_int, double *x_int, double tol, co
                     double abs_factor) {
     const Mesh *m = s->mesh;
     if (m->n_int_nodes == 0) return PIC_OK;
-    PcgArgs a = make_args(s, m->Ls, m->L_rec, s->L_Dinv.p, rhs_int, x_int, s->l_r.p, s->l_z.p, s->l_q.p,
+    PcgArgs a = make_args(s, m->Ls, m->Ls_val.p, m->L_rec, s->L_Dinv.p, rhs_int, x_int, s->l_r.p, s->l_z.p, s->l_q.p,
                           s->l_p0.p, s->l_p1.p, s->l_part.p, &s->dctl.p->lap, tol, s->cfg.init_tol, 20000, abs_src,
                           abs_factor, true, false);
     return launch_pcg_runs(&a, 1, s->cfg.solver_blocks_per_sm, s->stream);
@@ -2523,7 +2839,7 @@ int electrostatic_solve_noalloc(const Mesh *m, const double *rho_nodes, double *
             return PIC_ERR_STATE;
         }
         { k_recip_diag<<<(nin + 255) / 256, 256, 0, st>>>(nin, m->L_diag.p, v[6]); note_launch(); }
-        PcgArgs a = matrix_args(m->Ls, m->L_rec);
+        PcgArgs a = matrix_args(m->Ls, m->Ls_val.p, m->L_rec);
         a.Dinv = v[6];
         a.b = b;
         a.x = x;
