@@ -31,6 +31,7 @@
 // depend on scheduling.
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <cmath>
 #include <vector>
 
@@ -83,6 +84,21 @@ __global__ void k_final_sums(int nb, int nv, const double *__restrict__ part, do
     if (lane == 0) out[c] = s;
 }
 
+// the sum of nb partials, by one warp in the order of k_final_sums, handed to
+// the whole block
+__device__ __forceinline__ double block_total(int nb, const double *__restrict__ part) {
+    __shared__ double total;
+    if (threadIdx.x < 32) {
+        double s = 0.0;
+        for (int b = threadIdx.x; b < nb; b += 32) s += part[b];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xFFFFFFFFu, s, o);
+        if (threadIdx.x == 0) total = s;
+    }
+    __syncthreads();
+    return total;
+}
+
 // sum_i (x1_i y1_i), sum_i (x2_i y2_i) (x2 may be NULL), scaled by w_i when w != NULL
 __global__ void __launch_bounds__(kT) k_dot2(int n, const double *__restrict__ x1, const double *__restrict__ y1,
                                             const double *__restrict__ x2, const double *__restrict__ y2,
@@ -96,32 +112,45 @@ __global__ void __launch_bounds__(kT) k_dot2(int n, const double *__restrict__ x
     block_partial<2>(v, part);
 }
 
-// y = A x on SELL-32 (FP64)
-__global__ void __launch_bounds__(kT) k_spmv(int n, int nsl, const int *__restrict__ sp, const int *__restrict__ sw,
-                                            const int *__restrict__ col, const double *__restrict__ val,
-                                            const double *__restrict__ x, double *__restrict__ y) {
-    const int lane = threadIdx.x & 31;
-    for (int sl = blockIdx.x * kW + (threadIdx.x >> 5); sl < nsl; sl += gridDim.x * kW) {
-        const int kb = sp[sl] + lane, kw = sw[sl];
-        double s = 0.0;
-        for (int j = 0; j < kw; j++) s = fma(val[kb + 32 * j], x[col[kb + 32 * j]], s);
-        const int i = sl * 32 + lane;
-        if (i < n) y[i] = s;
-    }
-}
-
 // ---- static inputs: Ahat (SELL layout, FP32), 1/sqrt(d), log d ----
-__global__ void k_prep_rows(int n, const double *__restrict__ Dinv, double *__restrict__ isd,
-                            double *__restrict__ logd) {
+__global__ void k_prep_rows(int n, const int *__restrict__ edge, const double *__restrict__ Dinv,
+                            double *__restrict__ isd, double *__restrict__ logd) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) {
-        isd[i] = sqrt(Dinv[i]);
-        logd[i] = -log(Dinv[i]);
+        isd[i] = sqrt(Dinv[edge[i]]);
+        logd[i] = -log(Dinv[edge[i]]);
     }
 }
 
+// the columns of the network's rows: the rows of the edges that share a tet,
+// in increasing order (insertion in place), then the row itself
+__global__ void k_rows_cols(int n, int nsl, const int *__restrict__ sp, const int *__restrict__ sw,
+                            const int *__restrict__ canon, const int *__restrict__ tptr, const int *__restrict__ tref,
+                            const int *__restrict__ tet_edge, const int *__restrict__ row, int *__restrict__ col) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= 32 * nsl) return;
+    int *c = col + sp[i >> 5] + (i & 31);
+    const int w = sw[i >> 5];
+    int m = 0;
+    if (i < n)
+        for (int a = tptr[canon[i]]; a < tptr[canon[i] + 1]; a++)
+            for (int k = 0; k < 6; k++) {
+                const int e = tet_edge[6 * (size_t)(tref[a] / 6) + k];
+                if (e >= n) continue;
+                const int x = row[e];
+                int j = m;
+                while (j > 0 && c[32 * (j - 1)] > x) j--;
+                if ((j > 0 && c[32 * (j - 1)] == x) || m >= w) continue;
+                for (int q = m++; q > j; q--) c[32 * q] = c[32 * (q - 1)];
+                c[32 * j] = x;
+            }
+    for (; m < w; m++) c[32 * m] = min(i, n - 1);
+}
+
+// (element values are looked up in A's rows, whose padding has the value 0)
 __global__ void k_prep_ahat(int n, int nsl, const int *__restrict__ sp, const int *__restrict__ sw,
-                            const int *__restrict__ col, const double *__restrict__ val,
+                            const int *__restrict__ col, const int *__restrict__ edge, const int *__restrict__ asp,
+                            const int *__restrict__ asw, const int *__restrict__ acol, const double *__restrict__ val,
                             const double *__restrict__ isd, const double *__restrict__ logd,
                             const double *__restrict__ mean_logd, float *__restrict__ ahat,
                             float *__restrict__ feat_a) {
@@ -130,9 +159,18 @@ __global__ void k_prep_ahat(int n, int nsl, const int *__restrict__ sp, const in
     if (sl >= nsl) return;
     const int i = sl * 32 + lane, kb = sp[sl] + lane, kw = sw[sl];
     const double si = i < n ? isd[i] : 0.0;
+    const int e = i < n ? edge[i] : 0, ab = asp[e >> 5] + (e & 31), aw = asw[e >> 5];
+    int last = -1;   // columns increase along a row; padding repeats the row itself
     for (int j = 0; j < kw; j++) {
-        const int k = kb + 32 * j;
-        ahat[k] = i < n ? (float)(val[k] * si * isd[col[k]]) : 0.0f;
+        const int k = kb + 32 * j, c = col[k];
+        double v = 0.0;
+        if (i < n && c > last) {
+            const int ce = edge[c];
+            for (int q = 0; q < aw; q++)
+                if (acol[ab + 32 * q] == ce) v += val[ab + 32 * q];
+            last = c;
+        }
+        ahat[k] = i < n ? (float)(v * si * isd[c]) : 0.0f;
     }
     if (i < n) feat_a[i] = (float)(logd[i] - mean_logd[0] / n);
 }
@@ -144,32 +182,62 @@ __global__ void k_sum(int n, const double *__restrict__ a, double *part) {
 }
 
 // rho^2 n = sum r_i^2 / d_i
-__global__ void __launch_bounds__(kT) k_rnorm(int n, const double *__restrict__ r, const double *__restrict__ Dinv,
-                                             double *part) {
+__global__ void __launch_bounds__(kT) k_rnorm(int n, const int *__restrict__ edge, const double *__restrict__ r,
+                                             const double *__restrict__ Dinv, double *part) {
     double v[1] = {0.0};
-    for (int i = blockIdx.x * kT + threadIdx.x; i < n; i += gridDim.x * kT) v[0] = fma(r[i] * Dinv[i], r[i], v[0]);
+    for (int i = blockIdx.x * kT + threadIdx.x; i < n; i += gridDim.x * kT) {
+        const double re = r[edge[i]];
+        v[0] = fma(re * Dinv[edge[i]], re, v[0]);
+    }
     block_partial<1>(v, part);
 }
 
 __device__ __forceinline__ double rho_of(const double *nrm, int n) { return sqrt(nrm[0] / n); }
+// (by one thread of the block: division and root in every warp of it hold the
+// FP64 pipes for longer than a small kernel's own work)
+__device__ __forceinline__ double block_rho(const double *nrm, int n) {
+    __shared__ double rho;
+    if (threadIdx.x == 0) rho = rho_of(nrm, n);
+    __syncthreads();
+    return rho;
+}
 
 // ---- forward ----
+// The warp's 32 rows are scaled a lane each and the features formed row by row:
+// a lane per feature that scales its row itself repeats the row's FP64
+// division 32 times (136 -> 15 us at 220,256 rows).  nrm_part: the partials
+// of n rho^2; block 0 leaves their sum in nrm.
 template <bool KEEP>
-__global__ void __launch_bounds__(kT) k_embed(int n, const double *__restrict__ r, const double *__restrict__ isd,
-                                             const double *__restrict__ nrm, const float *__restrict__ feat_a,
+__global__ void __launch_bounds__(kT) k_embed(int n, const int *__restrict__ edge, const double *__restrict__ r,
+                                             const double *__restrict__ isd,
+                                             const double *__restrict__ nrm_part, double *__restrict__ nrm,
+                                             const float *__restrict__ feat_a,
                                              const unsigned short *__restrict__ th, float *__restrict__ xin,
                                              float *__restrict__ pre0, float *__restrict__ h0) {
+    __shared__ double s_rho;
     const int lane = threadIdx.x & 31;
-    const double rho = rho_of(nrm, n);
+    const double total = block_total(kGB, nrm_part);
+    if (threadIdx.x == 0) {
+        s_rho = sqrt(total / n);
+        if (blockIdx.x == 0) nrm[0] = total;
+    }
+    __syncthreads();
+    const double rho = s_rho;
     const float U = bf(th, kOffU + lane), V = bf(th, kOffV + lane), c = bf(th, kOffC + lane);
-    for (int i = blockIdx.x * kW + (threadIdx.x >> 5); i < n; i += gridDim.x * kW) {
-        const float x = rho > 0.0 ? (float)(r[i] * isd[i] / rho) : 0.0f;
-        const float p = fmaf(U, x, fmaf(V, feat_a[i], c));
-        if (KEEP) {
-            if (lane == 0) xin[i] = x;
-            pre0[(size_t)i * kH + lane] = p;
+    for (int base = (blockIdx.x * kW + (threadIdx.x >> 5)) * 32; base < n; base += gridDim.x * kT) {
+        const int i = base + lane, m = min(32, n - base);
+        float x = 0.0f, fa = 0.0f;
+        if (lane < m) {
+            x = rho > 0.0 ? (float)(r[edge[i]] * isd[i] / rho) : 0.0f;
+            fa = feat_a[i];
+            if (KEEP) xin[i] = x;
         }
-        h0[(size_t)i * kH + lane] = fmaxf(p, 0.0f);
+#pragma unroll 4
+        for (int k = 0; k < m; k++) {
+            const float p = fmaf(U, __shfl_sync(0xFFFFFFFFu, x, k), fmaf(V, __shfl_sync(0xFFFFFFFFu, fa, k), c));
+            if (KEEP) pre0[(size_t)(base + k) * kH + lane] = p;
+            h0[(size_t)(base + k) * kH + lane] = fmaxf(p, 0.0f);
+        }
     }
 }
 
@@ -208,8 +276,8 @@ __global__ void __launch_bounds__(kT) k_layer(int n, const int *__restrict__ sp,
                                              const int *__restrict__ col, const float *__restrict__ ahat,
                                              const float *__restrict__ hp, const unsigned short *__restrict__ th,
                                              int off, float *__restrict__ g, float *__restrict__ pre,
-                                             float *__restrict__ h, const double *__restrict__ r,
-                                             const double *__restrict__ Dinv, const double *__restrict__ isd,
+                                             float *__restrict__ h, const int *__restrict__ edge,
+                                             const double *__restrict__ r, const double *__restrict__ Dinv, const double *__restrict__ isd,
                                              const double *__restrict__ nrm, double *__restrict__ z) {
     __shared__ float Wt[kH * kH], Qt[kH * kH], bsh[kH], osh[kH];
     for (int t = threadIdx.x; t < kH * kH; t += kT) {
@@ -224,7 +292,7 @@ __global__ void __launch_bounds__(kT) k_layer(int n, const int *__restrict__ sp,
     __syncthreads();
     const int lane = threadIdx.x & 31;
     const float d0 = LAST ? bf(th, kOffD0) : 0.0f;
-    const double rho = LAST ? rho_of(nrm, n) : 0.0;
+    const double rho = LAST ? block_rho(nrm, n) : 0.0;
     for (int i = blockIdx.x * kW + (threadIdx.x >> 5); i < n; i += gridDim.x * kW) {
         const float hi = hp[(size_t)i * kH + lane];
         const float gi = aggregate(i, sp, sw, col, ahat, hp, 0.0f);
@@ -242,7 +310,10 @@ __global__ void __launch_bounds__(kT) k_layer(int n, const int *__restrict__ sp,
             float y = osh[lane] * hn;
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) y += __shfl_down_sync(0xFFFFFFFFu, y, o);
-            if (lane == 0) z[i] = fma(r[i], Dinv[i], rho * (double)(y + d0) * isd[i]);
+            if (lane == 0) {
+                const int e = edge[i];
+                z[e] = fma(r[e], Dinv[e], rho * (double)(y + d0) * isd[i]);
+            }
         }
     }
 }
@@ -300,11 +371,13 @@ __global__ void __launch_bounds__(kT, kTcBlocksPerSm) k_layer_tc(int n, const in
                                                                  const float *__restrict__ ahat,
                                                                  const float *__restrict__ hp,
                                                                  const unsigned short *__restrict__ th, int off,
-                                                                 float *__restrict__ h, const double *__restrict__ r,
+                                                                 float *__restrict__ h, const int *__restrict__ edge, const double *__restrict__ r,
                                                                  const double *__restrict__ Dinv,
                                                                  const double *__restrict__ isd,
                                                                  const double *__restrict__ nrm,
-                                                                 double *__restrict__ z) {
+                                                                 double *__restrict__ z,
+                                                                 const double *__restrict__ zo,
+                                                                 double *__restrict__ part) {
     // B fragments of [W Q]^T for k-step ks and column tile nt at Bf[(ks * 4 + nt) * 32 + lane]
     __shared__ __align__(16) float2 Bf[8 * 4 * 32];
     __shared__ __align__(16) float S[kW][kTileRows * kSRow];
@@ -327,7 +400,8 @@ __global__ void __launch_bounds__(kT, kTcBlocksPerSm) k_layer_tc(int n, const in
     const int g = lane >> 2, t4 = lane & 3;
     float *Sw = S[warp];
     const float d0 = LAST ? bf(th, kOffD0) : 0.0f;
-    const double rho = LAST ? rho_of(nrm, n) : 0.0;
+    const double rho = LAST ? block_rho(nrm, n) : 0.0;
+    double dots[2] = {0.0, 0.0};   // (r, z), (r, z_old)
     const int ntiles = (n + kTileRows - 1) / kTileRows;
     for (int tile = blockIdx.x * kW + warp; tile < ntiles; tile += gridDim.x * kW) {
         const int sl = tile >> 1, row0 = tile * kTileRows;
@@ -421,11 +495,24 @@ __global__ void __launch_bounds__(kT, kTcBlocksPerSm) k_layer_tc(int n, const in
                 y1 += __shfl_xor_sync(0xFFFFFFFFu, y1, o);
             }
             if (t4 == 0) {
-                if (i0 < n) z[i0] = fma(r[i0], Dinv[i0], rho * (double)(y0 + d0) * isd[i0]);
-                if (i1 < n) z[i1] = fma(r[i1], Dinv[i1], rho * (double)(y1 + d0) * isd[i1]);
+                const int ii[2] = {i0, i1};
+                const float yy[2] = {y0, y1};
+#pragma unroll
+                for (int q = 0; q < 2; q++) {
+                    const int i = ii[q];
+                    if (i >= n) continue;
+                    const int e = edge[i];
+                    const double ri = r[e], zi = fma(ri, Dinv[e], rho * (double)(yy[q] + d0) * isd[i]);
+                    z[e] = zi;
+                    if (zo) {
+                        dots[0] = fma(ri, zi, dots[0]);
+                        dots[1] = fma(ri, zo[e], dots[1]);
+                    }
+                }
             }
         }
     }
+    if (LAST && zo) block_partial<2>(dots, part);
 }
 
 // ---- backward ----
@@ -433,10 +520,10 @@ __global__ void __launch_bounds__(kT, kTcBlocksPerSm) k_layer_tc(int n, const in
 __global__ void __launch_bounds__(kT) k_gy(int n, int nsl, const int *__restrict__ sp, const int *__restrict__ sw,
                                           const int *__restrict__ col, const double *__restrict__ val,
                                           const double *__restrict__ z, const double *__restrict__ r,
-                                          const double *__restrict__ isd, const double *__restrict__ nrm,
-                                          double *__restrict__ gy, double *part) {
+                                          const int *__restrict__ row, const double *__restrict__ isd,
+                                          const double *__restrict__ nrm, double *__restrict__ gy, double *part) {
     const int lane = threadIdx.x & 31;
-    const double N = nrm[0], rho = rho_of(nrm, n);
+    const double N = nrm[0], rho = block_rho(nrm, n);
     double v[1] = {0.0};
     for (int sl = blockIdx.x * kW + (threadIdx.x >> 5); sl < nsl; sl += gridDim.x * kW) {
         const int kb = sp[sl] + lane, kw = sw[sl];
@@ -444,7 +531,8 @@ __global__ void __launch_bounds__(kT) k_gy(int n, int nsl, const int *__restrict
         for (int j = 0; j < kw; j++) s = fma(val[kb + 32 * j], z[col[kb + 32 * j]], s);
         const int i = sl * 32 + lane;
         if (i < n) {
-            gy[i] = N > 0.0 ? 2.0 * (s - r[i]) * rho * isd[i] / N : 0.0;
+            const int g = row[i];
+            gy[g] = N > 0.0 ? 2.0 * (s - r[i]) * rho * isd[g] / N : 0.0;
             v[0] += z[i] * s - 2.0 * z[i] * r[i];
         }
     }
@@ -573,14 +661,60 @@ __global__ void k_to_bf16(int np, const float *__restrict__ theta, unsigned shor
 }
 
 // ---- flexible PCG vector steps ----
-// x += alpha p, r -= alpha q with alpha = s[0] / s[1]
-__global__ void k_fpcg_xr(int n, const double *__restrict__ sc, const double *__restrict__ p,
-                          const double *__restrict__ q, double *__restrict__ x, double *__restrict__ r) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const double alpha = sc[0] / sc[1];
-    x[i] = fma(alpha, p[i], x[i]);
-    r[i] = fma(-alpha, q[i], r[i]);
+// q = A p, and (p, q)
+__global__ void __launch_bounds__(kT) k_spmv_dot(int n, int nsl, const int *__restrict__ sp, const int *__restrict__ sw,
+                                                const int *__restrict__ col, const double *__restrict__ val,
+                                                const double *__restrict__ p, double *__restrict__ q, double *part) {
+    const int lane = threadIdx.x & 31;
+    double v[1] = {0.0};
+    for (int sl = blockIdx.x * kW + (threadIdx.x >> 5); sl < nsl; sl += gridDim.x * kW) {
+        const int kb = sp[sl] + lane, kw = sw[sl];
+        double s = 0.0;
+#pragma unroll 8
+        for (int j = 0; j < kw; j++) s = fma(val[kb + 32 * j], p[col[kb + 32 * j]], s);
+        const int i = sl * 32 + lane;
+        if (i < n) {
+            q[i] = s;
+            v[0] = fma(p[i], s, v[0]);
+        }
+    }
+    block_partial<1>(v, part);
+}
+
+// x += alpha p, r -= alpha q with alpha = rz / (p, q), the latter from its
+// partials; then (r, r) and (r, D^-1 r)
+__global__ void __launch_bounds__(kT) k_fpcg_xr(int n, double rz, const double *__restrict__ pq_part,
+                                               const double *__restrict__ p, const double *__restrict__ q,
+                                               const double *__restrict__ Dinv, double *__restrict__ x,
+                                               double *__restrict__ r, double *part) {
+    __shared__ double s_alpha;
+    const double pq = block_total(kGB, pq_part);
+    if (threadIdx.x == 0) s_alpha = rz / pq;
+    __syncthreads();
+    const double alpha = s_alpha;
+    double v[2] = {0.0, 0.0};
+    for (int i = blockIdx.x * kT + threadIdx.x; i < n; i += gridDim.x * kT) {
+        x[i] = fma(alpha, p[i], x[i]);
+        const double ri = fma(-alpha, q[i], r[i]);
+        r[i] = ri;
+        v[0] = fma(ri, ri, v[0]);
+        v[1] = fma(ri * Dinv[i], ri, v[1]);
+    }
+    block_partial<2>(v, part);
+}
+
+// out[0] = (r, r) from na partials, out[1], out[2] = (r, z), (r, z_old) from nb
+// partials each: a warp a value
+__global__ void k_fpcg_sums(int na, const double *__restrict__ a, int nb, const double *__restrict__ b,
+                            double *__restrict__ out) {
+    const int lane = threadIdx.x & 31, c = threadIdx.x >> 5;
+    const double *v = c == 0 ? a : b + (size_t)(c - 1) * nb;
+    const int m = c == 0 ? na : nb;
+    double s = 0.0;
+    for (int k = lane; k < m; k += 32) s += v[k];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xFFFFFFFFu, s, o);
+    if (lane == 0) out[c] = s;
 }
 
 // p = z + beta p, beta = beta_num / rz_old
@@ -644,19 +778,61 @@ static int gnn_reduce_launch(Sim *s, int nv, double *out) {
     return PIC_OK;
 }
 
+// The network's row order and its SELL-32 pattern, packed: padding names the
+// row itself
+static int gnn_rows(Sim *s) {
+    GnnState &G = s->gnn;
+    const Mesh *m = s->mesh;
+    const int n = m->n_int_edges, nsl = (n + 31) / 32;
+    // rows by (length, canonical edge): counted, then placed in canonical order
+    int most = 0;
+    for (int e = 0; e < n; e++) most = std::max(most, m->h_row_len[e]);
+    std::vector<int> at(most + 2, 0), edge_of(n), row_of(n), canon(n);
+    for (int e = 0; e < n; e++) at[m->h_row_len[e] + 1]++;
+    for (int l = 0; l <= most; l++) at[l + 1] += at[l];
+    for (int c = 0; c < m->n_edges; c++) {
+        const int e = m->h_edge_internal[c];
+        if (e >= n) continue;
+        const int i = at[m->h_row_len[e]]++;
+        edge_of[i] = e;
+        row_of[e] = i;
+        canon[i] = c;
+    }
+    std::vector<int> ptr(nsl + 1, 0), width(nsl, 0);
+    for (int sl = 0; sl < nsl; sl++) {
+        width[sl] = m->h_row_len[edge_of[std::min(n, 32 * sl + 32) - 1]];
+        ptr[sl + 1] = ptr[sl] + 32 * width[sl];
+    }
+    G.rows.n_rows = n;
+    G.rows.n_slices = nsl;
+    G.rows.n_elems = ptr[nsl];
+    DevBuf<int> canon_dev;
+    int rc;
+    if ((rc = G.rows.ptr.upload(ptr)) || (rc = G.rows.width.upload(width)) || (rc = G.rows.col.alloc(ptr[nsl])) ||
+        (rc = G.edge_of.upload(edge_of)) || (rc = G.row_of.upload(row_of)) || (rc = canon_dev.upload(canon)))
+        return rc;
+    if (n > 0) {
+        { k_rows_cols<<<(32 * nsl + 255) / 256, 256, 0, s->stream>>>(n, nsl, G.rows.ptr.p, G.rows.width.p, canon_dev.p, m->e2t.rowptr.p, m->e2t.col.p, m->tet_edge.p, G.row_of.p, G.rows.col.p); note_launch(); }
+        FP_CUDA(cudaGetLastError());
+        FP_CUDA(cudaStreamSynchronize(s->stream));
+    }
+    return PIC_OK;
+}
+
 int gnn_prepare(Sim *s) {
     GnnState &G = s->gnn;
     if (G.ready) return PIC_OK;
     const Mesh *m = s->mesh;
     const int n = m->n_int_edges;
     const size_t nn = (size_t)std::max(n, 1), nh = nn * kH;
-    const long long nel = std::max(m->As.n_elems, 1LL);
     int rc;
+    if ((rc = gnn_rows(s))) return rc;
+    const long long nel = std::max(G.rows.n_elems, 1LL);
     if ((rc = G.theta.alloc(kGnnParams)) || (rc = G.theta_bf.alloc(kGnnParams)) || (rc = G.adam_m.alloc(kGnnParams)) ||
         (rc = G.adam_v.alloc(kGnnParams)) || (rc = G.grad.alloc(kGnnParams)) || (rc = G.ahat.alloc(nel)) ||
         (rc = G.isd.alloc(nn)) || (rc = G.logd.alloc(nn)) || (rc = G.feat_a.alloc(nn)) || (rc = G.xin.alloc(nn)) ||
         (rc = G.gy.alloc(nn)) || (rc = G.dh.alloc(nh)) || (rc = G.dh2.alloc(nh)) || (rc = G.tq.alloc(nh)) ||
-        (rc = G.part.alloc(8 * (size_t)kGB)) || (rc = G.sc.alloc(16)) ||
+        (rc = G.part.alloc(std::max<size_t>(8 * (size_t)kGB, 3 * (size_t)kGB + 2 * (size_t)tc_grid(n)))) || (rc = G.sc.alloc(16)) ||
         (rc = G.wpart.alloc((size_t)kGB * kNA * 32)) || (rc = G.dst.alloc(4 * kNA * 32)))
         return rc;
     for (int l = 0; l < 4; l++)
@@ -691,11 +867,11 @@ int gnn_prepare(Sim *s) {
     }
     FP_CUDA(cudaMemcpyAsync(G.dst.p, dst.data(), sizeof(int) * dst.size(), cudaMemcpyHostToDevice, s->stream));
     if (n > 0) {
-        { k_prep_rows<<<(n + 255) / 256, 256, 0, s->stream>>>(n, s->Dinv.p, G.isd.p, G.logd.p); note_launch(); }
+        { k_prep_rows<<<(n + 255) / 256, 256, 0, s->stream>>>(n, G.edge_of.p, s->Dinv.p, G.isd.p, G.logd.p); note_launch(); }
         { k_sum<<<kGB, kT, 0, s->stream>>>(n, G.logd.p, G.part.p); note_launch(); }
         if ((rc = gnn_reduce_launch(s, 1, G.sc.p + 8))) return rc;
-        const int nsl = m->As.n_slices;
-        { k_prep_ahat<<<(nsl * 32 + 255) / 256, 256, 0, s->stream>>>(n, nsl, m->As.ptr.p, m->As.width.p, m->As.col.p, s->A_val.p, G.isd.p, G.logd.p, G.sc.p + 8, G.ahat.p, G.feat_a.p); note_launch(); }
+        const int nsl = G.rows.n_slices;
+        { k_prep_ahat<<<(nsl * 32 + 255) / 256, 256, 0, s->stream>>>(n, nsl, G.rows.ptr.p, G.rows.width.p, G.rows.col.p, G.edge_of.p, m->As.ptr.p, m->As.width.p, m->As.col.p, s->A_val.p, G.isd.p, G.logd.p, G.sc.p + 8, G.ahat.p, G.feat_a.p); note_launch(); }
     }
     FP_CUDA(cudaGetLastError());
     G.ready = 1;
@@ -736,32 +912,39 @@ int gnn_get_weights(Sim *s, float *w, long long np) {
 }
 
 // z = P(r) on interior edges (internal order, device arrays); with `keep`
-// the activations a backward pass needs are stored.  G.sc[0] receives n rho^2.
-int gnn_forward(Sim *s, const double *r, double *z, bool keep) {
+// the activations a backward pass needs are stored.  G.sc[0] receives n rho^2,
+// from the kGB partials at nrm_part (NULL: formed here).  With zo, the partials
+// of (r, z) and (r, zo) go to dot_part, tc_grid(n) each.
+static int gnn_forward_dots(Sim *s, const double *r, double *z, bool keep, const double *nrm_part, const double *zo,
+                            double *dot_part) {
     GnnState &G = s->gnn;
-    const Mesh *m = s->mesh;
-    const int n = m->n_int_edges;
+    const int n = s->mesh->n_int_edges;
     if (n == 0) return PIC_OK;
-    const DevSell &A = m->As;
+    const DevSell &A = G.rows;
     cudaStream_t st = s->stream;
-    int rc;
-    { k_rnorm<<<kGB, kT, 0, st>>>(n, r, s->Dinv.p, G.part.p); note_launch(); }
-    if ((rc = gnn_reduce_launch(s, 1, G.sc.p))) return rc;
-    if (keep) { k_embed<true><<<kGB, kT, 0, st>>>(n, r, G.isd.p, G.sc.p, G.feat_a.p, G.theta_bf.p, G.xin.p, G.pre[0].p, G.h[0].p); note_launch(); }
-    else { k_embed<false><<<kGB, kT, 0, st>>>(n, r, G.isd.p, G.sc.p, G.feat_a.p, G.theta_bf.p, G.xin.p, G.pre[0].p, G.h[0].p); note_launch(); }
+    if (!nrm_part) {
+        { k_rnorm<<<kGB, kT, 0, st>>>(n, G.edge_of.p, r, s->Dinv.p, G.part.p); note_launch(); }
+        nrm_part = G.part.p;
+    }
+    if (keep) { k_embed<true><<<kGB, kT, 0, st>>>(n, G.edge_of.p, r, G.isd.p, nrm_part, G.sc.p, G.feat_a.p, G.theta_bf.p, G.xin.p, G.pre[0].p, G.h[0].p); note_launch(); }
+    else { k_embed<false><<<kGB, kT, 0, st>>>(n, G.edge_of.p, r, G.isd.p, nrm_part, G.sc.p, G.feat_a.p, G.theta_bf.p, G.xin.p, G.pre[0].p, G.h[0].p); note_launch(); }
     const int gr = rows_grid(n), gt = tc_grid(n);
     for (int l = 1; l <= 3; l++) {
         const int off = kOffL + (l - 1) * kLayer;
         // without keep, layers 1 and 2 ping-pong between h[0] and h[1]
         const float *hin = keep ? G.h[l - 1].p : G.h[(l - 1) & 1].p;
         float *hout = keep ? G.h[l].p : G.h[l & 1].p;
-        if (l < 3 && keep) { k_layer<false><<<gr, kT, 0, st>>>(n, A.ptr.p, A.width.p, A.col.p, G.ahat.p, hin, G.theta_bf.p, off, G.g[l].p, G.pre[l].p, hout, r, s->Dinv.p, G.isd.p, G.sc.p, z); note_launch(); }
-        else if (l < 3) { k_layer_tc<false><<<gt, kT, 0, st>>>(n, A.ptr.p, A.width.p, A.col.p, G.ahat.p, hin, G.theta_bf.p, off, hout, r, s->Dinv.p, G.isd.p, G.sc.p, z); note_launch(); }
-        else if (keep) { k_layer<true><<<gr, kT, 0, st>>>(n, A.ptr.p, A.width.p, A.col.p, G.ahat.p, hin, G.theta_bf.p, off, G.g[l].p, G.pre[l].p, hout, r, s->Dinv.p, G.isd.p, G.sc.p, z); note_launch(); }
-        else { k_layer_tc<true><<<gt, kT, 0, st>>>(n, A.ptr.p, A.width.p, A.col.p, G.ahat.p, hin, G.theta_bf.p, off, hout, r, s->Dinv.p, G.isd.p, G.sc.p, z); note_launch(); }
+        if (l < 3 && keep) { k_layer<false><<<gr, kT, 0, st>>>(n, A.ptr.p, A.width.p, A.col.p, G.ahat.p, hin, G.theta_bf.p, off, G.g[l].p, G.pre[l].p, hout, G.edge_of.p, r, s->Dinv.p, G.isd.p, G.sc.p, z); note_launch(); }
+        else if (l < 3) { k_layer_tc<false><<<gt, kT, 0, st>>>(n, A.ptr.p, A.width.p, A.col.p, G.ahat.p, hin, G.theta_bf.p, off, hout, G.edge_of.p, r, s->Dinv.p, G.isd.p, G.sc.p, z, nullptr, nullptr); note_launch(); }
+        else if (keep) { k_layer<true><<<gr, kT, 0, st>>>(n, A.ptr.p, A.width.p, A.col.p, G.ahat.p, hin, G.theta_bf.p, off, G.g[l].p, G.pre[l].p, hout, G.edge_of.p, r, s->Dinv.p, G.isd.p, G.sc.p, z); note_launch(); }
+        else { k_layer_tc<true><<<gt, kT, 0, st>>>(n, A.ptr.p, A.width.p, A.col.p, G.ahat.p, hin, G.theta_bf.p, off, hout, G.edge_of.p, r, s->Dinv.p, G.isd.p, G.sc.p, z, zo, dot_part); note_launch(); }
     }
     FP_CUDA(cudaGetLastError());
     return PIC_OK;
+}
+
+int gnn_forward(Sim *s, const double *r, double *z, bool keep) {
+    return gnn_forward_dots(s, r, z, keep, nullptr, nullptr, nullptr);
 }
 
 // loss and dL/dtheta (into G.grad, device) for residual r; loss -> G.sc[1]
@@ -777,7 +960,7 @@ int gnn_backward(Sim *s, const double *r, const double *z) {
         FP_CUDA(cudaMemsetAsync(G.sc.p + 1, 0, sizeof(double), st));
         return PIC_OK;
     }
-    { k_gy<<<kGB, kT, 0, st>>>(n, A.n_slices, A.ptr.p, A.width.p, A.col.p, s->A_val.p, z, r, G.isd.p, G.sc.p, G.gy.p, G.part.p); note_launch(); }
+    { k_gy<<<kGB, kT, 0, st>>>(n, A.n_slices, A.ptr.p, A.width.p, A.col.p, s->A_val.p, z, r, G.row_of.p, G.isd.p, G.sc.p, G.gy.p, G.part.p); note_launch(); }
     if ((rc = gnn_reduce_launch(s, 1, G.sc.p + 1))) return rc;
     constexpr int NA = kNA;
     // dh of layer l lives in cur; the layer writes W^T dpre into nxt and Q^T dpre into tq
@@ -787,7 +970,7 @@ int gnn_backward(Sim *s, const double *r, const double *z) {
         if (l == 3) { k_layer_bwd<true><<<kGB, kT, 0, st>>>(n, G.h[2].p, G.g[3].p, G.pre[3].p, G.h[3].p, nullptr, G.gy.p, G.theta_bf.p, off, nxt, G.tq.p, G.wpart.p); note_launch(); }
         else { k_layer_bwd<false><<<kGB, kT, 0, st>>>(n, G.h[l - 1].p, G.g[l].p, G.pre[l].p, G.h[l].p, cur, G.gy.p, G.theta_bf.p, off, nxt, G.tq.p, G.wpart.p); note_launch(); }
         { k_grad_final<<<(NA * 32 + 255) / 256, 256, 0, st>>>(kGB, NA, G.wpart.p, G.dst.p + (l - 1) * NA * 32, G.grad.p); note_launch(); }
-        { k_agg_bwd<<<rows_grid(n), kT, 0, st>>>(n, A.ptr.p, A.width.p, A.col.p, G.ahat.p, G.tq.p, nxt); note_launch(); }
+        { k_agg_bwd<<<rows_grid(n), kT, 0, st>>>(n, G.rows.ptr.p, G.rows.width.p, G.rows.col.p, G.ahat.p, G.tq.p, nxt); note_launch(); }
         std::swap(cur, nxt);
     }
     { k_embed_bwd<<<kGB, kT, 0, st>>>(n, G.xin.p, G.feat_a.p, G.pre[0].p, cur, G.wpart.p); note_launch(); }
@@ -904,16 +1087,26 @@ int fpcg_newmark(Sim *s, int *iters_out) {
             set_error("flexible PCG did not reach the tolerance");
             return PIC_ERR_CG_NO_CONVERGENCE;
         }
-        // x += alpha p, r -= alpha A p, alpha = r.z / p.A p
-        { k_spmv<<<kGB, kT, 0, st>>>(n, A.n_slices, A.ptr.p, A.width.p, A.col.p, s->A_val.p, p, q); note_launch(); }
-        { k_dot2<<<kGB, kT, 0, st>>>(n, p, q, nullptr, nullptr, nullptr, G.part.p); note_launch(); }
-        if ((rc = gnn_reduce_launch(s, 1, G.sc.p + 1))) return rc;
-        FP_CUDA(cudaMemcpyAsync(G.sc.p, &rzo, sizeof(double), cudaMemcpyHostToDevice, st));
-        { k_fpcg_xr<<<ge, 256, 0, st>>>(n, G.sc.p, p, q, x, r); note_launch(); }
+        // x += alpha p, r -= alpha A p, alpha = r.z / p.A p: partial sums go
+        // from kernel to kernel, and the host waits once an iteration
+        double *pq_part = G.part.p, *rr_part = G.part.p + kGB, *dot_part = G.part.p + 3 * kGB;
+        { k_spmv_dot<<<kGB, kT, 0, st>>>(n, A.n_slices, A.ptr.p, A.width.p, A.col.p, s->A_val.p, p, q, pq_part); note_launch(); }
+        { k_fpcg_xr<<<kGB, kT, 0, st>>>(n, rzo, pq_part, p, q, s->Dinv.p, x, r, rr_part); note_launch(); }
         std::swap(z, zo);
-        if ((rc = precond(r, z, jac))) return rc;
         double d1[2], d2[2];
-        if ((rc = dots(r, z, r, zo, d1)) || (rc = dots(r, r, nullptr, nullptr, d2))) return rc;
+        if (jac) {
+            if ((rc = precond(r, z, jac)) || (rc = dots(r, z, r, zo, d1)) || (rc = dots(r, r, nullptr, nullptr, d2))) return rc;
+        } else {
+            if ((rc = gnn_forward_dots(s, r, z, false, rr_part + kGB, zo, dot_part))) return rc;
+            { k_fpcg_sums<<<1, 96, 0, st>>>(kGB, rr_part, tc_grid(n), dot_part, G.sc.p + 4); note_launch(); }
+            FP_CUDA(cudaGetLastError());
+            double v[3];
+            FP_CUDA(cudaMemcpyAsync(v, G.sc.p + 4, sizeof(v), cudaMemcpyDeviceToHost, st));
+            FP_CUDA(cudaStreamSynchronize(st));
+            d2[0] = v[0];
+            d1[0] = v[1];
+            d1[1] = v[2];
+        }
         it++;
         rr = d2[0];
         bool restart = false;

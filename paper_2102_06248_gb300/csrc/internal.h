@@ -149,6 +149,7 @@ struct Mesh {
     std::vector<signed char> h_tet_sign;  // sign of det of the sorted tet
     std::vector<int> h_edge_internal;     // canonical -> internal edge id
     std::vector<int> h_edge_canonical;    // internal -> canonical
+    std::vector<int> h_row_len;           // entries of an interior edge's row of the Newmark matrix
     std::vector<double> h_xyz;
     std::vector<double> h_vol;
     std::vector<unsigned char> h_node_bnd;

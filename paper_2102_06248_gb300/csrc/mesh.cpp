@@ -476,6 +476,8 @@ int build_mesh(const pic_mesh_desc *d, Mesh *m) {
     HostCsr pa = pattern_from_groups(nie, nt, 6, nie, nie, [&](int t, int *out) {
         for (int k = 0; k < 6; k++) out[k] = tet_edge[6 * (size_t)t + k];
     });
+    m->h_row_len.resize(nie);
+    for (int e = 0; e < nie; e++) m->h_row_len[e] = pa.rowptr[e + 1] - pa.rowptr[e];
     std::vector<double> Mv(pa.col.size(), 0.0), Kv(pa.col.size(), 0.0);
     // [*mu^-1] on all faces
     HostCsr ph = pattern_from_groups(nf, nt, 4, nf, nf, [&](int t, int *out) {

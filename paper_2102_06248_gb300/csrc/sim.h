@@ -107,7 +107,12 @@ struct GnnState {
     DevBuf<float> theta, adam_m, adam_v;    // FP32 master weights and Adam moments
     DevBuf<unsigned short> theta_bf;        // bfloat16 copies used by the kernels
     DevBuf<double> grad;                    // dL/dtheta
-    DevBuf<float> ahat, feat_a, xin;        // D^-1/2 A D^-1/2 (SELL layout), log d - mean, x
+    // the network's rows: interior edges by the length of their row of A, in
+    // canonical order within one (its FP32 sums run in this order whatever the
+    // order of the edges elsewhere)
+    DevSell rows;
+    DevBuf<int> edge_of, row_of;            // edge of a row, row of an interior edge
+    DevBuf<float> ahat, feat_a, xin;        // D^-1/2 A D^-1/2 (layout of rows), log d - mean, x
     DevBuf<double> isd, logd, gy;
     DevBuf<float> h[4], pre[4], g[4];       // activations, 32 per row
     DevBuf<float> dh, dh2, tq;              // backward buffers, 32 per row
