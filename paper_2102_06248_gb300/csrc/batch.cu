@@ -89,14 +89,6 @@ int join_all(pic_batch *b) {
     return PIC_OK;
 }
 
-// a multigrid completion reads z_old in its first iteration: zero it
-int zero_mg_history(Sim *s) {
-    const Mesh *m = s->mesh;
-    if (m->mg_levels > 0 && m->n_int_nodes > 0 && m->n_int_edges > 0)
-        FP_CUDA(cudaMemsetAsync(s->l_p1.p, 0, sizeof(double) * m->n_int_nodes, s->stream));
-    return PIC_OK;
-}
-
 // (re)builds the completion table for the current completion blocks/SM
 int completion_table(pic_batch *b) {
     if (!b->use_mg || b->ct_bps == b->gc_blocks_per_sm) return PIC_OK;
@@ -123,10 +115,8 @@ int batch_step_once(pic_batch *b) {
         if (ps->s.mesh->n_int_edges > 0) runs.push_back(pcg_args_newmark(&ps->s));
     if ((rc = launch_pcg_runs(runs.data(), (int)runs.size(), b->blocks_per_sm, b->ms, b->build))) return rc;
     if ((rc = fork_all(b))) return rc;
-    for (auto *ps : b->sims) {
+    for (auto *ps : b->sims)
         if ((rc = gc_prepare(&ps->s))) return rc;
-        if (b->use_mg && (rc = zero_mg_history(&ps->s))) return rc;
-    }
     if ((rc = join_all(b))) return rc;
     if (b->use_mg) {
         if ((rc = launch_completion_table(b->ctable, b->ct_runs, b->ct_blocks, b->ms))) return rc;
@@ -195,12 +185,6 @@ int autotune(pic_batch *b) {
                 if (mg_launch) {
                     b->gc_blocks_per_sm = kTuneBps[c];
                     if ((rc = completion_table(b))) break;
-                    for (auto *ps : b->sims) {
-                        const Mesh *m = ps->s.mesh;
-                        if (m->mg_levels > 0 && m->n_int_nodes > 0 && m->n_int_edges > 0 &&
-                            cudaMemsetAsync(ps->s.l_p1.p, 0, sizeof(double) * m->n_int_nodes, b->ms) != cudaSuccess)
-                            rc = PIC_ERR_CUDA;
-                    }
                     if (!rc && cudaEventRecord(e0, b->ms) != cudaSuccess) rc = PIC_ERR_CUDA;
                     if (!rc) rc = launch_completion_table(b->ctable, b->ct_runs, b->ct_blocks, b->ms);
                     if (!rc && cudaEventRecord(e1, b->ms) != cudaSuccess) rc = PIC_ERR_CUDA;

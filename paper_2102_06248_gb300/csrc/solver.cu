@@ -800,7 +800,6 @@ extern __shared__ __align__(128) unsigned char s_ring[];   // dynamic shared mem
 // its iterations are bound by the latency and the FP64 rate of each SM).
 template <bool WIDE, int T, int RING>
 struct SolveCtx {
-    static constexpr int W = T / 32;
     template <typename V>
     using S = Stream<V, WIDE, RING, false>;
     using S64 = S<double>;
@@ -1431,12 +1430,21 @@ __device__ __forceinline__ void small_body(const PcgArgs &a, const int nb, const
 // scaled operators s0 L in FP32 with the residual divided by its maximum
 // (sigma), so z = sigma s0 V(r / sigma).  One persistent cooperative launch:
 // every phase that reads other rows' values starts after a grid barrier, and
-// the reductions combine in the last block to arrive (fixed order).  An
-// iteration has twelve such phases: the phases are bound by the latency of
-// dependent loads, so a sweep and the residual that follows it share a pass
-// where the neighbours' values can be formed on the fly, and q = L p comes as
-// L z + beta q right after the preconditioner.  Waits are bounded like those
-// of the Jacobi-PCG (timeout status, no hang).
+// the reductions have a fixed order (grid_reduce).  An iteration has twelve
+// such phases, bound by the latency of dependent loads, so
+//  * the row pointers of a block's level-0 slices and level-1 rows sit in
+//    shared memory, a row's indices and values are loaded together before
+//    its gathers, and what a phase gathers is one FP32 array: the update
+//    leaves the scaled residual and its first Jacobi sweep w0 r (scaled by the
+//    sigma of the iteration before; fac is the ratio to this one's), which the
+//    next V-cycle's first pass used to form from r in FP64 per entry;
+//  * L p is not formed: with w = L z and q = L p, (p', q') of p' = z + beta p
+//    is (z, w) + 2 beta (z, q) + beta^2 (p, q), so that one reduction after w
+//    gives beta and alpha, and p, q, x, r are updated in one pass.
+// 48^3 Poisson solve 2.02 -> 1.72 ms, 40^3 completion 0.78 -> 0.70 ms, 64^3 1.44 ->
+// 1.37 ms (there bound by its FP64 product and by streaming L: the hierarchy no
+// longer fits in L2 beside the vectors).  Waits are bounded
+// like those of the Jacobi-PCG (timeout status, no hang).
 // ---------------------------------------------------------------------------
 struct MgArgs {
     int n0, n1, n2, n_slices;
@@ -1484,33 +1492,41 @@ __device__ __forceinline__ float warp_sum_f(float v) {
     return v;
 }
 
-// Sum over one CSR row by a half warp (16 lanes; the two halves of a warp take
-// two rows at once), with every index and value of up to 64 entries loaded
-// before the first gather: the phases are bound by the latency of these
-// dependent loads, not by bandwidth.  val == nullptr means unit weights.
-__device__ __forceinline__ float half_row_dot(const int *__restrict__ ptr, const int *__restrict__ col,
-                                              const float *__restrict__ val, const float *__restrict__ x, int row,
-                                              bool ok, int hl) {
-    float s = 0.0f;
-    if (ok) {
-        const int kb = ptr[row], ke = ptr[row + 1];
-        for (int k0 = kb; k0 < ke; k0 += 64) {
-            int c[4];
-            float v[4];
+// Sums over two CSR rows (0 and 1) by a half warp, 16 lanes each row (the two
+// halves of a warp take four rows at once), with every index and value of up
+// to 48 entries of both loaded before the first gather: the phases are bound
+// by the latency of these dependent loads, not by bandwidth.  val == nullptr
+// means unit weights; get(c) is the gathered value of column c.
+template <typename Get>
+__device__ __forceinline__ float2 half_row_dots(int2 r0, int2 r1, const int *__restrict__ col,
+                                                const float *__restrict__ val, int hl, Get get) {
+    constexpr int kE = 3;
+    float s[2] = {0.0f, 0.0f};
+    while (r0.x < r0.y || r1.x < r1.y) {
+        int c[2][kE];
+        float v[2][kE];
 #pragma unroll
-            for (int u = 0; u < 4; u++) {
-                const int k = k0 + hl + 16 * u;
-                const bool in = k < ke;
-                c[u] = in ? col[k] : 0;
-                v[u] = in ? (val ? val[k] : 1.0f) : 0.0f;
-            }
-#pragma unroll
-            for (int u = 0; u < 4; u++) s = fmaf(v[u], x[c[u]], s);
+        for (int u = 0; u < kE; u++) {
+            const int k0 = r0.x + hl + 16 * u, k1 = r1.x + hl + 16 * u;
+            c[0][u] = k0 < r0.y ? col[k0] : -1;
+            c[1][u] = k1 < r1.y ? col[k1] : -1;
+            v[0][u] = k0 < r0.y ? (val ? val[k0] : 1.0f) : 0.0f;
+            v[1][u] = k1 < r1.y ? (val ? val[k1] : 1.0f) : 0.0f;
         }
+#pragma unroll
+        for (int h = 0; h < 2; h++)
+#pragma unroll
+            for (int u = 0; u < kE; u++)
+                if (c[h][u] >= 0) s[h] = fmaf(v[h][u], get(c[h][u]), s[h]);
+        r0.x += 16 * kE;
+        r1.x += 16 * kE;
     }
 #pragma unroll
-    for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
-    return s;
+    for (int o = 8; o > 0; o >>= 1) {
+        s[0] += __shfl_xor_sync(0xFFFFFFFFu, s[0], o);
+        s[1] += __shfl_xor_sync(0xFFFFFFFFu, s[1], o);
+    }
+    return make_float2(s[0], s[1]);
 }
 
 // the whole solve, run by block `bid` (T threads) of the nb blocks that own
@@ -1519,15 +1535,63 @@ template <int T>
 __device__ __forceinline__ void mg_body(const MgArgs &a, const int nb, const int bid, double *shv,
                                         unsigned long long *shm) {
     struct Scalars {
-        double thr, tol2, bb, rr, rz, rzo, alpha, beta, zs;
-        float inv;
+        double thr, tol2, bb, rr, rz, pq, alpha, beta, zs, inv;
+        float fac;
         int it, fresh, done, failed;
     };
     __shared__ Scalars sc;
-    const int G = nb * T, gt = bid * T + threadIdx.x;
-    const int lane = threadIdx.x & 31, nw = G >> 5, gw = gt >> 5;
+    // the run's threads, warps and half warps, numbered across the blocks first:
+    // what does not divide evenly (1.6 slices a warp, three coarse rows a half
+    // warp on the 64^3 mesh) then spreads over all SMs instead of loading the
+    // first blocks twice
+    const int G = nb * T, lane = threadIdx.x & 31;
+    const int nw = G >> 5, gw = (threadIdx.x >> 5) * nb + bid, gt = gw * 32 + lane;
     const long lim = a.spin_limit;
     unsigned int epoch = 0;
+    // row pointers: the k-th slice of warp w (k * W + w) and the k-th coarse
+    // row of half warp h (k * 2W + h), where the block has at most kPtrs of each
+    constexpr int W = T / 32, kPtrs = 4;
+    __shared__ int2 s_slice[kPtrs * W], s_l1[kPtrs * 2 * W], s_r0[kPtrs * 2 * W];
+    {
+        const int warp = threadIdx.x >> 5, half = threadIdx.x >> 4;
+        for (int k = lane; k < kPtrs; k += 32) {
+            const int sl = gw + k * nw;
+            if (sl < a.n_slices) s_slice[k * W + warp] = make_int2(a.sp[sl], a.sw[sl]);
+        }
+        for (int k = threadIdx.x & 15; k < kPtrs; k += 16) {
+            const int c = 2 * gw + (lane >> 4) + k * 2 * nw;
+            if (c < a.n1) {
+                s_l1[k * 2 * W + half] = make_int2(a.l1p[c], a.l1p[c + 1]);
+                s_r0[k * 2 * W + half] = make_int2(a.r0p[c], a.r0p[c + 1]);
+            }
+        }
+    }
+    auto slice = [&](int k, int sl) { return k < kPtrs ? s_slice[k * W + (threadIdx.x >> 5)] : make_int2(a.sp[sl], a.sw[sl]); };
+    auto coarse = [&](const int2 *sm, const int *ptr, int k, int c) {
+        return c >= a.n1 ? make_int2(0, 0) : k < kPtrs ? sm[k * 2 * W + (threadIdx.x >> 4)] : make_int2(ptr[c], ptr[c + 1]);
+    };
+    // sum over a SELL row (lane's row of the slice at h): eight entries' columns
+    // and values before their gathers
+    auto sell_row = [&](int2 h, const auto *__restrict__ val, const auto *x) {
+        using V = typename std::remove_cv<typename std::remove_reference<decltype(val[0])>::type>::type;
+        V s = 0;
+        const int kb = h.x + lane;
+        for (int j0 = 0; j0 < h.y; j0 += 8) {
+            int c[8];
+            V v[8];
+#pragma unroll
+            for (int u = 0; u < 8; u++) {
+                const bool in = j0 + u < h.y;
+                c[u] = in ? a.col[kb + 32 * (j0 + u)] : 0;
+                v[u] = in ? val[kb + 32 * (j0 + u)] : (V)0;
+            }
+#pragma unroll
+            for (int u = 0; u < 8; u++)
+                if (j0 + u < h.y) s = fma(v[u], x[c[u]], s);
+        }
+        return s;
+    };
+    __syncthreads();
     if (threadIdx.x == 0) {
         sc.thr = -1.0;
         sc.tol2 = a.fallback_tol2;
@@ -1538,7 +1602,7 @@ __device__ __forceinline__ void mg_body(const MgArgs &a, const int nb, const int
         sc.it = 0;
         sc.fresh = 1;
         sc.failed = 0;
-        sc.rzo = 0.0;
+        sc.inv = 1.0;
     }
     // after a residual: |r|^2 = t[0], max|r| = t[1]; sigma scales the next V-cycle
     auto residual = [&](const double *t, int wp, int l) {
@@ -1548,7 +1612,9 @@ __device__ __forceinline__ void mg_body(const MgArgs &a, const int nb, const int
         if (!done && sc.it >= a.max_iters) done = sc.failed = 1;
         sc.done = done;
         const double sigma = t[1] > 0.0 ? t[1] : 1.0;
-        sc.inv = (float)(1.0 / sigma);
+        const double inv = 1.0 / sigma;
+        sc.fac = (float)(inv / sc.inv);
+        sc.inv = inv;
         sc.zs = sigma * a.s0;
     };
     // x = 0, r = b; |b|^2 and max|r|
@@ -1578,11 +1644,9 @@ __device__ __forceinline__ void mg_body(const MgArgs &a, const int nb, const int
                 verify = false;
                 double v[1] = {0.0};
                 unsigned long long mx = 0;
-                for (int sl = gw; sl < a.n_slices; sl += nw) {
-                    const int row = sl * 32 + lane, kb = a.sp[sl] + lane, kw = a.sw[sl];
-                    double s = 0.0;
-#pragma unroll 4
-                    for (int j = 0; j < kw; j++) s = fma(a.Lv[kb + 32 * j], a.x[a.col[kb + 32 * j]], s);
+                for (int k = 0, sl = gw; sl < a.n_slices; k++, sl += nw) {
+                    const int row = sl * 32 + lane;
+                    const double s = sell_row(slice(k, sl), a.Lv, a.x);
                     if (row < a.n0) {
                         const double ri = a.b[row] - s;
                         a.r[row] = ri;
@@ -1599,64 +1663,77 @@ __device__ __forceinline__ void mg_body(const MgArgs &a, const int nb, const int
                 continue;
             }
             const bool first = sc.fresh != 0;
-            const float inv = sc.inv;
-            // V1: scaled residual r32, the first Jacobi sweep z0 = w0 r32 and
-            // t0 = r32 - L z0, with the neighbours' z0 formed from r on the fly
-            // (no barrier between the sweep and the residual)
-            for (int sl = gw; sl < a.n_slices; sl += nw) {
-                const int row = sl * 32 + lane, kb = a.sp[sl] + lane, kw = a.sw[sl];
-                float s = 0.0f;
-#pragma unroll 4
-                for (int j = 0; j < kw; j++) {
-                    const int cj = a.col[kb + 32 * j];
-                    s = fmaf(a.L32[kb + 32 * j], a.w0[cj] * ((float)a.r[cj] * inv), s);
+            float fac = sc.fac;
+            if (first) {
+                const double inv = sc.inv;
+                for (int i = gt; i < a.n0; i += G) {
+                    const float rs = (float)(a.r[i] * inv);
+                    a.r32[i] = rs;
+                    a.z0[i] = a.w0[i] * rs;
                 }
-                if (row < a.n0) {
-                    const float ri = (float)a.r[row] * inv;
-                    a.r32[row] = ri;
-                    a.z0[row] = a.w0[row] * ri;
-                    a.t0[row] = ri - s;
-                }
+                fac = 1.0f;
+                if (!grid_barrier(a.gb, ++epoch, nb, lim)) goto timeout;
+            }
+            // V1: t0 = r32 - L z0 with the first Jacobi sweep z0 = w0 r32
+            for (int k = 0, sl = gw; sl < a.n_slices; k++, sl += nw) {
+                const int row = sl * 32 + lane;
+                const float s = sell_row(slice(k, sl), a.L32, a.z0);
+                if (row < a.n0) a.t0[row] = fac * (a.r32[row] - s);
             }
             if (!grid_barrier(a.gb, ++epoch, nb, lim)) goto timeout;
-            // (coarse rows: half a warp per row, two rows per warp at a time)
-            const int hw = gt >> 4, nhw = G >> 4, hl = lane & 15;
+            // (coarse rows: half a warp takes two rows at once; the lanes 0 and 1
+            // of the half finish one each, their operands loaded beforehand)
+            const int hl = lane & 15, hw = 2 * gw + (lane >> 4), nhw = 2 * nw;
+            const bool ends = hl < 2;
             // V2: r1 = P0^T t0, the first Chebyshev step z1 = kCh1 w1 r1
-            for (int c0 = hw - (hw & 1); c0 < a.n1; c0 += nhw) {
-                const int c = c0 + (hw & 1);
-                const float sum = half_row_dot(a.r0p, a.r0c, a.r0v, a.t0, c, c < a.n1, hl);
-                if (hl == 0 && c < a.n1) {
-                    a.r1[c] = sum;
-                    a.z1[c] = kCh1 * a.w1[c] * sum;
+            for (int k = 0, c = hw; c - (hw & 1) < a.n1; k += 2, c += 2 * nhw) {
+                const int cm = c + hl * nhw;   // the row this lane finishes
+                const bool fin = ends && cm < a.n1;
+                const float wm = fin ? a.w1[cm] : 0.0f;
+                const float2 d = half_row_dots(coarse(s_r0, a.r0p, k, c), coarse(s_r0, a.r0p, k + 1, c + nhw), a.r0c,
+                                               a.r0v, hl, [&](int q) { return a.t0[q]; });
+                const float sum = hl ? d.y : d.x;
+                if (fin) {
+                    a.r1[cm] = sum;
+                    a.z1[cm] = kCh1 * wm * sum;
                 }
             }
             if (!grid_barrier(a.gb, ++epoch, nb, lim)) goto timeout;
             // V3: res = r1 - L1 z1 (into t1), the second step d1 = kCh2a z1 +
             // kCh2b w1 res, z1 + d1 (into z1b, since z1 is still read here)
-            for (int c0 = hw - (hw & 1); c0 < a.n1; c0 += nhw) {
-                const int c = c0 + (hw & 1);
-                const float sum = half_row_dot(a.l1p, a.l1c, a.l1v, a.z1, c, c < a.n1, hl);
-                if (hl == 0 && c < a.n1) {
-                    const float res = a.r1[c] - sum, zc = a.z1[c];
-                    const float d = kCh2a * zc + kCh2b * a.w1[c] * res;
-                    a.t1[c] = res;
-                    a.d1[c] = d;
-                    a.z1b[c] = zc + d;
+            for (int k = 0, c = hw; c - (hw & 1) < a.n1; k += 2, c += 2 * nhw) {
+                const int cm = c + hl * nhw;
+                const bool fin = ends && cm < a.n1;
+                const float wm = fin ? a.w1[cm] : 0.0f, rm = fin ? a.r1[cm] : 0.0f, zm = fin ? a.z1[cm] : 0.0f;
+                const float2 d = half_row_dots(coarse(s_l1, a.l1p, k, c), coarse(s_l1, a.l1p, k + 1, c + nhw), a.l1c,
+                                               a.l1v, hl, [&](int q) { return a.z1[q]; });
+                if (fin) {
+                    const float res = rm - (hl ? d.y : d.x);
+                    const float dd = kCh2a * zm + kCh2b * wm * res;
+                    a.t1[cm] = res;
+                    a.d1[cm] = dd;
+                    a.z1b[cm] = zm + dd;
                 }
             }
             if (!grid_barrier(a.gb, ++epoch, nb, lim)) goto timeout;
             // V3b: the residual after the pre-smoothing, t1 = res - L1 d1
-            for (int c0 = hw - (hw & 1); c0 < a.n1; c0 += nhw) {
-                const int c = c0 + (hw & 1);
-                const float sum = half_row_dot(a.l1p, a.l1c, a.l1v, a.d1, c, c < a.n1, hl);
-                if (hl == 0 && c < a.n1) a.t1[c] -= sum;
+            for (int k = 0, c = hw; c - (hw & 1) < a.n1; k += 2, c += 2 * nhw) {
+                const int cm = c + hl * nhw;
+                const bool fin = ends && cm < a.n1;
+                const float tm = fin ? a.t1[cm] : 0.0f;
+                const float2 d = half_row_dots(coarse(s_l1, a.l1p, k, c), coarse(s_l1, a.l1p, k + 1, c + nhw), a.l1c,
+                                               a.l1v, hl, [&](int q) { return a.d1[q]; });
+                if (fin) a.t1[cm] = tm - (hl ? d.y : d.x);
             }
             if (!grid_barrier(a.gb, ++epoch, nb, lim)) goto timeout;
             // V4: r2 = sum of t1 over each level-2 aggregate
-            for (int g0 = hw - (hw & 1); g0 < a.n2; g0 += nhw) {
-                const int g = g0 + (hw & 1);
-                const float sum = half_row_dot(a.r1p, a.r1c, nullptr, a.t1, g, g < a.n2, hl);
-                if (hl == 0 && g < a.n2) a.r2[g] = sum;
+            for (int g = gw; g < a.n2; g += nw) {
+                const int kb = a.r1p[g], ke = a.r1p[g + 1];
+                float s = 0.0f;
+#pragma unroll 4
+                for (int k = kb + lane; k < ke; k += 32) s += a.t1[a.r1c[k]];
+                s = warp_sum_f(s);
+                if (lane == 0) a.r2[g] = s;
             }
             if (!grid_barrier(a.gb, ++epoch, nb, lim)) goto timeout;
             // V5: z2 = L2^-1 r2 (dense)
@@ -1672,52 +1749,40 @@ __device__ __forceinline__ void mg_body(const MgArgs &a, const int nb, const int
             // V6: coarse correction and the first post-smoothing step in one
             // pass: zc = z1b + z2[agg] (the corrected neighbours formed on the
             // fly), res = r1 - L1 zc (into t1), d1 = kCh1 w1 res, zc + d1 (into z1)
-            for (int c0 = hw - (hw & 1); c0 < a.n1; c0 += nhw) {
-                const int c = c0 + (hw & 1);
-                const bool ok = c < a.n1;
-                float s = 0.0f;
-                if (ok) {
-                    const int kb = a.l1p[c], ke = a.l1p[c + 1];
-                    for (int k0 = kb; k0 < ke; k0 += 64) {
-                        int cc[4];
-                        float v[4];
-#pragma unroll
-                        for (int u = 0; u < 4; u++) {
-                            const int k = k0 + hl + 16 * u;
-                            const bool in = k < ke;
-                            cc[u] = in ? a.l1c[k] : 0;
-                            v[u] = in ? a.l1v[k] : 0.0f;
-                        }
-#pragma unroll
-                        for (int u = 0; u < 4; u++) s = fmaf(v[u], a.z1b[cc[u]] + a.z2[a.agg1[cc[u]]], s);
-                    }
-                }
-#pragma unroll
-                for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
-                if (hl == 0 && ok) {
-                    const float zc = a.z1b[c] + a.z2[a.agg1[c]];
-                    const float res = a.r1[c] - s, d = kCh1 * a.w1[c] * res;
-                    a.t1[c] = res;
-                    a.d1[c] = d;
-                    a.z1[c] = zc + d;
+            for (int k = 0, c = hw; c - (hw & 1) < a.n1; k += 2, c += 2 * nhw) {
+                const int cm = c + hl * nhw;
+                const bool fin = ends && cm < a.n1;
+                const float wm = fin ? a.w1[cm] : 0.0f, rm = fin ? a.r1[cm] : 0.0f;
+                const float zm = fin ? a.z1b[cm] + a.z2[a.agg1[cm]] : 0.0f;
+                const float2 d = half_row_dots(coarse(s_l1, a.l1p, k, c), coarse(s_l1, a.l1p, k + 1, c + nhw), a.l1c,
+                                               a.l1v, hl, [&](int q) { return a.z1b[q] + a.z2[a.agg1[q]]; });
+                if (fin) {
+                    const float res = rm - (hl ? d.y : d.x), dd = kCh1 * wm * res;
+                    a.t1[cm] = res;
+                    a.d1[cm] = dd;
+                    a.z1[cm] = zm + dd;
                 }
             }
             if (!grid_barrier(a.gb, ++epoch, nb, lim)) goto timeout;
             // V6b: the second post-smoothing step, res -= L1 d1,
             // z1b = z1 + kCh2a d1 + kCh2b w1 res
-            for (int c0 = hw - (hw & 1); c0 < a.n1; c0 += nhw) {
-                const int c = c0 + (hw & 1);
-                const float sum = half_row_dot(a.l1p, a.l1c, a.l1v, a.d1, c, c < a.n1, hl);
-                if (hl == 0 && c < a.n1) {
-                    const float res = a.t1[c] - sum;
-                    a.z1b[c] = a.z1[c] + (kCh2a * a.d1[c] + kCh2b * a.w1[c] * res);
+            for (int k = 0, c = hw; c - (hw & 1) < a.n1; k += 2, c += 2 * nhw) {
+                const int cm = c + hl * nhw;
+                const bool fin = ends && cm < a.n1;
+                const float wm = fin ? a.w1[cm] : 0.0f, tm = fin ? a.t1[cm] : 0.0f, zm = fin ? a.z1[cm] : 0.0f,
+                            dm = fin ? a.d1[cm] : 0.0f;
+                const float2 d = half_row_dots(coarse(s_l1, a.l1p, k, c), coarse(s_l1, a.l1p, k + 1, c + nhw), a.l1c,
+                                               a.l1v, hl, [&](int q) { return a.d1[q]; });
+                if (fin) {
+                    const float res = tm - (hl ? d.y : d.x);
+                    a.z1b[cm] = zm + (kCh2a * dm + kCh2b * wm * res);
                 }
             }
             if (!grid_barrier(a.gb, ++epoch, nb, lim)) goto timeout;
             // V7: coarse correction of level 0 (into t0, free now); the row's
             // indices and values (up to 8) are loaded before the gathers
             for (int i = gt; i < a.n0; i += G) {
-                float s = a.z0[i];
+                float s = fac * a.z0[i];
                 const int kb = a.p0p[i], ke = a.p0p[i + 1];
                 for (int k0 = kb; k0 < ke; k0 += 8) {
                     int c[8];
@@ -1734,68 +1799,70 @@ __device__ __forceinline__ void mg_body(const MgArgs &a, const int nb, const int
                 a.t0[i] = s;
             }
             if (!grid_barrier(a.gb, ++epoch, nb, lim)) goto timeout;
-            // V8: post-smoothing on level 0, z = sigma s0 z0 in FP64; (r, z), (r, z_old)
+            // V8: post-smoothing on level 0, z = sigma s0 z0 in FP64
             {
-                double v[2] = {0.0, 0.0};
                 const double zs = sc.zs;
-                for (int sl = gw; sl < a.n_slices; sl += nw) {
-                    const int row = sl * 32 + lane, kb = a.sp[sl] + lane, kw = a.sw[sl];
-                    float s = 0.0f;
-#pragma unroll 4
-                    for (int j = 0; j < kw; j++) s = fmaf(a.L32[kb + 32 * j], a.t0[a.col[kb + 32 * j]], s);
+                for (int k = 0, sl = gw; sl < a.n_slices; k++, sl += nw) {
+                    const int row = sl * 32 + lane;
+                    const float s = sell_row(slice(k, sl), a.L32, a.t0);
+                    if (row < a.n0)
+                        a.z[row] = zs * (double)(a.t0[row] + a.w0[row] * (fac * a.r32[row] - s));
+                }
+            }
+            if (!grid_barrier(a.gb, ++epoch, nb, lim)) goto timeout;
+            // w = L z (in z_old's place once (r, z_old) has read it), and
+            // (r, z), (r, z_old), (z, w), (z, q)
+            {
+                double v[4] = {0.0, 0.0, 0.0, 0.0};
+                for (int k = 0, sl = gw; sl < a.n_slices; k++, sl += nw) {
+                    const int row = sl * 32 + lane;
+                    const double s = sell_row(slice(k, sl), a.Lv, a.z);
                     if (row < a.n0) {
-                        const double zi = zs * (double)(a.t0[row] + a.w0[row] * (a.r32[row] - s));
-                        const double ri = a.r[row];
-                        v[0] += ri * zi;
-                        v[1] += ri * a.zo[row];
-                        a.z[row] = zi;
+                        const double zi = a.z[row], ri = a.r[row];
+                        v[0] = fma(ri, zi, v[0]);
+                        if (!first) {   // z_old, q not read before set
+                            v[1] = fma(ri, a.zo[row], v[1]);
+                            v[3] = fma(zi, a.q[row], v[3]);
+                        }
+                        v[2] = fma(zi, s, v[2]);
+                        a.zo[row] = s;
                     }
                 }
-                if (!grid_reduce<2, T>(a.gb, a.part, v, 0ull, shv, shm, ++epoch, nb, bid, T / 32, lim, [&](const double *t, int wp, int l) {
-                        if (wp + l != 0) return;
-                        sc.rz = t[0];
-                        sc.beta = sc.fresh ? 0.0 : (t[0] - t[1]) / sc.rzo;
-                        sc.rzo = t[0];
-                    }))
+                if (!grid_reduce<4, T>(a.gb, a.part, v, 0ull, shv, shm, ++epoch, nb, bid, T / 32, lim,
+                                       [&](const double *t, int wp, int l) {
+                                           if (wp + l != 0) return;
+                                           const double be = sc.fresh ? 0.0 : (t[0] - t[1]) / sc.rz;
+                                           const double pq = sc.fresh ? t[2] : t[2] + be * (2.0 * t[3] + be * sc.pq);
+                                           sc.beta = be;
+                                           sc.rz = t[0];
+                                           sc.pq = pq;
+                                           sc.alpha = t[0] / pq;
+                                           sc.it++;
+                                           sc.fresh = 0;
+                                       }))
                     goto timeout;
             }
-            const double beta = sc.beta;
-            // w = L z (z is complete: the reduction above was a grid barrier),
-            // p = z + beta p, q = w + beta q (= L p), and (p, q)
+            // p = z + beta p, q = w + beta q, x += alpha p, r -= alpha q; |r|^2
+            // and max|r|; the scaled residual and first sweep of the next V-cycle
             {
-                double v[1] = {0.0};
-                for (int sl = gw; sl < a.n_slices; sl += nw) {
-                    const int row = sl * 32 + lane, kb = a.sp[sl] + lane, kw = a.sw[sl];
-                    double s = 0.0;
-#pragma unroll 4
-                    for (int j = 0; j < kw; j++) s = fma(a.Lv[kb + 32 * j], a.z[a.col[kb + 32 * j]], s);
-                    if (row < a.n0) {
-                        const double zi = a.z[row];
-                        const double pi = first ? zi : zi + beta * a.p[row];   // p, q not read before set
-                        const double qi = first ? s : s + beta * a.q[row];
-                        a.p[row] = pi;
-                        a.q[row] = qi;
-                        a.zo[row] = zi;
-                        v[0] += pi * qi;
-                    }
-                }
-                if (!grid_reduce<1, T>(a.gb, a.part, v, 0ull, shv, shm, ++epoch, nb, bid, T / 32, lim, [&](const double *t, int wp, int l) {
-                        if (wp + l != 0) return;
-                        sc.alpha = sc.rz / t[0];
-                        sc.it++;
-                        sc.fresh = 0;
-                    }))
-                    goto timeout;
-            }
-            const double alpha = sc.alpha;
-            // x += alpha p, r -= alpha q; |r|^2 and max|r|
-            {
+                const double alpha = sc.alpha, beta = sc.beta, inv = sc.inv;
                 double v[1] = {0.0};
                 unsigned long long mx = 0;
-                for (int i = gt; i < a.n0; i += G) {
-                    a.x[i] = fma(alpha, a.p[i], a.x[i]);
-                    const double ri = fma(-alpha, a.q[i], a.r[i]);
+                for (int k = 0, sl = gw; sl < a.n_slices; k++, sl += nw) {
+                    const int i = sl * 32 + lane;
+                    if (i >= a.n0) continue;
+                    const double zi = a.z[i], wi = a.zo[i];
+                    const double pi = first ? zi : fma(beta, a.p[i], zi);
+                    const double qi = first ? wi : fma(beta, a.q[i], wi);
+                    const double ri = fma(-alpha, qi, a.r[i]);
+                    a.p[i] = pi;
+                    a.q[i] = qi;
+                    a.zo[i] = zi;
+                    a.x[i] = fma(alpha, pi, a.x[i]);
                     a.r[i] = ri;
+                    const float rs = (float)(ri * inv);
+                    a.r32[i] = rs;
+                    a.z0[i] = a.w0[i] * rs;
                     v[0] += ri * ri;
                     mx = max(mx, abs_bits(ri));
                 }
@@ -2461,8 +2528,6 @@ static int mg_args(Sim *s, MgArgs &a) {
 
 // launches a multigrid solve on `per_sm` blocks per SM (0: one)
 static int launch_mg(MgArgs &a, int per_sm, cudaStream_t st) {
-    // z_old starts at zero (the first beta is 0 and ignores it, but it is read)
-    FP_CUDA(cudaMemsetAsync(a.zo, 0, sizeof(double) * a.n0, st));
     static CoopKernel kernel((const void *)k_mg_pcg, kMgThreads, 0);
     const int fit = kernel.per_sm();
     if (fit <= 0) {
@@ -2622,8 +2687,7 @@ int prepare_completion_table(Sim *const *sims, int n, int blocks_per_sm, void *t
     return PIC_OK;
 }
 
-// One launch of the table's solves on st (the members' l_p1 zeroed first by
-// the caller for the multigrid runs).  total_blocks: the table's block count,
+// One launch of the table's solves on st.  total_blocks: the table's block count,
 // negative when a run's records are wide.
 int launch_completion_table(const void *table_dev, int n_runs, int total_blocks, cudaStream_t st) {
     if (n_runs <= 0) return PIC_OK;
