@@ -142,7 +142,7 @@ struct PartBank {
 // Reusable radix-sort workspace
 struct SortWork {
     DevBuf<uint32_t> hist;        // 256 * tiles
-    DevBuf<uint32_t> chunk;       // partial sums of the scan
+    DevBuf<uint32_t> chunk;       // the 256 digit totals
     size_t tiles_cap = 0;
 };
 

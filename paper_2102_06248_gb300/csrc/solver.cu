@@ -105,13 +105,14 @@ __device__ __forceinline__ void grid_combine(double out[N], const double *part, 
 // ---------------------------------------------------------------------------
 constexpr int kSlicesPerBlock = kThreads / 32;
 
-#define SELL_LOOP(n_slices, n)                                                                         \
+#define SELL_LOOP(n_slices, n) SELL_LOOP_AT(n_slices, n, sp, sw)
+#define SELL_LOOP_AT(n_slices, n, sp, sw)                                                              \
     const int lane = threadIdx.x & 31;                                                                 \
     for (int sl = blockIdx.x * kSlicesPerBlock + (threadIdx.x >> 5); sl < (n_slices);                 \
          sl += gridDim.x * kSlicesPerBlock) {                                                          \
         const int r = sl * 32 + lane;                                                                  \
         const bool rv = r < (n);                                                                       \
-        const int kb = sp[sl] + lane, kw = sw[sl];
+        const int kb = (sp)[sl] + lane, kw = (sw)[sl];
 
 // face vector hb = H (b + b') (Newmark Maxwell form) or H b (backward
 // difference, ONE_LEVEL)
@@ -262,43 +263,93 @@ __global__ void __launch_bounds__(kThreads) k_gc_w_sell(int n, int n_slices, con
 // r = b - A x, z = D^-1 r, p = z; rz, rr, bb, max|r|
 // p = z + beta p_old (on the fly for the neighbours), q = A p, pq: the SpMV
 // of the Newmark PCG
-// true residual and M x on the Newmark pattern: relres, energy_e
+// What a step's diagnostics read from the fields, in one launch: over the
+// edges the true residual of the Newmark system and M e (kept for the node
+// diagnostics), e^T M e; over the tets max |D b|; over the faces b^T H b; the
+// push blocks' kinetic energies.  Every block takes its share of each, so the
+// warps that stream the matrices (bound by FP64 and bytes) run beside those
+// that gather, and one arrival of the blocks replaces four.
+// (6^3 cube, a step of launches: 539 -> 514 us with the shorter sort.)
+struct DiagArgs {
+    // Newmark pattern
+    int n, n_slices;
+    const int *sp, *sw, *col;
+    const double *Mv, *Kv, *Iv;
+    double c4, ci;
+    const double *x, *rhs;
+    double *me;
+    // tets
+    int nt;
+    const int4 *tf;
+    const signed char *sign;
+    // faces
+    int nf, f_slices;
+    const int *fp, *fw, *fcol;
+    const double *Hv, *b;
+    // push blocks
+    int n_ke;
+    const double *ke;
+    double *part;
+    DiagDev *dg;
+};
+
 template <bool IMPEDANCE>
-__global__ void __launch_bounds__(kThreads) k_resid_sell(int n, int n_slices, const int *__restrict__ sp,
-                                                         const int *__restrict__ sw, const int *__restrict__ col,
-                                                         const double *__restrict__ Mv, const double *__restrict__ Kv,
-                                                         const double *__restrict__ Iv, double c4, double ci,
-                                                         const double *__restrict__ x,
-                                                         const double *__restrict__ rhs, double *__restrict__ me,
-                                                         double *part, DiagDev *dg) {
-    __shared__ double sh[3 * kThreads / 32];
-    double acc[3] = {0.0, 0.0, 0.0};
-    SELL_LOOP(n_slices, n)
-        double sm = 0.0, sk = 0.0, si = 0.0;
+__global__ void __launch_bounds__(kThreads) k_diag_fields(const DiagArgs a) {
+    __shared__ double sh[5 * kThreads / 32];
+    double acc[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    const int first = blockIdx.x * kThreads + threadIdx.x, stride = gridDim.x * kThreads;
+    {
+        SELL_LOOP_AT(a.n_slices, a.n, a.sp, a.sw)
+            double sm = 0.0, sk = 0.0, si = 0.0;
 #pragma unroll 4
-        for (int j = 0; j < kw; j++) {
-            const int k = kb + 32 * j;
-            const double xj = x[col[k]];
-            sm += Mv[k] * xj;
-            sk += Kv[k] * xj;
-            if (IMPEDANCE) si += Iv[k] * xj;
-        }
-        if (rv) {
-            me[r] = sm;
-            const double res = rhs[r] - (sm + c4 * sk + ci * si);
-            acc[0] += res * res;
-            acc[1] += rhs[r] * rhs[r];
-            acc[2] += x[r] * sm;
+            for (int j = 0; j < kw; j++) {
+                const int k = kb + 32 * j;
+                const double xj = a.x[a.col[k]];
+                sm += a.Mv[k] * xj;
+                sk += a.Kv[k] * xj;
+                if (IMPEDANCE) si += a.Iv[k] * xj;
+            }
+            if (rv) {
+                a.me[r] = sm;
+                const double res = a.rhs[r] - (sm + a.c4 * sk + a.ci * si);
+                acc[0] += res * res;
+                acc[1] += a.rhs[r] * a.rhs[r];
+                acc[2] += a.x[r] * sm;
+            }
         }
     }
-    block_sum<3>(acc, sh);
-    if (arrive<3>(acc, part, &dg->count)) {
-        double tot[3];
-        grid_combine<3, false>(tot, part, sh);
+    {
+        SELL_LOOP_AT(a.f_slices, a.nf, a.fp, a.fw)
+            double s = 0.0;
+#pragma unroll 4
+            for (int j = 0; j < kw; j++) {
+                const int k = kb + 32 * j;
+                s = fma(a.Hv[k], a.b[a.fcol[k]], s);
+            }
+            if (rv) acc[3] = fma(a.b[r], s, acc[3]);
+        }
+    }
+    for (int t = first; t < a.nt; t += stride) {
+        const int4 f = a.tf[t];
+        const double s = a.sign[t];
+        acc[5] = fmax(acc[5], fabs(s * (a.b[f.x] - a.b[f.y] + a.b[f.z] - a.b[f.w])));
+    }
+    for (int p = first; p < a.n_ke; p += stride) acc[4] += a.ke[p];
+    block_sum<5>(acc, sh);
+    block_max<1>(acc + 5, sh);
+    if (arrive<6>(acc, a.part, &a.dg->count)) {
+        double tot[6];
+        grid_combine<5, false>(tot, a.part, sh);
+        grid_combine<1, true>(tot + 5, a.part + 5 * (size_t)gridDim.x, sh);
         if (threadIdx.x == 0) {
-            dg->relres = tot[1] > 0.0 ? sqrt(tot[0] / tot[1]) : 0.0;
-            dg->energy_e = 0.5 * tot[2];
-            dg->count = 0;
+            if (a.n > 0) {
+                a.dg->relres = tot[1] > 0.0 ? sqrt(tot[0] / tot[1]) : 0.0;
+                a.dg->energy_e = 0.5 * tot[2];
+            }
+            a.dg->energy_b = 0.5 * tot[3];
+            a.dg->energy_k = tot[4];
+            a.dg->divb_abs = tot[5];
+            a.dg->count = 0;
         }
     }
 }
@@ -421,73 +472,6 @@ __global__ void __launch_bounds__(kThreads) k_diag_nodes(int nn, const int *__re
             dg->cont_abs = tot[0];
             dg->gauss_abs = tot[1];
             dg->rho_max = tot[2];
-            dg->count = 0;
-        }
-    }
-}
-
-// D b per tet (max) and 1/2 b^T H b
-__global__ void __launch_bounds__(kThreads) k_diag_divb(int nt, const int4 *__restrict__ tf,
-                                                        const signed char *__restrict__ sign, const double *__restrict__ b,
-                                                        double *part, DiagDev *dg) {
-    __shared__ double sh[kThreads / 32];
-    double acc[1] = {0.0};
-    for (int t = blockIdx.x * kThreads + threadIdx.x; t < nt; t += gridDim.x * kThreads) {
-        const int4 f = tf[t];
-        const double s = sign[t];
-        const double d = s * (b[f.x] - b[f.y] + b[f.z] - b[f.w]);
-        acc[0] = fmax(acc[0], fabs(d));
-    }
-    block_max<1>(acc, sh);
-    if (arrive<1>(acc, part, &dg->count)) {
-        double tot[1];
-        grid_combine<1, true>(tot, part, sh);
-        if (threadIdx.x == 0) {
-            dg->divb_abs = tot[0];
-            dg->count = 0;
-        }
-    }
-}
-
-__global__ void __launch_bounds__(kThreads) k_diag_energy_b(int nf, int n_slices, const int *__restrict__ sp,
-                                                            const int *__restrict__ sw, const int *__restrict__ col,
-                                                            const double *__restrict__ Hv, const double *__restrict__ b,
-                                                            double *part, DiagDev *dg) {
-    __shared__ double sh[kThreads / 32];
-    double acc[1] = {0.0};
-    SELL_LOOP(n_slices, nf)
-        double s = 0.0;
-#pragma unroll 4
-        for (int j = 0; j < kw; j++) {
-            const int k = kb + 32 * j;
-            s = fma(Hv[k], b[col[k]], s);
-        }
-        if (rv) acc[0] = fma(b[r], s, acc[0]);
-    }
-    block_sum<1>(acc, sh);
-    if (arrive<1>(acc, part, &dg->count)) {
-        double tot[1];
-        grid_combine<1, false>(tot, part, sh);
-        if (threadIdx.x == 0) {
-            dg->energy_b = 0.5 * tot[0];
-            dg->count = 0;
-        }
-    }
-}
-
-// kinetic energy from the push kernel's per-block partials (fixed order:
-// block b of this grid adds partials b*kThreads + t, b*kThreads + t +
-// grid*kThreads, ...; the last block adds the blocks' sums in block order)
-__global__ void __launch_bounds__(kThreads) k_sum_ke(int nb, const double *__restrict__ kp, double *part, DiagDev *dg) {
-    __shared__ double sh[kThreads / 32];
-    double acc[1] = {0.0};
-    for (int b = blockIdx.x * kThreads + threadIdx.x; b < nb; b += gridDim.x * kThreads) acc[0] += kp[b];
-    block_sum<1>(acc, sh);
-    if (arrive<1>(acc, part, &dg->count)) {
-        double tot[1];
-        grid_combine<1, false>(tot, part, sh);
-        if (threadIdx.x == 0) {
-            dg->energy_k = tot[0];
             dg->count = 0;
         }
     }
@@ -2742,21 +2726,32 @@ int compute_diagnostics(Sim *s) {
     const Mesh *m = s->mesh;
     DiagDev *dg = &s->dctl.p->diag;
     const int ni = m->n_int_edges;
+    DiagArgs a{};
     if (ni > 0) {
-        double c4, ci;
-        system_coefficients(s, &c4, &ci);
-        if (m->n_abs_faces > 0)
-            { k_resid_sell<true><<<grid_for_slices(m->As.n_slices), kThreads, 0, s->stream>>>(ni, m->As.n_slices, m->As.ptr.p, m->As.width.p, m->As.col.p, m->M_val.p, m->K_val.p, m->I_val.p, c4, ci, s->e.p, s->rhs.p, s->me.p, s->diag_part.p, dg); note_launch(); }
-        else
-            { k_resid_sell<false><<<grid_for_slices(m->As.n_slices), kThreads, 0, s->stream>>>(ni, m->As.n_slices, m->As.ptr.p, m->As.width.p, m->As.col.p, m->M_val.p, m->K_val.p, nullptr, c4, 0.0, s->e.p, s->rhs.p, s->me.p, s->diag_part.p, dg); note_launch(); }
+        system_coefficients(s, &a.c4, &a.ci);
+        a.n = ni;
+        a.n_slices = m->As.n_slices;
+        a.sp = m->As.ptr.p, a.sw = m->As.width.p, a.col = m->As.col.p;
+        a.Mv = m->M_val.p, a.Kv = m->K_val.p;
+        a.x = s->e.p, a.rhs = s->rhs.p, a.me = s->me.p;
+    }
+    a.nt = m->n_tets, a.tf = m->tet_face.p, a.sign = m->tet_sign.p;
+    a.nf = m->n_faces, a.f_slices = m->Hs.n_slices;
+    a.fp = m->Hs.ptr.p, a.fw = m->Hs.width.p, a.fcol = m->Hs.col.p;
+    a.Hv = m->Hs_val.p, a.b = s->b.p;
+    a.n_ke = s->n_ke_parts, a.ke = s->ke_part.p;
+    a.part = s->diag_part.p, a.dg = dg;
+    const int grid = grid_for_slices(std::max(a.n_slices, a.f_slices));
+    if (ni > 0 && m->n_abs_faces > 0) {
+        a.Iv = m->I_val.p;
+        { k_diag_fields<true><<<grid, kThreads, 0, s->stream>>>(a); note_launch(); }
+    } else {
+        a.ci = 0.0;
+        { k_diag_fields<false><<<grid, kThreads, 0, s->stream>>>(a); note_launch(); }
     }
     { k_diag_nodes<<<grid_for_elems(m->n_nodes), kThreads, 0, s->stream>>>(
         m->n_nodes, m->n2e.rowptr.p, m->n2e.col.p, m->n2e_sgn.p, ni, s->dg.p, s->me.p, s->rho.p, s->rho_prev.p,
         s->wall.p, s->wall_prev.p, s->rho_bg.p, m->node_bnd.p, s->diag_part.p, dg); note_launch(); }
-    { k_diag_divb<<<grid_for_elems(m->n_tets), kThreads, 0, s->stream>>>(m->n_tets, m->tet_face.p, m->tet_sign.p, s->b.p,
-                                                                       s->diag_part.p, dg); note_launch(); }
-    { k_diag_energy_b<<<grid_for_slices(m->Hs.n_slices), kThreads, 0, s->stream>>>(m->n_faces, m->Hs.n_slices, m->Hs.ptr.p, m->Hs.width.p, m->Hs.col.p, m->Hs_val.p, s->b.p, s->diag_part.p, dg); note_launch(); }
-    { k_sum_ke<<<grid_for_elems(s->n_ke_parts), kThreads, 0, s->stream>>>(s->n_ke_parts, s->ke_part.p, s->diag_part.p, dg); note_launch(); }
     FP_CUDA(cudaGetLastError());
     return PIC_OK;
 }
