@@ -28,8 +28,8 @@
 
 #include "sim.h"
 
-// tuner candidates: blocks per SM and kernel build (0: 64 registers, 1: 80,
-// 2: 40, 3: 32)
+// tuner candidates: blocks per SM and kernel build (0: 64 registers, 1: 80;
+// 2 and 3 stand for four blocks of 0)
 constexpr int kTuneCands = 9;
 constexpr int kTuneBps[kTuneCands] = {2, 3, 4, 2, 3, 5, 6, 7, 8};
 constexpr int kTuneBuild[kTuneCands] = {0, 0, 0, 1, 1, 2, 2, 3, 3};
