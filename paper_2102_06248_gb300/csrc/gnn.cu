@@ -241,82 +241,160 @@ __global__ void __launch_bounds__(kT) k_embed(int n, const int *__restrict__ edg
     }
 }
 
-// sum_j Ahat_ij v_j for feature `lane` of row i: the row's (column, weight)
-// pairs are loaded by one lane each, 32 at a time, and broadcast with
-// shuffles, so all neighbour loads of a chunk are independent and in flight
-// together
-__device__ __forceinline__ float aggregate(int i, const int *__restrict__ sp, const int *__restrict__ sw,
-                                           const int *__restrict__ col, const float *__restrict__ ahat,
-                                           const float *__restrict__ v, float acc) {
-    const int lane = threadIdx.x & 31;
-    const int sl = i >> 5, kb = sp[sl] + (i & 31), kw = sw[sl];
-    for (int j0 = 0; j0 < kw; j0 += 32) {
-        const int m = min(32, kw - j0);
-        int cj = 0;
-        float aj = 0.0f;
-        if (lane < m) {
-            cj = col[kb + 32 * (j0 + lane)];
-            aj = ahat[kb + 32 * (j0 + lane)];
+constexpr int kTileRows = 16;
+constexpr int kSRow = 2 * kH + 4;       // padded row of S: conflict-free fragment loads
+
+__device__ __forceinline__ void load4(const float *p, float v[4]) {
+    const float4 x = *reinterpret_cast<const float4 *>(p);
+    v[0] = x.x;
+    v[1] = x.y;
+    v[2] = x.z;
+    v[3] = x.w;
+}
+
+__device__ __forceinline__ void fma4(float4 &acc, float a, float4 v) {
+    acc.x = fmaf(a, v.x, acc.x);
+    acc.y = fmaf(a, v.y, acc.y);
+    acc.z = fmaf(a, v.z, acc.z);
+    acc.w = fmaf(a, v.w, acc.w);
+}
+
+// acc[p] += sum_j Ahat_ij v_j for the rows i = 16 tile + rs + 4p (rs = lane >> 3)
+// and their features 4 (lane & 7) .. + 3, entries in increasing order: each
+// 16-byte gather of the warp reads four whole 128-byte feature rows, and a
+// row's column and weight are read by the eight lanes that use them.  SELL padding
+// has weight 0 and names an existing row.
+__device__ __forceinline__ void aggregate_tile(int tile, const int *__restrict__ sp, const int *__restrict__ sw,
+                                               const int *__restrict__ col, const float *__restrict__ ahat,
+                                               const float *__restrict__ v, float4 acc[4]) {
+    const int lane = threadIdx.x & 31, rs = lane >> 3, q8 = lane & 7;
+    const int sl = tile >> 1, kb0 = sp[sl] + (tile & 1) * kTileRows, kw = sw[sl];
+#pragma unroll 2
+    for (int j = 0; j < kw; j++) {
+        int c[4];
+        float a[4];
+#pragma unroll
+        for (int p = 0; p < 4; p++) {
+            const int e = kb0 + rs + 4 * p + 32 * j;
+            c[p] = col[e];
+            a[p] = ahat[e];
         }
-#pragma unroll 8
-        for (int j = 0; j < m; j++) {
-            const int c = __shfl_sync(0xFFFFFFFFu, cj, j);
-            const float a = __shfl_sync(0xFFFFFFFFu, aj, j);
-            acc = fmaf(a, v[(size_t)c * kH + lane], acc);
-        }
+#pragma unroll
+        for (int p = 0; p < 4; p++)
+            fma4(acc[p], a[p], __ldg(reinterpret_cast<const float4 *>(v + (size_t)c[p] * kH + 4 * q8)));
     }
-    return acc;
 }
 
 // one message-passing layer of the training forward pass; the last one also
 // forms z.  It stores the aggregates and pre-activations the backward pass
-// reads (a preconditioner application uses k_layer_tc below instead)
+// reads (a preconditioner application uses k_layer_tc below instead).  FP32
+// throughout, each sum in one fixed order.  A warp takes 16 consecutive
+// rows: the tile's h and g go to shared memory and each lane forms 4 features
+// of 4 rows, so that 16 words read from shared memory serve 32 multiply-adds
+// (the words that come back from shared memory or by shuffles bound it: 152 a
+// row with a warp per row, 244 us at 220,256 rows; 68 with a feature a lane,
+// 86 us; 32 now, 77 us).
 template <bool LAST>
 __global__ void __launch_bounds__(kT) k_layer(int n, const int *__restrict__ sp, const int *__restrict__ sw,
                                              const int *__restrict__ col, const float *__restrict__ ahat,
                                              const float *__restrict__ hp, const unsigned short *__restrict__ th,
                                              int off, float *__restrict__ g, float *__restrict__ pre,
                                              float *__restrict__ h, const int *__restrict__ edge,
-                                             const double *__restrict__ r, const double *__restrict__ Dinv, const double *__restrict__ isd,
-                                             const double *__restrict__ nrm, double *__restrict__ z) {
-    __shared__ float Wt[kH * kH], Qt[kH * kH], bsh[kH], osh[kH];
+                                             const double *__restrict__ r, const double *__restrict__ Dinv,
+                                             const double *__restrict__ isd, const double *__restrict__ nrm,
+                                             double *__restrict__ z) {
+    extern __shared__ __align__(16) float layer_sh[];
+    float *Wt = layer_sh, *Qt = Wt + kH * kH;
+    float *S = Qt + kH * kH + (threadIdx.x >> 5) * kTileRows * kSRow;
     for (int t = threadIdx.x; t < kH * kH; t += kT) {
         const int f = t >> 5, k = t & 31;   // W[f][k] -> Wt[k][f]
         Wt[k * kH + f] = bf(th, off + t);
         Qt[k * kH + f] = bf(th, off + kH * kH + t);
     }
-    if (threadIdx.x < kH) {
-        bsh[threadIdx.x] = bf(th, off + 2 * kH * kH + threadIdx.x);
-        osh[threadIdx.x] = LAST ? bf(th, kOffO + threadIdx.x) : 0.0f;
-    }
-    __syncthreads();
-    const int lane = threadIdx.x & 31;
-    const float d0 = LAST ? bf(th, kOffD0) : 0.0f;
     const double rho = LAST ? block_rho(nrm, n) : 0.0;
-    for (int i = blockIdx.x * kW + (threadIdx.x >> 5); i < n; i += gridDim.x * kW) {
-        const float hi = hp[(size_t)i * kH + lane];
-        const float gi = aggregate(i, sp, sw, col, ahat, hp, 0.0f);
-        float p = bsh[lane];
+    __syncthreads();
+    const int lane = threadIdx.x & 31, rs = lane >> 3, q8 = lane & 7;
+    float b[4], o[4];
 #pragma unroll
-        for (int k = 0; k < kH; k++) {
-            p = fmaf(Wt[k * kH + lane], __shfl_sync(0xFFFFFFFFu, hi, k), p);
-            p = fmaf(Qt[k * kH + lane], __shfl_sync(0xFFFFFFFFu, gi, k), p);
-        }
-        const float hn = fmaxf(p, 0.0f);
-        g[(size_t)i * kH + lane] = gi;
-        pre[(size_t)i * kH + lane] = p;
-        h[(size_t)i * kH + lane] = hn;
-        if (LAST) {
-            float y = osh[lane] * hn;
+    for (int u = 0; u < 4; u++) {
+        b[u] = bf(th, off + 2 * kH * kH + 4 * q8 + u);
+        o[u] = LAST ? bf(th, kOffO + 4 * q8 + u) : 0.0f;
+    }
+    const float d0 = LAST ? bf(th, kOffD0) : 0.0f;
+    const int ntiles = (n + kTileRows - 1) / kTileRows;
+    for (int tile = blockIdx.x * kW + (threadIdx.x >> 5); tile < ntiles; tile += gridDim.x * kW) {
+        const int row0 = tile * kTileRows;
+        float4 acc[4];
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) y += __shfl_down_sync(0xFFFFFFFFu, y, o);
-            if (lane == 0) {
-                const int e = edge[i];
-                z[e] = fma(r[e], Dinv[e], rho * (double)(y + d0) * isd[i]);
+        for (int p = 0; p < 4; p++) acc[p] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        aggregate_tile(tile, sp, sw, col, ahat, hp, acc);
+        __syncwarp();   // the previous tile has been read
+#pragma unroll
+        for (int p = 0; p < 4; p++) {
+            const int i = row0 + rs + 4 * p;
+            float *srow = S + (rs + 4 * p) * kSRow + 4 * q8;
+            float4 hv = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            if (i < n) {
+                hv = __ldg(reinterpret_cast<const float4 *>(hp + (size_t)i * kH + 4 * q8));
+                *reinterpret_cast<float4 *>(g + (size_t)i * kH + 4 * q8) = acc[p];
             }
+            *reinterpret_cast<float4 *>(srow) = hv;
+            *reinterpret_cast<float4 *>(srow + kH) = acc[p];
+        }
+        __syncwarp();
+        // rows rs + 4p, features 4 q8 + u
+        float v[4][4];
+#pragma unroll
+        for (int p = 0; p < 4; p++)
+#pragma unroll
+            for (int u = 0; u < 4; u++) v[p][u] = b[u];
+#pragma unroll 2
+        for (int k = 0; k < kH; k += 4) {
+            float hk[4][4], gk[4][4];
+#pragma unroll
+            for (int p = 0; p < 4; p++) {
+                load4(S + (rs + 4 * p) * kSRow + k, hk[p]);
+                load4(S + (rs + 4 * p) * kSRow + kH + k, gk[p]);
+            }
+#pragma unroll
+            for (int t = 0; t < 4; t++) {
+                float w[4], q[4];
+                load4(Wt + (k + t) * kH + 4 * q8, w);
+                load4(Qt + (k + t) * kH + 4 * q8, q);
+#pragma unroll
+                for (int p = 0; p < 4; p++)
+#pragma unroll
+                    for (int u = 0; u < 4; u++) v[p][u] = fmaf(q[u], gk[p][t], fmaf(w[u], hk[p][t], v[p][u]));
+            }
+        }
+        float yrow = 0.0f;
+#pragma unroll
+        for (int p = 0; p < 4; p++) {
+            const int i = row0 + rs + 4 * p;
+            const float4 hn = make_float4(fmaxf(v[p][0], 0.0f), fmaxf(v[p][1], 0.0f), fmaxf(v[p][2], 0.0f), fmaxf(v[p][3], 0.0f));
+            if (i < n) {
+                *reinterpret_cast<float4 *>(pre + (size_t)i * kH + 4 * q8) = make_float4(v[p][0], v[p][1], v[p][2], v[p][3]);
+                *reinterpret_cast<float4 *>(h + (size_t)i * kH + 4 * q8) = hn;
+            }
+            if (LAST) {
+                // the 32 features added as a tree: f + 16, + 8, + 4, + 2, + 1
+                float y[4] = {o[0] * hn.x, o[1] * hn.y, o[2] * hn.z, o[3] * hn.w};
+#pragma unroll
+                for (int t = 4; t > 0; t >>= 1)
+#pragma unroll
+                    for (int u = 0; u < 4; u++) y[u] += __shfl_down_sync(0xFFFFFFFFu, y[u], t, 8);
+                const float yi = (y[0] + y[2]) + (y[1] + y[3]);
+                const float yr = __shfl_sync(0xFFFFFFFFu, yi, 0, 8);
+                if (q8 == p) yrow = yr;
+            }
+        }
+        if (LAST && q8 < 4 && row0 + rs + 4 * q8 < n) {
+            const int i = row0 + rs + 4 * q8, e = edge[i];
+            z[e] = fma(r[e], Dinv[e], rho * (double)(yrow + d0) * isd[i]);
         }
     }
 }
+constexpr int kLayerShared = (2 * kH * kH + kW * kTileRows * kSRow) * (int)sizeof(float);
 
 // ---- inference layer on the tensor cores ----
 // The preconditioner application inside the flexible PCG (no backward pass,
@@ -339,8 +417,6 @@ __global__ void __launch_bounds__(kT) k_layer(int n, const int *__restrict__ sp,
 //   A: a0 (g, t), a1 (g + 8, t), a2 (g, t + 4), a3 (g + 8, t + 4)
 //   B: b0 (k = t, n = g), b1 (k = t + 4, n = g)
 //   C: c0 (g, 2t), c1 (g, 2t + 1), c2 (g + 8, 2t), c3 (g + 8, 2t + 1)
-constexpr int kTileRows = 16;
-constexpr int kSRow = 2 * kH + 4;       // padded row of S: conflict-free fragment loads
 constexpr int kTcBlocksPerSm = 4;
 
 __device__ __forceinline__ uint32_t to_tf32(float x) {
@@ -355,13 +431,6 @@ __device__ __forceinline__ void mma_tf32(float c[4], const uint32_t a[4], float2
         "{%0, %1, %2, %3};"
         : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(__float_as_uint(b.x)), "r"(__float_as_uint(b.y)));
-}
-
-__device__ __forceinline__ void fma4(float4 &acc, float a, float4 v) {
-    acc.x = fmaf(a, v.x, acc.x);
-    acc.y = fmaf(a, v.y, acc.y);
-    acc.z = fmaf(a, v.z, acc.z);
-    acc.w = fmaf(a, v.w, acc.w);
 }
 
 template <bool LAST>
@@ -404,30 +473,14 @@ __global__ void __launch_bounds__(kT, kTcBlocksPerSm) k_layer_tc(int n, const in
     double dots[2] = {0.0, 0.0};   // (r, z), (r, z_old)
     const int ntiles = (n + kTileRows - 1) / kTileRows;
     for (int tile = blockIdx.x * kW + warp; tile < ntiles; tile += gridDim.x * kW) {
-        const int sl = tile >> 1, row0 = tile * kTileRows;
-        const int kb0 = sp[sl] + (tile & 1) * kTileRows, kw = sw[sl];
+        const int row0 = tile * kTileRows;
         float4 acc[4], hv[4];
 #pragma unroll
         for (int p = 0; p < 4; p++) {
             acc[p] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
             hv[p] = acc[p];
         }
-        // SELL padding points at the row itself with weight 0; the slice's
-        // entries exist for all its 32 lanes, so rows past n read weight 0
-#pragma unroll 2
-        for (int j = 0; j < kw; j++) {
-            int c[4];
-            float a[4];
-#pragma unroll
-            for (int p = 0; p < 4; p++) {
-                const int e = kb0 + rs + 4 * p + 32 * j;
-                c[p] = col[e];
-                a[p] = ahat[e];
-            }
-#pragma unroll
-            for (int p = 0; p < 4; p++)
-                fma4(acc[p], a[p], __ldg(reinterpret_cast<const float4 *>(hp + (size_t)c[p] * kH + 4 * q8)));
-        }
+        aggregate_tile(tile, sp, sw, col, ahat, hp, acc);
 #pragma unroll
         for (int p = 0; p < 4; p++) {
             const int i = row0 + rs + 4 * p;
@@ -554,90 +607,247 @@ __device__ __forceinline__ void block_accumulate(const float acc[NA], float *sh,
     for (int t = threadIdx.x; t < NA * 32; t += kT) part[(size_t)blockIdx.x * NA * 32 + t] = sh[t];
 }
 
-// Layer l backward.  dpre = dh * [pre > 0]; per-lane (f) accumulators of
-// dW[f][k], dQ[f][k], db[f] (and, for the last layer, do[f], dd0); writes
+// Layer l backward.  dpre = dh * [pre > 0]; dW[f][k] += dpre_f h_k, dQ[f][k] +=
+// dpre_f g_k, db[f] += dpre_f (and, for the last layer, do[f], dd0); writes
 // own = W^T dpre into dh_out and t = Q^T dpre into tq (aggregated next).
+// A warp takes kBwdRows of its rows at a time through shared memory, the next ones
+// in flight meanwhile (128 registers leave 16 warps an SM).  A lane holds 8 x 4
+// entries of dW and dQ and forms 4 entries of own or t for 4 rows, 48 words
+// read from shared memory a row.  220,256 rows: 210 us with a warp per row and
+// 160 words read or shuffled, 131 without the fetch ahead, 73 us now.  A
+// warp's rows stay a grid apart and are added in increasing order, one sum per entry, so
+// the sums do not depend on this split.
+constexpr int kBwdRows = 8;
+constexpr int kBRow = 4 * kH + 4, kARow = kH + 4;   // padded rows: no bank conflicts
+
+// 16 or 8 bytes of global memory to shared memory, asynchronously; zeros where !ok
+template <int BYTES>
+__device__ __forceinline__ void copy_async(float *dst, const void *src, bool ok) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(d), "l"(src), "n"(BYTES), "r"(ok ? BYTES : 0)
+                 : "memory");
+}
+
 template <bool LAST>
-__global__ void __launch_bounds__(kT, 1) k_layer_bwd(int n, const float *__restrict__ hp,
+__global__ void __launch_bounds__(kT, 2) k_layer_bwd(int n, const float *__restrict__ hp,
                                                     const float *__restrict__ g, const float *__restrict__ pre,
                                                     const float *__restrict__ hcur, const float *__restrict__ dh_in,
                                                     const double *__restrict__ gy,
                                                     const unsigned short *__restrict__ th, int off,
                                                     float *__restrict__ dh_out, float *__restrict__ tq,
                                                     float *__restrict__ part) {
-    __shared__ float Wsh[kH * kH], Qsh[kH * kH], osh[kH];
-    __shared__ float acc_sh[(2 * kH + 3) * 32];
-    for (int t = threadIdx.x; t < kH * kH; t += kT) {
-        Wsh[t] = bf(th, off + t);
-        Qsh[t] = bf(th, off + kH * kH + t);
-    }
-    if (threadIdx.x < kH) osh[threadIdx.x] = LAST ? bf(th, kOffO + threadIdx.x) : 0.0f;
+    extern __shared__ __align__(16) float bwd_sh[];
+    float *WQ = bwd_sh;                                             // W, then Q
+    float *acc_sh = WQ + 2 * kH * kH;                               // dW, then dQ: [f][k]
+    float *vec_sh = acc_sh + 2 * kH * kARow;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // two batches of rows a warp: h, g, pre (then dpre), dh (last layer: h of the layer), gy
+    float *rows_sh = vec_sh + 3 * 32 + warp * 2 * kBwdRows * kBRow;
+    for (int t = threadIdx.x; t < 2 * kH * kH; t += kT) WQ[t] = bf(th, off + t);
     __syncthreads();
-    const int lane = threadIdx.x & 31;
-    constexpr int NA = kNA;   // dW row, dQ row, db, do, dd0
-    float acc[NA];
+    const float o = LAST ? bf(th, kOffO + lane) : 0.0f;
+    const int f0 = 8 * (lane >> 3), k0 = 4 * (lane & 7);            // entries of dW, dQ
+    const int m0 = 4 * (lane >> 4), q = (lane >> 3) & 1;            // rows, own (0) or t (1), ...
+    const float *M = WQ + q * kH * kH + k0;                         // ... entries k0 .. k0 + 3
+    float *out = q ? tq : dh_out;
+    float aw[8][4], aq[8][4], vec[3] = {0.0f, 0.0f, 0.0f};          // vec: db, do, dd0
 #pragma unroll
-    for (int q = 0; q < NA; q++) acc[q] = 0.0f;
-    for (int i = blockIdx.x * kW + (threadIdx.x >> 5); i < n; i += gridDim.x * kW) {
-        float dh;
-        if (LAST) {
-            const float gyi = (float)gy[i];
-            dh = gyi * osh[lane];
-            acc[2 * kH + 1] = fmaf(gyi, hcur[(size_t)i * kH + lane], acc[2 * kH + 1]);
-            if (lane == 0) acc[2 * kH + 2] += gyi;
-        } else {
-            dh = dh_in[(size_t)i * kH + lane];
-        }
-        const float dp = pre[(size_t)i * kH + lane] > 0.0f ? dh : 0.0f;
-        const float hv = hp[(size_t)i * kH + lane], gv = g[(size_t)i * kH + lane];
-        float own = 0.0f, t = 0.0f;
+    for (int f = 0; f < 8; f++)
 #pragma unroll
-        for (int k = 0; k < kH; k++) {
-            acc[k] = fmaf(dp, __shfl_sync(0xFFFFFFFFu, hv, k), acc[k]);
-            acc[kH + k] = fmaf(dp, __shfl_sync(0xFFFFFFFFu, gv, k), acc[kH + k]);
-            const float dpk = __shfl_sync(0xFFFFFFFFu, dp, k);   // dpre of feature f = k
-            own = fmaf(Wsh[k * kH + lane], dpk, own);
-            t = fmaf(Qsh[k * kH + lane], dpk, t);
+        for (int u = 0; u < 4; u++) aw[f][u] = aq[f][u] = 0.0f;
+    const int stride = gridDim.x * kW;
+    // four rows an instruction, eight lanes a row (a row past the end: zeros)
+    auto fetch = [&](int i0, float *S) {
+#pragma unroll
+        for (int half = 0; half < 2; half++) {
+            const int m = 4 * half + (lane >> 3), i = i0 + m * stride;
+            const bool ok = i < n;
+            const size_t at = (size_t)(ok ? i : 0) * kH + k0;
+            float *row = S + m * kBRow + k0;
+            copy_async<16>(row, hp + at, ok);
+            copy_async<16>(row + kH, g + at, ok);
+            copy_async<16>(row + 2 * kH, pre + at, ok);
+            copy_async<16>(row + 3 * kH, (LAST ? hcur : dh_in) + at, ok);
         }
-        acc[2 * kH] += dp;
-        dh_out[(size_t)i * kH + lane] = own;
-        tq[(size_t)i * kH + lane] = t;
+        if (LAST && lane < kBwdRows) {
+            const int i = i0 + lane * stride;
+            copy_async<8>(S + lane * kBRow + 4 * kH, gy + (i < n ? i : 0), i < n);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    int i0 = blockIdx.x * kW + warp;
+    fetch(i0, rows_sh);
+    for (int buf = 0; i0 < n; i0 += kBwdRows * stride, buf ^= 1) {
+        float *S = rows_sh + buf * kBwdRows * kBRow;
+        fetch(i0 + kBwdRows * stride, rows_sh + (buf ^ 1) * kBwdRows * kBRow);
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncwarp();
+#pragma unroll
+        for (int m = 0; m < kBwdRows; m++) {
+            float *row = S + m * kBRow;
+            float dh = row[3 * kH + lane];
+            if (LAST) {
+                const float gyi = (float)*reinterpret_cast<const double *>(row + 4 * kH);
+                vec[1] = fmaf(gyi, dh, vec[1]);
+                vec[2] += gyi;
+                dh = gyi * o;
+            }
+            const float dp = row[2 * kH + lane] > 0.0f ? dh : 0.0f;
+            vec[0] += dp;
+            row[2 * kH + lane] = dp;
+        }
+        __syncwarp();
+#pragma unroll 2
+        for (int m = 0; m < kBwdRows; m++) {
+            float d[8], h4[4], g4[4];
+            load4(S + m * kBRow + 2 * kH + f0, d);
+            load4(S + m * kBRow + 2 * kH + f0 + 4, d + 4);
+            load4(S + m * kBRow + k0, h4);
+            load4(S + m * kBRow + kH + k0, g4);
+#pragma unroll
+            for (int f = 0; f < 8; f++)
+#pragma unroll
+                for (int u = 0; u < 4; u++) {
+                    aw[f][u] = fmaf(d[f], h4[u], aw[f][u]);
+                    aq[f][u] = fmaf(d[f], g4[u], aq[f][u]);
+                }
+        }
+        float y[4][4];
+#pragma unroll
+        for (int m = 0; m < 4; m++)
+#pragma unroll
+            for (int u = 0; u < 4; u++) y[m][u] = 0.0f;
+#pragma unroll 2
+        for (int f = 0; f < kH; f += 4) {
+            float d[4][4];
+#pragma unroll
+            for (int m = 0; m < 4; m++) load4(S + (m0 + m) * kBRow + 2 * kH + f, d[m]);
+#pragma unroll
+            for (int t = 0; t < 4; t++) {
+                float w[4];
+                load4(M + (f + t) * kH, w);
+#pragma unroll
+                for (int m = 0; m < 4; m++)
+#pragma unroll
+                    for (int u = 0; u < 4; u++) y[m][u] = fmaf(w[u], d[m][t], y[m][u]);
+            }
+        }
+#pragma unroll
+        for (int m = 0; m < 4; m++) {
+            const int i = i0 + (m0 + m) * stride;
+            if (i < n) *reinterpret_cast<float4 *>(out + (size_t)i * kH + k0) = make_float4(y[m][0], y[m][1], y[m][2], y[m][3]);
+        }
+        __syncwarp();   // the batch has been read: the next fetch may overwrite it
     }
-    block_accumulate<NA>(acc, acc_sh, part);
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    // the warps' sums in warp order, then the block's partials [q * 32 + f]
+    for (int w = 0; w < kW; w++) {
+        if (warp == w) {
+#pragma unroll
+            for (int f = 0; f < 8; f++) {
+                float *pw = acc_sh + (f0 + f) * kARow + k0, *pq = pw + kH * kARow;
+                float sw4[4] = {0.0f, 0.0f, 0.0f, 0.0f}, sq4[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+                if (w > 0) {
+                    load4(pw, sw4);
+                    load4(pq, sq4);
+                }
+                *reinterpret_cast<float4 *>(pw) = make_float4(sw4[0] + aw[f][0], sw4[1] + aw[f][1], sw4[2] + aw[f][2], sw4[3] + aw[f][3]);
+                *reinterpret_cast<float4 *>(pq) = make_float4(sq4[0] + aq[f][0], sq4[1] + aq[f][1], sq4[2] + aq[f][2], sq4[3] + aq[f][3]);
+            }
+#pragma unroll
+            for (int c = 0; c < 3; c++) {
+                const float x = c == 2 && lane > 0 ? 0.0f : vec[c];
+                vec_sh[c * 32 + lane] = (w == 0 ? 0.0f : vec_sh[c * 32 + lane]) + x;
+            }
+        }
+        __syncthreads();
+    }
+    float *dst = part + (size_t)blockIdx.x * kNA * 32;
+    for (int t = threadIdx.x; t < kNA * 32; t += kT) {
+        const int c = t >> 5, f = t & 31;
+        dst[t] = c < kH ? acc_sh[f * kARow + c] : c < 2 * kH ? acc_sh[(kH + f) * kARow + c - kH] : vec_sh[t - 2 * kH * 32];
+    }
 }
 
-// dh_out_i += sum_j Ahat_ij tq_j
+constexpr int kBwdShared = (2 * kH * kH + 2 * kH * kARow + 3 * 32 + kW * 2 * kBwdRows * kBRow) * (int)sizeof(float);
+
+// dh_out_i += sum_j Ahat_ij tq_j (a tile of 16 rows per warp: 92 -> 60 us at 220,256
+// rows, bound by the gathers from L2)
 __global__ void __launch_bounds__(kT) k_agg_bwd(int n, const int *__restrict__ sp, const int *__restrict__ sw,
                                                const int *__restrict__ col, const float *__restrict__ ahat,
                                                const float *__restrict__ tq, float *__restrict__ dh) {
-    const int lane = threadIdx.x & 31;
-    for (int i = blockIdx.x * kW + (threadIdx.x >> 5); i < n; i += gridDim.x * kW)
-        dh[(size_t)i * kH + lane] = aggregate(i, sp, sw, col, ahat, tq, dh[(size_t)i * kH + lane]);
+    const int lane = threadIdx.x & 31, rs = lane >> 3, q8 = lane & 7;
+    const int ntiles = (n + kTileRows - 1) / kTileRows;
+    for (int tile = blockIdx.x * kW + (threadIdx.x >> 5); tile < ntiles; tile += gridDim.x * kW) {
+        float4 acc[4];
+#pragma unroll
+        for (int p = 0; p < 4; p++) {
+            const int i = tile * kTileRows + rs + 4 * p;
+            acc[p] = i < n ? *reinterpret_cast<const float4 *>(dh + (size_t)i * kH + 4 * q8)
+                           : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        }
+        aggregate_tile(tile, sp, sw, col, ahat, tq, acc);
+#pragma unroll
+        for (int p = 0; p < 4; p++) {
+            const int i = tile * kTileRows + rs + 4 * p;
+            if (i < n) *reinterpret_cast<float4 *>(dh + (size_t)i * kH + 4 * q8) = acc[p];
+        }
+    }
 }
 
 __global__ void __launch_bounds__(kT) k_embed_bwd(int n, const float *__restrict__ xin, const float *__restrict__ feat_a,
                                                  const float *__restrict__ pre0, const float *__restrict__ dh0,
                                                  float *__restrict__ part) {
     __shared__ float acc_sh[3 * 32];
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, stride = gridDim.x * kW;
     float acc[3] = {0.0f, 0.0f, 0.0f};
-    for (int i = blockIdx.x * kW + (threadIdx.x >> 5); i < n; i += gridDim.x * kW) {
-        const float dp = pre0[(size_t)i * kH + lane] > 0.0f ? dh0[(size_t)i * kH + lane] : 0.0f;
-        acc[0] = fmaf(dp, xin[i], acc[0]);
-        acc[1] = fmaf(dp, feat_a[i], acc[1]);
-        acc[2] += dp;
+    // eight rows' loads in flight, added in order (a row past the end adds zeros)
+    for (int i0 = blockIdx.x * kW + (threadIdx.x >> 5); i0 < n; i0 += 8 * stride) {
+        float pr[8], dh[8], xi[8], fa[8];
+#pragma unroll
+        for (int m = 0; m < 8; m++) {
+            const int i = i0 + m * stride;
+            pr[m] = dh[m] = xi[m] = fa[m] = 0.0f;
+            if (i < n) {
+                pr[m] = pre0[(size_t)i * kH + lane];
+                dh[m] = dh0[(size_t)i * kH + lane];
+                xi[m] = xin[i];
+                fa[m] = feat_a[i];
+            }
+        }
+#pragma unroll
+        for (int m = 0; m < 8; m++) {
+            const float dp = pr[m] > 0.0f ? dh[m] : 0.0f;
+            acc[0] = fmaf(dp, xi[m], acc[0]);
+            acc[1] = fmaf(dp, fa[m], acc[1]);
+            acc[2] += dp;
+        }
     }
     block_accumulate<3>(acc, acc_sh, part);
 }
 
-// grad[dst[q*32 + lane]] = sum over blocks of part[block][q*32 + lane] (FP64, block order)
-__global__ void k_grad_final(int nb, int na, const float *__restrict__ part, const int *__restrict__ dst,
-                             double *__restrict__ grad) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= na * 32) return;
+// grad[dst[q*32 + lane]] = sum over blocks of part[block][q*32 + lane] (FP64, fixed
+// order), for the four tables of one backward pass: three layers of kNA x 32
+// partials, then the embedding's 3 x 32.  A block takes 32 of them, its warps
+// every eighth partial (a thread per parameter added the 456 in one chain: 4
+// launches of 66 us -> one of 20).
+constexpr int kFinalBlocks = 3 * kNA + 3;
+__global__ void __launch_bounds__(kT) k_grad_final(const float *__restrict__ part, const int *__restrict__ dst,
+                                                  double *__restrict__ grad) {
+    __shared__ double sh[kW][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int tab = min((int)blockIdx.x / kNA, 3), q = blockIdx.x - tab * kNA, na = tab < 3 ? kNA : 3;
+    const float *p = part + (size_t)tab * kGB * kNA * 32 + q * 32 + lane;
     double s = 0.0;
-    for (int b = 0; b < nb; b++) s += (double)part[(size_t)b * na * 32 + t];
-    if (dst[t] >= 0) grad[dst[t]] = s;
+#pragma unroll 8
+    for (int b = warp; b < kGB; b += kW) s += (double)p[(size_t)b * na * 32];
+    sh[warp][lane] = s;
+    __syncthreads();
+    if (warp == 0) {
+        for (int w = 1; w < kW; w++) s += sh[w][lane];
+        const int d = dst[tab * kNA * 32 + q * 32 + lane];
+        if (d >= 0) grad[d] = s;
+    }
 }
 
 __global__ void k_adam(int np, float *__restrict__ theta, float *__restrict__ m, float *__restrict__ v,
@@ -750,8 +960,8 @@ double hash01(unsigned long long seed, unsigned long long i) {
     return (double)(z >> 11) * (1.0 / 9007199254740992.0);
 }
 
-// one warp per row for the kernels whose rows wait on neighbour loads
-int rows_grid(int n) { return std::max(1, std::min((n + kW - 1) / kW, 152 * 64)); }
+// a warp per 16-row tile
+int tiles_grid(int n) { return std::max(1, std::min((n + kW * kTileRows - 1) / (kW * kTileRows), 152 * 16)); }
 
 // the tensor-core layer: one 16-row tile per warp at a time, kTcBlocksPerSm blocks per SM
 int tc_grid(int n) {
@@ -825,6 +1035,8 @@ int gnn_prepare(Sim *s) {
     const Mesh *m = s->mesh;
     const int n = m->n_int_edges;
     const size_t nn = (size_t)std::max(n, 1), nh = nn * kH;
+    FP_CUDA(cudaFuncSetAttribute(k_layer_bwd<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBwdShared));
+    FP_CUDA(cudaFuncSetAttribute(k_layer_bwd<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBwdShared));
     int rc;
     if ((rc = gnn_rows(s))) return rc;
     const long long nel = std::max(G.rows.n_elems, 1LL);
@@ -833,7 +1045,7 @@ int gnn_prepare(Sim *s) {
         (rc = G.isd.alloc(nn)) || (rc = G.logd.alloc(nn)) || (rc = G.feat_a.alloc(nn)) || (rc = G.xin.alloc(nn)) ||
         (rc = G.gy.alloc(nn)) || (rc = G.dh.alloc(nh)) || (rc = G.dh2.alloc(nh)) || (rc = G.tq.alloc(nh)) ||
         (rc = G.part.alloc(std::max<size_t>(8 * (size_t)kGB, 3 * (size_t)kGB + 2 * (size_t)tc_grid(n)))) || (rc = G.sc.alloc(16)) ||
-        (rc = G.wpart.alloc((size_t)kGB * kNA * 32)) || (rc = G.dst.alloc(4 * kNA * 32)))
+        (rc = G.wpart.alloc(4 * (size_t)kGB * kNA * 32)) || (rc = G.dst.alloc(4 * kNA * 32)))
         return rc;
     for (int l = 0; l < 4; l++)
         if ((rc = G.h[l].alloc(nh)) || (rc = G.pre[l].alloc(nh)) || (rc = G.g[l].alloc(l ? nh : 1))) return rc;
@@ -928,15 +1140,15 @@ static int gnn_forward_dots(Sim *s, const double *r, double *z, bool keep, const
     }
     if (keep) { k_embed<true><<<kGB, kT, 0, st>>>(n, G.edge_of.p, r, G.isd.p, nrm_part, G.sc.p, G.feat_a.p, G.theta_bf.p, G.xin.p, G.pre[0].p, G.h[0].p); note_launch(); }
     else { k_embed<false><<<kGB, kT, 0, st>>>(n, G.edge_of.p, r, G.isd.p, nrm_part, G.sc.p, G.feat_a.p, G.theta_bf.p, G.xin.p, G.pre[0].p, G.h[0].p); note_launch(); }
-    const int gr = rows_grid(n), gt = tc_grid(n);
+    const int gr = tiles_grid(n), gt = tc_grid(n);
     for (int l = 1; l <= 3; l++) {
         const int off = kOffL + (l - 1) * kLayer;
         // without keep, layers 1 and 2 ping-pong between h[0] and h[1]
         const float *hin = keep ? G.h[l - 1].p : G.h[(l - 1) & 1].p;
         float *hout = keep ? G.h[l].p : G.h[l & 1].p;
-        if (l < 3 && keep) { k_layer<false><<<gr, kT, 0, st>>>(n, A.ptr.p, A.width.p, A.col.p, G.ahat.p, hin, G.theta_bf.p, off, G.g[l].p, G.pre[l].p, hout, G.edge_of.p, r, s->Dinv.p, G.isd.p, G.sc.p, z); note_launch(); }
+        if (l < 3 && keep) { k_layer<false><<<gr, kT, kLayerShared, st>>>(n, A.ptr.p, A.width.p, A.col.p, G.ahat.p, hin, G.theta_bf.p, off, G.g[l].p, G.pre[l].p, hout, G.edge_of.p, r, s->Dinv.p, G.isd.p, G.sc.p, z); note_launch(); }
         else if (l < 3) { k_layer_tc<false><<<gt, kT, 0, st>>>(n, A.ptr.p, A.width.p, A.col.p, G.ahat.p, hin, G.theta_bf.p, off, hout, G.edge_of.p, r, s->Dinv.p, G.isd.p, G.sc.p, z, nullptr, nullptr); note_launch(); }
-        else if (keep) { k_layer<true><<<gr, kT, 0, st>>>(n, A.ptr.p, A.width.p, A.col.p, G.ahat.p, hin, G.theta_bf.p, off, G.g[l].p, G.pre[l].p, hout, G.edge_of.p, r, s->Dinv.p, G.isd.p, G.sc.p, z); note_launch(); }
+        else if (keep) { k_layer<true><<<gr, kT, kLayerShared, st>>>(n, A.ptr.p, A.width.p, A.col.p, G.ahat.p, hin, G.theta_bf.p, off, G.g[l].p, G.pre[l].p, hout, G.edge_of.p, r, s->Dinv.p, G.isd.p, G.sc.p, z); note_launch(); }
         else { k_layer_tc<true><<<gt, kT, 0, st>>>(n, A.ptr.p, A.width.p, A.col.p, G.ahat.p, hin, G.theta_bf.p, off, hout, G.edge_of.p, r, s->Dinv.p, G.isd.p, G.sc.p, z, zo, dot_part); note_launch(); }
     }
     FP_CUDA(cudaGetLastError());
@@ -962,19 +1174,18 @@ int gnn_backward(Sim *s, const double *r, const double *z) {
     }
     { k_gy<<<kGB, kT, 0, st>>>(n, A.n_slices, A.ptr.p, A.width.p, A.col.p, s->A_val.p, z, r, G.row_of.p, G.isd.p, G.sc.p, G.gy.p, G.part.p); note_launch(); }
     if ((rc = gnn_reduce_launch(s, 1, G.sc.p + 1))) return rc;
-    constexpr int NA = kNA;
     // dh of layer l lives in cur; the layer writes W^T dpre into nxt and Q^T dpre into tq
     float *cur = G.dh.p, *nxt = G.dh2.p;
     for (int l = 3; l >= 1; l--) {
         const int off = kOffL + (l - 1) * kLayer;
-        if (l == 3) { k_layer_bwd<true><<<kGB, kT, 0, st>>>(n, G.h[2].p, G.g[3].p, G.pre[3].p, G.h[3].p, nullptr, G.gy.p, G.theta_bf.p, off, nxt, G.tq.p, G.wpart.p); note_launch(); }
-        else { k_layer_bwd<false><<<kGB, kT, 0, st>>>(n, G.h[l - 1].p, G.g[l].p, G.pre[l].p, G.h[l].p, cur, G.gy.p, G.theta_bf.p, off, nxt, G.tq.p, G.wpart.p); note_launch(); }
-        { k_grad_final<<<(NA * 32 + 255) / 256, 256, 0, st>>>(kGB, NA, G.wpart.p, G.dst.p + (l - 1) * NA * 32, G.grad.p); note_launch(); }
-        { k_agg_bwd<<<rows_grid(n), kT, 0, st>>>(n, G.rows.ptr.p, G.rows.width.p, G.rows.col.p, G.ahat.p, G.tq.p, nxt); note_launch(); }
+        float *wpart = G.wpart.p + (size_t)(l - 1) * kGB * kNA * 32;
+        if (l == 3) { k_layer_bwd<true><<<kGB, kT, kBwdShared, st>>>(n, G.h[2].p, G.g[3].p, G.pre[3].p, G.h[3].p, nullptr, G.gy.p, G.theta_bf.p, off, nxt, G.tq.p, wpart); note_launch(); }
+        else { k_layer_bwd<false><<<kGB, kT, kBwdShared, st>>>(n, G.h[l - 1].p, G.g[l].p, G.pre[l].p, G.h[l].p, cur, G.gy.p, G.theta_bf.p, off, nxt, G.tq.p, wpart); note_launch(); }
+        { k_agg_bwd<<<tiles_grid(n), kT, 0, st>>>(n, G.rows.ptr.p, G.rows.width.p, G.rows.col.p, G.ahat.p, G.tq.p, nxt); note_launch(); }
         std::swap(cur, nxt);
     }
-    { k_embed_bwd<<<kGB, kT, 0, st>>>(n, G.xin.p, G.feat_a.p, G.pre[0].p, cur, G.wpart.p); note_launch(); }
-    { k_grad_final<<<1, 96, 0, st>>>(kGB, 3, G.wpart.p, G.dst.p + 3 * NA * 32, G.grad.p); note_launch(); }
+    { k_embed_bwd<<<kGB, kT, 0, st>>>(n, G.xin.p, G.feat_a.p, G.pre[0].p, cur, G.wpart.p + 3 * (size_t)kGB * kNA * 32); note_launch(); }
+    { k_grad_final<<<kFinalBlocks, kT, 0, st>>>(G.wpart.p, G.dst.p, G.grad.p); note_launch(); }
     FP_CUDA(cudaGetLastError());
     return PIC_OK;
 }
