@@ -43,7 +43,8 @@ namespace {
 constexpr int kH = 32;
 constexpr int kT = 256;                 // threads per block
 constexpr int kW = kT / 32;             // warps per block
-constexpr int kGB = 456;                // blocks of the row kernels (3 per SM)
+constexpr int kGB = 456;                // blocks of the row kernels whose FP32 sums go by block (3 per SM)
+constexpr int kRowBlocks = 152 * 6;     // most blocks of the others: all rows at once on small meshes
 constexpr int kLayer = 2 * kH * kH + kH;
 constexpr int kOffU = 0, kOffV = kH, kOffC = 2 * kH, kOffL = 3 * kH;
 constexpr int kOffO = kOffL + 3 * kLayer, kOffD0 = kOffO + kH;
@@ -210,13 +211,13 @@ __device__ __forceinline__ double block_rho(const double *nrm, int n) {
 template <bool KEEP>
 __global__ void __launch_bounds__(kT) k_embed(int n, const int *__restrict__ edge, const double *__restrict__ r,
                                              const double *__restrict__ isd,
-                                             const double *__restrict__ nrm_part, double *__restrict__ nrm,
+                                             int n_part, const double *__restrict__ nrm_part, double *__restrict__ nrm,
                                              const float *__restrict__ feat_a,
                                              const unsigned short *__restrict__ th, float *__restrict__ xin,
                                              float *__restrict__ pre0, float *__restrict__ h0) {
     __shared__ double s_rho;
     const int lane = threadIdx.x & 31;
-    const double total = block_total(kGB, nrm_part);
+    const double total = block_total(n_part, nrm_part);
     if (threadIdx.x == 0) {
         s_rho = sqrt(total / n);
         if (blockIdx.x == 0) nrm[0] = total;
@@ -893,12 +894,12 @@ __global__ void __launch_bounds__(kT) k_spmv_dot(int n, int nsl, const int *__re
 
 // x += alpha p, r -= alpha q with alpha = rz / (p, q), the latter from its
 // partials; then (r, r) and (r, D^-1 r)
-__global__ void __launch_bounds__(kT) k_fpcg_xr(int n, double rz, const double *__restrict__ pq_part,
+__global__ void __launch_bounds__(kT) k_fpcg_xr(int n, double rz, int n_part, const double *__restrict__ pq_part,
                                                const double *__restrict__ p, const double *__restrict__ q,
                                                const double *__restrict__ Dinv, double *__restrict__ x,
                                                double *__restrict__ r, double *part) {
     __shared__ double s_alpha;
-    const double pq = block_total(kGB, pq_part);
+    const double pq = block_total(n_part, pq_part);
     if (threadIdx.x == 0) s_alpha = rz / pq;
     __syncthreads();
     const double alpha = s_alpha;
@@ -960,6 +961,10 @@ double hash01(unsigned long long seed, unsigned long long i) {
     return (double)(z >> 11) * (1.0 / 9007199254740992.0);
 }
 
+// a thread per row (220,256 rows: A p and (p, q) 24 -> 16 us, the embedding 17 ->
+// 14 us against 456 blocks, whose warps took two slices in turn)
+int row_blocks(int n) { return std::max(1, std::min((n + kT - 1) / kT, kRowBlocks)); }
+
 // a warp per 16-row tile
 int tiles_grid(int n) { return std::max(1, std::min((n + kW * kTileRows - 1) / (kW * kTileRows), 152 * 16)); }
 
@@ -981,9 +986,9 @@ int tc_grid(int n) {
 // ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
-static int gnn_reduce_launch(Sim *s, int nv, double *out) {
+static int gnn_reduce_launch(Sim *s, int nv, double *out, int nb = kGB) {
     GnnState &G = s->gnn;
-    { k_final_sums<<<1, 32 * nv, 0, s->stream>>>(kGB, nv, G.part.p, out); note_launch(); }
+    { k_final_sums<<<1, 32 * nv, 0, s->stream>>>(nb, nv, G.part.p, out); note_launch(); }
     FP_CUDA(cudaGetLastError());
     return PIC_OK;
 }
@@ -1044,7 +1049,7 @@ int gnn_prepare(Sim *s) {
         (rc = G.adam_v.alloc(kGnnParams)) || (rc = G.grad.alloc(kGnnParams)) || (rc = G.ahat.alloc(nel)) ||
         (rc = G.isd.alloc(nn)) || (rc = G.logd.alloc(nn)) || (rc = G.feat_a.alloc(nn)) || (rc = G.xin.alloc(nn)) ||
         (rc = G.gy.alloc(nn)) || (rc = G.dh.alloc(nh)) || (rc = G.dh2.alloc(nh)) || (rc = G.tq.alloc(nh)) ||
-        (rc = G.part.alloc(std::max<size_t>(8 * (size_t)kGB, 3 * (size_t)kGB + 2 * (size_t)tc_grid(n)))) || (rc = G.sc.alloc(16)) ||
+        (rc = G.part.alloc(std::max<size_t>(8 * (size_t)kGB, 3 * (size_t)kRowBlocks + 2 * (size_t)tc_grid(n)))) || (rc = G.sc.alloc(16)) ||
         (rc = G.wpart.alloc(4 * (size_t)kGB * kNA * 32)) || (rc = G.dst.alloc(4 * kNA * 32)))
         return rc;
     for (int l = 0; l < 4; l++)
@@ -1125,9 +1130,9 @@ int gnn_get_weights(Sim *s, float *w, long long np) {
 
 // z = P(r) on interior edges (internal order, device arrays); with `keep`
 // the activations a backward pass needs are stored.  G.sc[0] receives n rho^2,
-// from the kGB partials at nrm_part (NULL: formed here).  With zo, the partials
+// from the n_part partials at nrm_part (NULL: formed here).  With zo, the partials
 // of (r, z) and (r, zo) go to dot_part, tc_grid(n) each.
-static int gnn_forward_dots(Sim *s, const double *r, double *z, bool keep, const double *nrm_part, const double *zo,
+static int gnn_forward_dots(Sim *s, const double *r, double *z, bool keep, int n_part, const double *nrm_part, const double *zo,
                             double *dot_part) {
     GnnState &G = s->gnn;
     const int n = s->mesh->n_int_edges;
@@ -1137,9 +1142,11 @@ static int gnn_forward_dots(Sim *s, const double *r, double *z, bool keep, const
     if (!nrm_part) {
         { k_rnorm<<<kGB, kT, 0, st>>>(n, G.edge_of.p, r, s->Dinv.p, G.part.p); note_launch(); }
         nrm_part = G.part.p;
+        n_part = kGB;
     }
-    if (keep) { k_embed<true><<<kGB, kT, 0, st>>>(n, G.edge_of.p, r, G.isd.p, nrm_part, G.sc.p, G.feat_a.p, G.theta_bf.p, G.xin.p, G.pre[0].p, G.h[0].p); note_launch(); }
-    else { k_embed<false><<<kGB, kT, 0, st>>>(n, G.edge_of.p, r, G.isd.p, nrm_part, G.sc.p, G.feat_a.p, G.theta_bf.p, G.xin.p, G.pre[0].p, G.h[0].p); note_launch(); }
+    const int rb = row_blocks(n);
+    if (keep) { k_embed<true><<<rb, kT, 0, st>>>(n, G.edge_of.p, r, G.isd.p, n_part, nrm_part, G.sc.p, G.feat_a.p, G.theta_bf.p, G.xin.p, G.pre[0].p, G.h[0].p); note_launch(); }
+    else { k_embed<false><<<rb, kT, 0, st>>>(n, G.edge_of.p, r, G.isd.p, n_part, nrm_part, G.sc.p, G.feat_a.p, G.theta_bf.p, G.xin.p, G.pre[0].p, G.h[0].p); note_launch(); }
     const int gr = tiles_grid(n), gt = tc_grid(n);
     for (int l = 1; l <= 3; l++) {
         const int off = kOffL + (l - 1) * kLayer;
@@ -1156,7 +1163,7 @@ static int gnn_forward_dots(Sim *s, const double *r, double *z, bool keep, const
 }
 
 int gnn_forward(Sim *s, const double *r, double *z, bool keep) {
-    return gnn_forward_dots(s, r, z, keep, nullptr, nullptr, nullptr);
+    return gnn_forward_dots(s, r, z, keep, 0, nullptr, nullptr, nullptr);
 }
 
 // loss and dL/dtheta (into G.grad, device) for residual r; loss -> G.sc[1]
@@ -1172,8 +1179,8 @@ int gnn_backward(Sim *s, const double *r, const double *z) {
         FP_CUDA(cudaMemsetAsync(G.sc.p + 1, 0, sizeof(double), st));
         return PIC_OK;
     }
-    { k_gy<<<kGB, kT, 0, st>>>(n, A.n_slices, A.ptr.p, A.width.p, A.col.p, s->A_val.p, z, r, G.row_of.p, G.isd.p, G.sc.p, G.gy.p, G.part.p); note_launch(); }
-    if ((rc = gnn_reduce_launch(s, 1, G.sc.p + 1))) return rc;
+    { k_gy<<<row_blocks(n), kT, 0, st>>>(n, A.n_slices, A.ptr.p, A.width.p, A.col.p, s->A_val.p, z, r, G.row_of.p, G.isd.p, G.sc.p, G.gy.p, G.part.p); note_launch(); }
+    if ((rc = gnn_reduce_launch(s, 1, G.sc.p + 1, row_blocks(n)))) return rc;
     // dh of layer l lives in cur; the layer writes W^T dpre into nxt and Q^T dpre into tq
     float *cur = G.dh.p, *nxt = G.dh2.p;
     for (int l = 3; l >= 1; l--) {
@@ -1270,7 +1277,7 @@ int fpcg_newmark(Sim *s, int *iters_out) {
         }
         return gnn_forward(s, rr, zz, false);
     };
-    { k_resid<<<kGB, kT, 0, st>>>(n, A.n_slices, A.ptr.p, A.width.p, A.col.p, s->A_val.p, b, x, r); note_launch(); }
+    { k_resid<<<row_blocks(n), kT, 0, st>>>(n, A.n_slices, A.ptr.p, A.width.p, A.col.p, s->A_val.p, b, x, r); note_launch(); }
     double bb_rr[2];
     if ((rc = dots(b, b, r, r, bb_rr))) return rc;
     const double bb = bb_rr[0], tol2 = s->cfg.cg_tol * s->cfg.cg_tol;
@@ -1300,16 +1307,17 @@ int fpcg_newmark(Sim *s, int *iters_out) {
         }
         // x += alpha p, r -= alpha A p, alpha = r.z / p.A p: partial sums go
         // from kernel to kernel, and the host waits once an iteration
-        double *pq_part = G.part.p, *rr_part = G.part.p + kGB, *dot_part = G.part.p + 3 * kGB;
-        { k_spmv_dot<<<kGB, kT, 0, st>>>(n, A.n_slices, A.ptr.p, A.width.p, A.col.p, s->A_val.p, p, q, pq_part); note_launch(); }
-        { k_fpcg_xr<<<kGB, kT, 0, st>>>(n, rzo, pq_part, p, q, s->Dinv.p, x, r, rr_part); note_launch(); }
+        const int rb = row_blocks(n);
+        double *pq_part = G.part.p, *rr_part = pq_part + rb, *dot_part = rr_part + 2 * rb;
+        { k_spmv_dot<<<rb, kT, 0, st>>>(n, A.n_slices, A.ptr.p, A.width.p, A.col.p, s->A_val.p, p, q, pq_part); note_launch(); }
+        { k_fpcg_xr<<<rb, kT, 0, st>>>(n, rzo, rb, pq_part, p, q, s->Dinv.p, x, r, rr_part); note_launch(); }
         std::swap(z, zo);
         double d1[2], d2[2];
         if (jac) {
             if ((rc = precond(r, z, jac)) || (rc = dots(r, z, r, zo, d1)) || (rc = dots(r, r, nullptr, nullptr, d2))) return rc;
         } else {
-            if ((rc = gnn_forward_dots(s, r, z, false, rr_part + kGB, zo, dot_part))) return rc;
-            { k_fpcg_sums<<<1, 96, 0, st>>>(kGB, rr_part, tc_grid(n), dot_part, G.sc.p + 4); note_launch(); }
+            if ((rc = gnn_forward_dots(s, r, z, false, rb, rr_part + rb, zo, dot_part))) return rc;
+            { k_fpcg_sums<<<1, 96, 0, st>>>(rb, rr_part, tc_grid(n), dot_part, G.sc.p + 4); note_launch(); }
             FP_CUDA(cudaGetLastError());
             double v[3];
             FP_CUDA(cudaMemcpyAsync(v, G.sc.p + 4, sizeof(v), cudaMemcpyDeviceToHost, st));
