@@ -44,21 +44,21 @@ FALLBACK_HBM_GBS = 6800.0
 CLOCK_LOG = None   # --clock-log: where the clock samples of the timed region go ({gpu}: the GPU index)
 FP64_NOMINAL_TFLOPS = 1.25   # GB300 dense FP64 (non-tensor) nominal rate
 # DRAM bytes over algorithmic bytes of the MIXED Newmark launch
-# (k_pcg_persistent<1>), from one ncu capture of that kernel (its current code)
-# on the 64^3 plasma ball: 15.664 GB (dram__bytes_read.sum +
+# (k_pcg_persistent<1, 0>), from one ncu capture of that kernel (its current
+# code) on the 64^3 plasma ball: 10.374 GB (dram__bytes_read.sum +
 # dram__bytes_write.sum) for 60 FP32 + 2 FP64 iterations whose algorithmic
-# bytes are 19.938 GB (below 1: with the matrix loaded evict-first, the
+# bytes are 14.440 GB (below 1: with the matrix loaded evict-first, the
 # vectors written each iteration stay in L2).  The FP64 Newmark form has no
 # capture of its current code: its traffic is reported as null.
-TRAFFIC_RATIO_MIXED = (15.561853 + 0.102376) / 19.937848
+TRAFFIC_RATIO_MIXED = (10.271964 + 0.101604) / 14.439829
 # DRAM bytes of one MIXED push launch (k_push_mixed<0>) on the 64^3 plasma-ball
 # mesh with 4M + 4M particles, from one ncu capture of the current kernel:
-# 0.408 + 0.336 GB (93 B per particle, per-tet bytes included); scaled to a
+# 0.445 + 0.352 GB (100 B per particle, per-tet bytes included); scaled to a
 # launch by the particles it pushes
-PUSH_TRAFFIC_SMALL = (0.408e9 + 0.336e9, 8_000_000)
-# Warp instructions of the same capture (smsp__inst_executed.sum): 245M for the
+PUSH_TRAFFIC_SMALL = (0.445e9 + 0.352e9, 8_000_000)
+# Warp instructions of the same capture (smsp__inst_executed.sum): 231M for the
 # 8M particles, the push's binding resource being instruction issue
-PUSH_WARP_INST_SMALL = (245.0e6, 8_000_000)
+PUSH_WARP_INST_SMALL = (231.0e6, 8_000_000)
 SCHEDULERS_PER_SM = 4   # warp schedulers per SM, one warp instruction issued per cycle each
 TRAFFIC_RATIO_PLAIN = None
 
@@ -296,10 +296,11 @@ def issue_roofline(n_particles: float, avg_ms: float, sms: int, sm_mhz: float) -
 
 def pcg_iter_bytes(n_rows: int, nnz: int) -> float:
     """Algorithmic bytes of one iteration of the persistent Chronopoulos-Gear
-    PCG on SELL-32: values + columns once (12 B/nnz) and two slice headers per
-    32 rows; the SpMV reads u once and writes w; the vector phase reads u, w,
-    p, s, x, r, D^-1 and writes p, s, x, r, u (14 vector passes of 8 B)."""
-    return 12.0 * nnz + 8.0 * (n_rows + 31) / 32 + 8.0 * 14 * n_rows
+    PCG: values + one-byte columns once (9 B/nnz; the benchmark meshes have a
+    regular node numbering) and two slice headers per 32 rows; the SpMV reads
+    u once and writes w; the vector phase reads u, w, p, s, x, r, D^-1 and
+    writes p, s, x, r, u (14 vector passes of 8 B)."""
+    return 9.0 * nnz + 8.0 * (n_rows + 31) / 32 + 8.0 * 14 * n_rows
 
 
 def pcg_iter_flops(n_rows: int, nnz: int) -> float:
@@ -310,14 +311,14 @@ def pcg_iter_flops(n_rows: int, nnz: int) -> float:
 
 def refine_bytes(n_rows: int, nnz: int, inner_iters: float, outer: float) -> float:
     """Algorithmic bytes of one MIXED Newmark solve (FP64 refinement with FP32
-    correction solves on the diagonally scaled system): per FP32 iteration 8 B
-    per nonzero (FP32 value + column) + 11 vector passes of 4 B per row (SpMV:
-    r read, w written; vector phase: w, p, s, x, r read, p, s, x, r written);
-    per refinement step one FP64 residual (12 B per nonzero, b read, x
+    correction solves on the diagonally scaled system): per FP32 iteration 5 B
+    per nonzero (FP32 value + one-byte column) + 11 vector passes of 4 B per row
+    (SpMV: r read, w written; vector phase: w, p, s, x, r read, p, s, x, r
+    written); per refinement step one FP64 residual (9 B per nonzero, b read, x
     gathered, r in FP32 written: 20 B per row) and the update x += d (20 B per
     row); plus the final residual check."""
-    inner = inner_iters * (8.0 * nnz + 4.0 * 11 * n_rows)
-    return inner + (outer + 1) * (12.0 * nnz + 20.0 * n_rows) + outer * 20.0 * n_rows
+    inner = inner_iters * (5.0 * nnz + 4.0 * 11 * n_rows)
+    return inner + (outer + 1) * (9.0 * nnz + 20.0 * n_rows) + outer * 20.0 * n_rows
 
 
 def beam_leg(F, torch, stream, args):
@@ -442,7 +443,7 @@ def batched_leg(F, torch, args):
             "tuned": {"newmark": {"blocks_per_sm": info["solver_blocks_per_sm"], "build": info["solver_build"]},
                       "completion": {"blocks_per_sm": info["completion_blocks_per_sm"],
                                      "build": info["completion_build"]},
-                      "candidates": "blocks/SM 2, 3, 4 (64-register build), 2, 3 (80-register), 5, 6 (40-register), 7, 8 (32-register)",
+                      "candidates": "blocks/SM 2, 3, 4 (64-register build), 2, 3 (80-register); 5 to 8 stand for four blocks of the first",
                       "tune_newmark_ms": [round(v, 3) for v in info["tune_newmark_ms"]],
                       "tune_completion_ms": [round(v, 3) for v in info["tune_completion_ms"]]}}
 
@@ -756,13 +757,13 @@ def gpu_arm(args):
         if outer > 0:
             # MIXED: FP64 refinement steps (the last solve's count) around FP32 correction iterations
             kernel = ("k_pcg_persistent (Newmark: FP64 refinement, FP32 Chronopoulos-Gear corrections, "
-                      "SELL-32)")
+                      "streamed records)")
             alg = refine_bytes(mesh.n_int_edges, nnz_A, iters_per_launch, outer)
             traffic = alg * TRAFFIC_RATIO_MIXED if TRAFFIC_RATIO_MIXED else None
             fp64 = {"note": "the FP32 correction iterations issue no FP64 arithmetic", "outer_steps": outer,
                     "fp32_iters_per_launch": iters_per_launch}
         else:
-            kernel = "k_pcg_persistent (Newmark PCG, Chronopoulos-Gear, SELL-32)"
+            kernel = "k_pcg_persistent (Newmark PCG, Chronopoulos-Gear, streamed records)"
             alg = iters_per_launch * pcg_iter_bytes(mesh.n_int_edges, nnz_A)
             traffic = alg * TRAFFIC_RATIO_PLAIN if TRAFFIC_RATIO_PLAIN else None
             flops = iters_per_launch * pcg_iter_flops(mesh.n_int_edges, nnz_A)
