@@ -19,14 +19,12 @@
 //   L = (z^T A z - 2 z^T r) / (r^T D^-1 r),
 // the A-norm error of z against A^-1 r up to a constant (no solve needed).
 //
-// Layout: activations row-major (32 floats = 128 B per row).  Training: one
-// warp per row, lane f = feature f, so a neighbour's features are one
-// coalesced load; the 32x32 products broadcast the row's features with
-// shuffles and read the weights from shared memory (transposed where that
-// avoids bank conflicts).  A preconditioner application runs its layers on
-// the tensor cores instead (k_layer_tc: 16-row tiles, TF32 products of split
-// activations), since the training layout spends most of its issue slots on
-// shuffles and shared loads rather than on the data.  Every reduction (weight gradients, rho, the loss, the PCG dot
+// Layout: activations row-major (32 floats = 128 B per row), rows in an order
+// of their own (by row length, then canonical edge).  Both passes work on tiles
+// of rows in shared memory and gather four whole feature rows an instruction.
+// Training keeps FP32 multiply-adds and one summation order; a preconditioner
+// application runs its layers on the tensor cores (k_layer_tc: TF32 products of split
+// activations).  Every reduction (weight gradients, rho, the loss, the PCG dot
 // products) uses per-block partials combined in a fixed order: results do not
 // depend on scheduling.
 #include <cuda_bf16.h>

@@ -260,9 +260,6 @@ __global__ void __launch_bounds__(kThreads) k_gc_w_sell(int n, int n_slices, con
     }
 }
 
-// r = b - A x, z = D^-1 r, p = z; rz, rr, bb, max|r|
-// p = z + beta p_old (on the fly for the neighbours), q = A p, pq: the SpMV
-// of the Newmark PCG
 // What a step's diagnostics read from the fields, in one launch: over the
 // edges the true residual of the Newmark system and M e (kept for the node
 // diagnostics), e^T M e; over the tets max |D b|; over the faces b^T H b; the

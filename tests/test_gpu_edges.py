@@ -90,3 +90,34 @@ def test_electrostatic_sizes(F, cells, shuffled):                               
     torch.cuda.synchronize()
     ref = sim.field("PHI")
     assert rel_err(phi.cpu().numpy(), ref) <= 2e-11
+
+
+# 26 rows (two tiles, one of 10 rows; every backward batch past the end), 117,
+# 665 rows, regular and shuffled numberings; the tolerances of the network's
+# comparison with its oracle (FP32 sums)
+@pytest.mark.parametrize("cells,shuffled", [(2, False), (3, True), (5, False), (5, True)])
+def test_network_sizes(F, oracle_lib, cells, shuffled):                                         # noqa: F811
+    from oracle import gnn_oracle as GO
+    from test_gpu_gnn import random_weights
+    wl = W.thermal_plasma_cube(n_cells=cells, n_particles=500, seed=61)
+    if shuffled:
+        wl = renumbered(wl, 62)
+    dt = 2 * DT_CFL_6 * 6 / cells
+    sim = F.sim_from_workload(wl, dt, precision="plain")
+    A, ids = GO.interior_system(oracle_lib.OracleMesh(wl.mesh.xyz, wl.mesh.tets), dt)
+    w = random_weights(63)
+    sim.gnn_set_weights(w)
+    r = np.zeros(sim.mesh.n_edges)
+    r[ids] = np.random.default_rng(64).normal(size=ids.size)
+    net = GO.EdgeNet(A)
+    z, (zo, _) = sim.gnn_apply(r), net.forward(r[ids], GO.bf16(w))
+    assert np.abs(z[ids] - zo).max() <= 1e-5 * np.abs(zo).max()
+    L, g = sim.gnn_loss_grad(r)
+    Lo, go, _ = net.loss_and_grad(r[ids], GO.bf16(w))
+    assert L == pytest.approx(Lo, rel=1e-5, abs=1e-6)
+    for name, (o, s) in GO.OFFSETS.items():
+        if name == "_size":
+            continue
+        sl = slice(o, o + int(np.prod(s)))
+        scale = max(np.abs(go[sl]).max(), 1e-3 * np.abs(go).max())
+        assert np.abs(g[sl] - go[sl]).max() <= 1e-3 * scale, name
