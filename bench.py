@@ -58,7 +58,10 @@ TRAFFIC_RATIO_MIXED = (10.271964 + 0.101604) / 14.439829
 PUSH_TRAFFIC_SMALL = (0.445e9 + 0.352e9, 8_000_000)
 # Warp instructions of the same capture (smsp__inst_executed.sum): 231M for the
 # 8M particles, the push's binding resource being instruction issue
-PUSH_WARP_INST_SMALL = (231.0e6, 8_000_000)
+PUSH_WARP_INST = (231.0e6, 8_000_000)
+# ... and of the launch issue_roofline's formula was checked on (245M, 0.434 ms,
+# ncu issue active 45.5%; the push that reduced block by block), its default
+PUSH_WARP_INST_SMALL = (245.0e6, 8_000_000)
 SCHEDULERS_PER_SM = 4   # warp schedulers per SM, one warp instruction issued per cycle each
 TRAFFIC_RATIO_PLAIN = None
 
@@ -277,12 +280,13 @@ def measured_sm_mhz() -> float:
         return 2070.0
 
 
-def issue_roofline(n_particles: float, avg_ms: float, sms: int, sm_mhz: float) -> dict:
+def issue_roofline(n_particles: float, avg_ms: float, sms: int, sm_mhz: float,
+                   counted: tuple = PUSH_WARP_INST_SMALL) -> dict:
     """The push against its binding resource, instruction issue: the warp
     instructions of one launch (the ncu count per particle of the captured
     launch times the particles pushed) over its duration, against every
     scheduler issuing one warp instruction per cycle at the given SM clock."""
-    per_particle = PUSH_WARP_INST_SMALL[0] / PUSH_WARP_INST_SMALL[1]
+    per_particle = counted[0] / counted[1]
     inst = per_particle * n_particles
     achieved = inst / (avg_ms / 1e3)
     peak = float(sms) * SCHEDULERS_PER_SM * sm_mhz * 1e6
@@ -791,7 +795,7 @@ def gpu_arm(args):
                                        "scaled by the particles pushed",
                      "issue": issue_roofline(alive_m, push_avg,
                                              torch.cuda.get_device_properties(device).multi_processor_count,
-                                             measured_sm_mhz())
+                                             measured_sm_mhz(), PUSH_WARP_INST)
                      if args.cells == 64 and args.workload == "plasma_ball" else None}
 
     # ---- learned preconditioner on the same workload ----
