@@ -408,7 +408,7 @@ typedef struct {
     int32_t pad_;
     /* tuning times (ms) per candidate: blocks per SM 2, 3, 4 with build 0;
      * 2, 3 with build 1; 5, 6 with build 2 and 7, 8 with build 3 (the time of
- * four blocks of build 0, which they stand for).  -1: not
+     * four blocks of build 0, which they stand for).  -1: not
      * timed (the choice came from an earlier batch of the same shape in this
      * process, or, for the completion of a batch with multigrid members, the
      * candidate's build does not exist for the combined launch) */
