@@ -41,7 +41,7 @@ def _flags(src: str) -> List[str]:
 def _stale(obj: str, src: str) -> bool:
     if not os.path.exists(obj):
         return True
-    deps = [src] + [os.path.join(CSRC, h) for h in os.listdir(CSRC) if h.endswith(".h")]
+    deps = [src] + [os.path.join(CSRC, h) for h in os.listdir(CSRC) if h.endswith((".h", ".cuh"))]
     deps.append(os.path.join(INCLUDE, "fempic.h"))
     return os.path.getmtime(obj) < max(os.path.getmtime(d) for d in deps)
 
