@@ -529,10 +529,10 @@ constexpr int kMaxPcgBlocks = 4 * kThreads;    // most blocks of one solve
 // PCG and anything on wide records, and the refinement on narrow ones
 template <bool REFINE, bool WIDE>
 struct PcgShape {
-    // (refinement, FP32 gathers in flight: 512, 768, 1024 threads 3.50, 2.79,
-    // 2.88 ms per Newmark solve of the 64^3 plasma ball, 128, 80, 64
-    // registers; FP64, bound by the FP64 pipes: 512 and 768 threads 1.75 and
-    // 1.87 ms on 40^3)
+    // (refinement, bound by the gathers that its warps have in flight: 512,
+    // 768, 1024 threads 3.50, 2.79, 2.88 ms per Newmark solve of the 64^3
+    // plasma ball, 128, 80, 64 registers; FP64, bound by the FP64 pipes: 512
+    // and 768 threads 1.75 and 1.87 ms on 40^3)
     static constexpr int threads = REFINE && !WIDE ? 768 : 512;
     static constexpr int ring = REFINE && !WIDE ? 2 * Record<double, false>::bytes : 8192;
 };
@@ -782,7 +782,7 @@ extern __shared__ __align__(128) unsigned char s_ring[];   // dynamic shared mem
 template <bool WIDE, int T, int RING>
 struct SolveCtx {
     template <typename V>
-    using S = Stream<V, WIDE, RING, false>;
+    using S = Stream<V, WIDE, RING>;
     using S64 = S<double>;
     using S32 = S<float>;
     const PcgArgs *a;
@@ -1005,7 +1005,7 @@ __device__ __forceinline__ void pcg_body(const PcgArgs &a, const int nb, const i
                                          unsigned long long *shm) {
     constexpr int W = T / 32;
     __shared__ unsigned short s_width[kSmemSlices];
-    __shared__ __align__(8) unsigned long long s_bars[W][kMaxStages];
+    __shared__ __align__(8) unsigned long long s_bars[W][kStreamBars];
     __shared__ CgScalars scal;
     __shared__ int s_range[2];
     struct Refine {

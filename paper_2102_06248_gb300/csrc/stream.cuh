@@ -83,13 +83,27 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_
         : "memory");
 }
 
+__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+
 constexpr int kMaxStages = 8;
-constexpr int kCopySpin = 1 << 20;   // polls of one copy's barrier before the solve gives up (each poll suspends for a while)
+constexpr int kStreamBars = 2 * kMaxStages;   // mbarriers of a warp: per stage one for its copy, one for its release
+constexpr int kCopySpin = 1 << 20;   // polls of one mbarrier before the solve gives up (each poll suspends for a while)
+
+// polls until the phase of that parity has completed; false when the bound ends the wait
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
+    for (int k = 0; k < kCopySpin; k++)
+        if (mbar_try(bar, parity)) return true;
+    return false;
+}
 
 // A warp's part of the matrix and its ring.  Copy number q of a stream (counted
-// from begin) lands in stage q % stages and completes that stage's mbarrier
-// phase (q / stages) & 1; `stage` and `parity` track the next one to consume,
-// `inflight` the copies issued and not yet consumed.
+// from begin) lands in stage q % stages and completes phase q / stages of that
+// stage's first mbarrier; once the 32 lanes have read the stage they complete
+// the same phase of its second mbarrier, and the next copy into it waits for
+// that.  `stage` and `parity` track the next copy to consume, `inflight` the
+// copies issued and not yet consumed.
 struct WarpStream {
     uint32_t ring, bars;         // shared addresses of the warp's ring and its mbarriers
     int s0, s1;                  // slices [s0, s1)
@@ -101,24 +115,26 @@ struct WarpStream {
     uint64_t policy;
 };
 
-// One record type streamed through a warp's ring of RING bytes.  DEEP: the
-// gathers of a record are in flight while the one before it is summed (twice
-// the registers; FP32 products, which wait on their gathers.  FP64 ones wait
-// on the FP64 pipe).
-template <typename V, bool WIDE, int RING, bool DEEP>
+// One record type streamed through a warp's ring of RING bytes.
+template <typename V, bool WIDE, int RING>
 struct Stream {
     using Rec = Record<V, WIDE>;
     static constexpr int stages = RING / Rec::bytes < kMaxStages ? RING / Rec::bytes : kMaxStages;
     static_assert(stages >= 2, "a ring holds at least two records");
 
-    // never: 0, formed from what the stage's last use loaded (see pass)
-    __device__ static void issue(WarpStream &w, const unsigned char *recs, int stage, uint32_t never) {
-        if ((threadIdx.x & 31) == 0) {
-            const uint32_t bar = w.bars + 8u * stage + 16u * never;
-            mbar_expect(bar, Rec::bytes);
+    __device__ static uint32_t full(const WarpStream &w, int stage) { return w.bars + 8u * stage; }
+    __device__ static uint32_t empty(const WarpStream &w, int stage) { return w.bars + 8u * (kMaxStages + stage); }
+
+    // lane 0 fetches the next record into `stage`; `reused`: once the lanes have
+    // released what the stage held (the phase of `parity`).  A release that does
+    // not come within the bound leaves the copy out, and its consumer gives up.
+    __device__ static void issue(WarpStream &w, const unsigned char *recs, int stage, bool reused, uint32_t parity) {
+        if ((threadIdx.x & 31) == 0 && (!reused || mbar_wait(empty(w, stage), parity))) {
+            mbar_expect(full(w, stage), Rec::bytes);
             bulk_load(w.ring + (uint32_t)stage * Rec::bytes, recs + (size_t)(w.rec0 + w.next) * Rec::bytes, Rec::bytes,
-                      bar, w.policy);
+                      full(w, stage), w.policy);
         }
+        __syncwarp();
         w.next = w.next + 1 == w.nrec ? 0 : w.next + 1;
         w.inflight++;
     }
@@ -129,18 +145,19 @@ struct Stream {
         w.parity = 0;
         if (w.nrec == 0) return;
         if ((threadIdx.x & 31) == 0) {
-            for (int k = 0; k < stages; k++) mbar_init(w.bars + 8u * k, 1);
+            for (int k = 0; k < stages; k++) {
+                mbar_init(full(w, k), 1);
+                mbar_init(empty(w, k), 32);
+            }
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         }
         __syncwarp();
-        for (int k = 0; k < stages && k < most; k++) issue(w, recs, k, 0);
+        for (int k = 0; k < stages && k < most; k++) issue(w, recs, k, false, 0);
     }
+    // the copy of the next stage to consume has landed (the same answer in every lane)
     __device__ static bool wait(const WarpStream &w) {
-        const uint32_t bar = w.bars + 8u * w.stage;
-        for (int k = 0; k < kCopySpin; k++)
-            if (mbar_try(bar, w.parity)) return true;
-        return false;
+        return __all_sync(0xFFFFFFFFu, mbar_wait(full(w, w.stage), w.parity));
     }
     __device__ static void step(WarpStream &w) {
         w.inflight--;
@@ -160,7 +177,10 @@ struct Stream {
         }
         __syncwarp();
         if ((threadIdx.x & 31) == 0)
-            for (int k = 0; k < stages; k++) asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(w.bars + 8u * k) : "memory");
+            for (int k = 0; k < stages; k++) {
+                asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(full(w, k)) : "memory");
+                asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(empty(w, k)) : "memory");
+            }
         __syncwarp();
         return ok;
     }
@@ -169,8 +189,13 @@ struct Stream {
     struct Frag {
         V a[kCols], g[kCols];
     };
-    // loads the record of the next stage and starts its gathers
-    __device__ static void fetch(const WarpStream &w, const V *v, Frag &f) {
+    // Loads the record of the next stage, releases the stage if a copy will
+    // follow into it, and starts the record's gathers.  The release: every lane
+    // orders its reads before the async proxy's writes and arrives on the
+    // stage's second mbarrier, which lane 0 waits for before it issues the copy
+    // (loads merely issued were seen overtaken by the copy).  It comes before
+    // the gathers, so that lane 0 finds it complete.
+    __device__ static void fetch(const WarpStream &w, const V *v, bool follows, Frag &f) {
         const int lane = threadIdx.x & 31;
         const uint32_t st = w.ring + (uint32_t)w.stage * Rec::bytes;
         int col[kCols];
@@ -207,26 +232,12 @@ struct Stream {
                 col[4 + j] += lane + (int)((hi >> (8 * j)) & 255u);
             }
         }
+        if (follows) {
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            mbar_arrive(empty(w, w.stage));
+        }
 #pragma unroll
         for (int j = 0; j < kCols; j++) f.g[j] = v[col[j]];
-    }
-    // 0, formed from a value of each load of the record (a comparison that
-    // does not hold, which the compiler does not know).  A stage may take its
-    // next copy only when its loads have delivered: one that was merely issued
-    // can be overtaken by the copy's write when gathers hold up the load pipe
-    // (seen as wrong sums once little L1 was left).  A copy whose operands
-    // depend on this value waits for them.
-    __device__ static uint32_t delivered(const Frag &f) {
-        uint32_t seen = 0, same = 0xFFFFFFFFu;
-#pragma unroll
-        for (int j = 0; j < kCols; j += 16 / (int)sizeof(V)) {
-            uint32_t b;
-            if constexpr (sizeof(V) == 4) b = __float_as_uint(f.a[j]);
-            else b = (uint32_t)__double2hiint(f.a[j]);
-            seen |= b;
-            same &= b;
-        }
-        return (uint32_t)(seen == 0xFFC0DE5Au) & (uint32_t)(same == 0x7FC0DE5Au);
     }
     // One product over the warp's rows: fin(i, sum_j A_ij v_j, v_i), the sum in
     // column order.  width(sl): entries of a row of slice sl.  With `more` the
@@ -275,48 +286,21 @@ struct Stream {
                 }
             }
         };
-        // the record c in `f` came from `stage`, which takes the next copy
-        auto release = [&](int c, int stage, const Frag &f) {
-            const uint32_t never = delivered(f);
-            __syncwarp();
-            if (more || c + stages < w.nrec) issue(w, recs, stage, never);
-        };
-        auto skip_first = [&](Frag &f) {
-#pragma unroll
-            for (int j = 0; j < kCols; j++)
-                if (j < w.skip) f.a[j] = 0;
-        };
-        Frag f0;
-        if constexpr (!DEEP) {
-            for (int c = 0; c < w.nrec; c++) {
-                if (!wait(w)) return false;
-                fetch(w, v, f0);
-                const int stage = w.stage;
-                step(w);
-                release(c, stage, f0);
-                if (c == 0) skip_first(f0);
-                sum(f0);
-            }
-        } else {
-            Frag f1;
+        Frag f;
+        for (int c = 0; c < w.nrec; c++) {
             if (!wait(w)) return false;
-            fetch(w, v, f0);
-            auto turn = [&](int c, Frag &cur, Frag &nxt) -> bool {
-                const int stage = w.stage;
-                step(w);
-                if (c + 1 < w.nrec) {
-                    if (!wait(w)) return false;
-                    fetch(w, v, nxt);
-                }
-                release(c, stage, cur);
-                if (c == 0) skip_first(cur);
-                sum(cur);
-                return true;
-            };
-            for (int c = 0; c < w.nrec; c += 2) {
-                if (!turn(c, f0, f1)) return false;
-                if (c + 1 < w.nrec && !turn(c + 1, f1, f0)) return false;
+            const bool follows = more || c + stages < w.nrec;
+            const int stage = w.stage;
+            const uint32_t parity = w.parity;
+            fetch(w, v, follows, f);
+            step(w);
+            if (follows) issue(w, recs, stage, true, parity);
+            if (c == 0) {
+#pragma unroll
+                for (int j = 0; j < kCols; j++)
+                    if (j < w.skip) f.a[j] = 0;
             }
+            sum(f);
         }
         return true;
     }
