@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstring>
 #include <mutex>
@@ -1161,9 +1162,16 @@ __device__ __forceinline__ void pcg_body(const PcgArgs &a, const int nb, const i
 //    the blocks per iteration, and n does not wait for the scalars, so the
 //    product runs while four more warps of the block add the partials and form
 //    the scalars;
-//  * the iterates are those of PCG up to rounding, which the longer recurrence
-//    amplifies: the solution is checked against b - A x and continued from,
-//    twice at most, if it misses the stopping rule by more than 2%.
+//  * its rounding errors grow with the condition number where those of the
+//    recurrence with two meetings (cg_core) do not: at 24^3 cells of sides
+//    1 : 10 : 100 and a tolerance of 1e-13, or at 300 times the explicit time
+//    step and 1e-10, its residual stops falling above the tolerance or parts from
+//    b - A x.  So it ends when its residual has not fallen for kSmallStall
+//    iterations (13 in a row at most in systems where it converged), a solution
+//    that it ends with counts once b - A x itself meets the rule, and otherwise the
+//    recurrence with two meetings goes on from there, with max_iters
+//    iterations of its own.  Tolerances below kSmallTol2 (absolute ones
+//    against the largest entry of b) take that one from the start.
 // Per iteration, streamed form and this: 20^3 (52,460 rows) 12.2 and 7.5 us,
 // 16^3 (26,416 rows) 10.7 and 7.1 us, 6^3 (1,206 rows) 9.6 and 6.2 us.
 // ---------------------------------------------------------------------------
@@ -1171,7 +1179,8 @@ constexpr int kSmallWarps = 12;               // slices of a block; four more wa
 constexpr int kSmallThreads = 32 * (kSmallWarps + 4);
 constexpr int kSmallWidth = 32;               // columns of a slice held in shared memory
 constexpr int kSmallSlice = kSmallWidth * 32 * 12;
-constexpr int kSmallRestarts = 2;
+constexpr int kSmallStall = 32;
+constexpr double kSmallAim2 = 0.96;           // the pipelined recurrence aims 2% below the tolerance (squared)
 constexpr double kSmallTol2 = 0.9e-26;        // smallest relative tolerance (squared) of the pipelined recurrence
 constexpr int kSmallBlocks = 160;             // partials a warp adds with five loads a lane
 
@@ -1182,8 +1191,8 @@ __device__ __forceinline__ void small_body(const PcgArgs &a, const int nb, const
     __shared__ double res[4];
     struct Scalars {
         double alpha, ralpha, rgamma, beta;   // in this order (lanes 0..3)
-        double gamma, rr, bb, stop, abs_inf, tol2;
-        int iters, fresh, done, failed, ok, checked;
+        double gamma, rr, bb, stop, abs_inf, tol2, best;
+        int iters, limit, since, fresh, plain, done, failed, ok;
     };
     __shared__ Scalars sc;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1215,7 +1224,8 @@ __device__ __forceinline__ void small_body(const PcgArgs &a, const int nb, const
             if (qv > 0.0) sc.abs_inf = a.abs_factor * qv;
             else sc.tol2 = a.fallback_tol2;
         }
-        sc.iters = sc.done = sc.failed = sc.checked = 0;
+        sc.iters = sc.done = sc.failed = sc.plain = 0;
+        sc.limit = a.max_iters;
         sc.fresh = 1;
     }
     unsigned int epoch = 0;
@@ -1307,78 +1317,114 @@ __device__ __forceinline__ void small_body(const PcgArgs &a, const int nb, const
         __syncthreads();
         return true;
     };
+    // meets with (r, u), |r|^2, (w, u) and max|r|: the next alpha and beta of
+    // either recurrence, and its tests
+    auto advance = [&](auto work) -> bool {
+        return reduce(r * u, r * r, w * u, r, work, [&](const double *t, int wp, int l) {
+            if (wp == 0) {
+                const double be = sc.fresh ? 0.0 : t[0] * sc.rgamma;
+                const double den = sc.fresh ? t[2] : t[2] - be * t[0] * sc.ralpha;
+                __syncwarp();
+                const double o = (l == 0 ? t[0] : l == 1 ? den : 1.0) / (l == 0 ? den : t[0]);
+                if (l < 4) (&sc.alpha)[l] = l == 3 ? be : o;
+            } else if (l == 0) {
+                const double aim = sc.plain ? 1.0 : kSmallAim2, aim_inf = sc.plain ? 1.0 : 0.98;
+                sc.gamma = t[0];
+                sc.rr = t[1];
+                int done = sc.bb == 0.0 || t[1] <= aim * sc.stop || t[3] <= aim_inf * sc.abs_inf;
+                if (!done && sc.iters >= sc.limit) {
+                    done = 1;
+                    sc.failed = !(t[1] <= sc.stop || t[3] <= sc.abs_inf);
+                }
+                if (!done && !sc.plain) {
+                    const bool falls = t[1] < sc.best;
+                    sc.best = falls ? t[1] : sc.best;
+                    sc.since = falls ? 0 : sc.since + 1;
+                    done = sc.since >= kSmallStall;
+                }
+                sc.done = done;
+            }
+        });
+    };
     double *buf[2] = {a.u, a.w};
     int turn = 0;
     bool good = true;
+    const double x0 = x;
     // r = b - A x (x in memory, complete in every block)
     if (holds) r = a.x_zero ? b : b - spmv(a.x);
     while (true) {
-        // from r: u = D^-1 r, w = A u, m = D^-1 w, no directions yet
+        // from r: u = D^-1 r, w = A u, no directions yet
         u = d * r;
         p = s = q = z = 0;
         if (holds) buf[turn][i] = u;
-        good = reduce(b * b, 0.0, 0.0, 0.0, [&]() { if (holds) w = spmv(buf[turn]); },
+        good = reduce(b * b, 0.0, 0.0, b, [&]() { if (holds) w = spmv(buf[turn]); },
                       [&](const double *t, int wp, int l) {
                           if (wp + l == 0) {
                               sc.bb = t[0];
                               sc.stop = sc.tol2 * t[0];
+                              sc.best = 1.7976931348623157e308;
+                              sc.since = 0;
+                              if (sc.tol2 < kSmallTol2 && !(sc.abs_inf > 0.0 && sc.abs_inf * sc.abs_inf >= kSmallTol2 * t[3] * t[3]))
+                                  sc.plain = 1;
                           }
                       });
         if (!good) break;
         turn ^= 1;
-        m = d * w;
-        while (true) {
-            if (holds) buf[turn][i] = m;
+        const bool plain = sc.plain != 0;
+        if (plain) good = advance([]() {});
+        while (good) {
             double n = 0;
-            good = reduce(r * u, r * r, w * u, r, [&]() { if (holds) n = spmv(buf[turn]); },
-                          [&](const double *t, int wp, int l) {
-                              if (wp == 0) {
-                                  const double be = sc.fresh ? 0.0 : t[0] * sc.rgamma;
-                                  const double den = sc.fresh ? t[2] : t[2] - be * t[0] * sc.ralpha;
-                                  __syncwarp();
-                                  const double o = (l == 0 ? t[0] : l == 1 ? den : 1.0) / (l == 0 ? den : t[0]);
-                                  if (l < 4) (&sc.alpha)[l] = l == 3 ? be : o;
-                              } else if (l == 0) {
-                                  sc.gamma = t[0];
-                                  sc.rr = t[1];
-                                  int done = sc.bb == 0.0 || t[1] <= sc.stop || t[3] <= sc.abs_inf;
-                                  if (!done && sc.iters >= a.max_iters) done = sc.failed = 1;
-                                  sc.done = done;
-                              }
-                          });
-            if (!good || sc.done) break;
-            turn ^= 1;
+            if (plain) {
+                if (sc.done) break;
+            } else {
+                m = d * w;
+                if (holds) buf[turn][i] = m;
+                good = advance([&]() { if (holds) n = spmv(buf[turn]); });
+                if (!good || sc.done) break;
+                turn ^= 1;
+            }
             const double al = sc.alpha, be = sc.beta;
-            z = fma(be, z, n);
-            q = fma(be, q, m);
             s = fma(be, s, w);
             p = fma(be, p, u);
             x = fma(al, p, x);
             r = fma(-al, s, r);
-            u = fma(-al, q, u);
-            w = fma(-al, z, w);
-            m = d * w;
+            if (!plain) {
+                z = fma(be, z, n);
+                q = fma(be, q, m);
+                u = fma(-al, q, u);
+                w = fma(-al, z, w);
+            }
             if (threadIdx.x == 0) {
                 sc.iters++;
                 sc.fresh = 0;
             }
+            if (plain) {
+                u = d * r;
+                if (holds) buf[turn][i] = u;
+                if (!(good = meet())) break;
+                if (holds) w = spmv(buf[turn]);
+                turn ^= 1;
+                good = advance([]() {});
+            }
         }
         if (!good) break;
         if (sc.bb == 0.0) x = 0.0;
+        else if (!plain && !isfinite(sc.rr)) x = x0;   // broke down: from the start again
         if (holds) {
             a.x[i] = x;
             a.r[i] = r;
         }
-        if (sc.failed || sc.bb == 0.0 || sc.checked >= kSmallRestarts) break;
-        // the residual of x itself
+        if (plain || sc.failed || sc.bb == 0.0) break;
+        // the residual of x itself decides
         if (!(good = meet())) break;
         double t = 0;
         if (holds) t = b - spmv(a.x);
         good = reduce(t * t, 0.0, 0.0, t, []() {}, [&](const double *v, int wp, int l) {
             if (wp + l == 0) {
-                sc.done = v[0] <= 1.04 * sc.stop || v[3] <= 1.02 * sc.abs_inf;
-                sc.checked++;
-                sc.fresh = 1;
+                sc.rr = v[0];
+                sc.done = v[0] <= sc.stop || v[3] <= sc.abs_inf;
+                sc.fresh = sc.plain = 1;
+                sc.limit = a.max_iters < INT_MAX - sc.iters ? sc.iters + a.max_iters : INT_MAX;
             }
         });
         if (!good || sc.done) break;
@@ -2209,8 +2255,8 @@ static int assign_blocks(PcgArgs *runs, int n_runs, int budget) {
 // warp for the whole solve, whatever the launch shape asked for.  20^3 (52,460
 // rows, 1,640 slices, 227 iterations) 2.77 -> 1.70 ms; systems beyond take the streamed
 // form, whose iteration is bound by the FP64 pipes rather than by latency.  So
-// do relative tolerances below 1e-13, which the pipelined recurrence reaches
-// only with restarts (20^3 Laplacian, 1e-14: 3.0 ms against 1.3 ms).  A run
+// do relative tolerances below 1e-13, which the pipelined recurrence does not
+// reach (20^3 Laplacian, 1e-14: 3.0 ms with two restarts against 1.3 ms).  A run
 // gets the same blocks alone and in a batch, so its results are the same
 // bits.
 static int launch_small(PcgArgs *runs, int n_runs, cudaStream_t st, bool *launched) {
