@@ -444,8 +444,9 @@ int64_t pic_launch_count(void);
  * must be the one that holds that copy (PIC_ERR_INVALID_ARG otherwise).  The
  * first call on each device looks up the array's device address.  All calls
  * share the array and it keeps the last call's contents (the call sets
- * everything it reads); calls that overlap on the GPU, from two streams or
- * two threads, race on it.  Synchronises `stream` for its result
+ * everything it reads); a call holds the device's array until its work has
+ * ended, so calls from several threads or on several streams wait for one
+ * another.  Synchronises `stream` for its result
  * (PIC_ERR_STATE when `stream` is being captured). */
 int pic_electrostatic_solve_noalloc(const pic_mesh *mesh, const double *rho_nodes, double *phi_nodes, double tol,
                                     void *stream);

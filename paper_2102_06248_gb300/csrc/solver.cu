@@ -2841,8 +2841,9 @@ int read_control(Sim *s) {
 // The array is a file-scope device variable: every GPU on which this library's
 // solver module is loaded holds its 37.9 MB until the process exits.  It
 // bounds the problem to kNoAllocMaxNodes interior nodes.  All calls share it
-// and it keeps the last call's contents; calls whose work overlaps on the GPU
-// (different streams, or different host threads on one device) race on it.
+// and it keeps the last call's contents; a call holds the device's lock until
+// its work on the stream has ended, so calls from several threads or on several
+// streams follow one another.
 // ---------------------------------------------------------------------------
 constexpr int kNoAllocMaxNodes = 524288;
 constexpr size_t kNoAllocVectors = 9;   // b, x, r, p, q, z and z_old (or D^-1), then FP32 scratch
@@ -2850,8 +2851,9 @@ constexpr size_t kNoAllocDoubles = kNoAllocVectors * kNoAllocMaxNodes + 8 * (siz
 static __device__ __align__(256) double g_noalloc_scratch[kNoAllocDoubles];
 
 namespace {
-std::mutex g_noalloc_mutex;
+std::mutex g_noalloc_mutex;                            // of the address table
 constexpr int kNoAllocMaxDevices = 64;
+std::mutex g_noalloc_busy[kNoAllocMaxDevices];         // of a device's array
 double *g_noalloc_ptr[kNoAllocMaxDevices] = {};
 
 // device address of the scratch array on the current device (looked up once
@@ -2873,45 +2875,13 @@ int noalloc_scratch(double **out) {
     *out = g_noalloc_ptr[dev];
     return PIC_OK;
 }
-}  // namespace
 
-int electrostatic_solve_noalloc(const Mesh *m, const double *rho_nodes, double *phi_nodes, double tol,
-                                cudaStream_t st) {
+// the solve in the scratch array at base, which the caller holds
+int noalloc_solve(const Mesh *m, const double *rho_nodes, double *phi_nodes, double tol, double *base,
+                  cudaStream_t st) {
     const int nin = m->n_int_nodes;
-    if (nin > kNoAllocMaxNodes) {
-        set_error("pic_electrostatic_solve_noalloc: " + std::to_string(nin) + " interior nodes exceed the limit of " +
-                  std::to_string(kNoAllocMaxNodes));
-        return PIC_ERR_INVALID_ARG;
-    }
-    if (!m->uploaded) {
-        set_error("pic_electrostatic_solve_noalloc: the mesh has no device copy yet (create a simulation on it first)");
-        return PIC_ERR_STATE;
-    }
-    if (!(tol > 0) || !rho_nodes || !phi_nodes) {
-        set_error("pic_electrostatic_solve_noalloc: needs tol > 0 and device arrays for rho and phi");
-        return PIC_ERR_INVALID_ARG;
-    }
-    int dev = -1;
-    FP_CUDA(cudaGetDevice(&dev));
-    if (dev != m->device) {
-        set_error("pic_electrostatic_solve_noalloc: the current device (" + std::to_string(dev) +
-                  ") is not the device that holds the mesh (" + std::to_string(m->device) + ")");
-        return PIC_ERR_INVALID_ARG;
-    }
-    // the result is read back and waited for below, which a stream under
-    // capture does not allow
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    FP_CUDA(cudaStreamIsCapturing(st, &cap));
-    if (cap != cudaStreamCaptureStatusNone) {
-        set_error("pic_electrostatic_solve_noalloc: the stream is being captured; the call waits on the stream "
-                  "for its result");
-        return PIC_ERR_STATE;
-    }
-    double *base = nullptr;
-    int rc = noalloc_scratch(&base);
-    if (rc) return rc;
     FP_CUDA(cudaMemsetAsync(phi_nodes, 0, sizeof(double) * m->n_nodes, st));
-    if (nin == 0) return PIC_OK;
+    int rc;
     double *v[7];
     for (size_t k = 0; k < 7; k++) v[k] = base + k * kNoAllocMaxNodes;
     float *scratch = reinterpret_cast<float *>(base + 7 * (size_t)kNoAllocMaxNodes);
@@ -2973,6 +2943,52 @@ int electrostatic_solve_noalloc(const Mesh *m, const double *rho_nodes, double *
     FP_CUDA(cudaGetLastError());
     FP_CUDA(cudaStreamSynchronize(st));
     return PIC_OK;
+}
+}  // namespace
+
+int electrostatic_solve_noalloc(const Mesh *m, const double *rho_nodes, double *phi_nodes, double tol,
+                                cudaStream_t st) {
+    const int nin = m->n_int_nodes;
+    if (nin > kNoAllocMaxNodes) {
+        set_error("pic_electrostatic_solve_noalloc: " + std::to_string(nin) + " interior nodes exceed the limit of " +
+                  std::to_string(kNoAllocMaxNodes));
+        return PIC_ERR_INVALID_ARG;
+    }
+    if (!m->uploaded) {
+        set_error("pic_electrostatic_solve_noalloc: the mesh has no device copy yet (create a simulation on it first)");
+        return PIC_ERR_STATE;
+    }
+    if (!(tol > 0) || !rho_nodes || !phi_nodes) {
+        set_error("pic_electrostatic_solve_noalloc: needs tol > 0 and device arrays for rho and phi");
+        return PIC_ERR_INVALID_ARG;
+    }
+    int dev = -1;
+    FP_CUDA(cudaGetDevice(&dev));
+    if (dev != m->device) {
+        set_error("pic_electrostatic_solve_noalloc: the current device (" + std::to_string(dev) +
+                  ") is not the device that holds the mesh (" + std::to_string(m->device) + ")");
+        return PIC_ERR_INVALID_ARG;
+    }
+    // the result is read back and waited for below, which a stream under
+    // capture does not allow
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    FP_CUDA(cudaStreamIsCapturing(st, &cap));
+    if (cap != cudaStreamCaptureStatusNone) {
+        set_error("pic_electrostatic_solve_noalloc: the stream is being captured; the call waits on the stream "
+                  "for its result");
+        return PIC_ERR_STATE;
+    }
+    double *base = nullptr;
+    int rc = noalloc_scratch(&base);
+    if (rc) return rc;
+    if (nin == 0) {
+        FP_CUDA(cudaMemsetAsync(phi_nodes, 0, sizeof(double) * m->n_nodes, st));
+        return PIC_OK;
+    }
+    std::lock_guard<std::mutex> hold(g_noalloc_busy[dev]);
+    rc = noalloc_solve(m, rho_nodes, phi_nodes, tol, base, st);
+    if (rc) cudaStreamSynchronize(st);   // what was enqueued before the error leaves the array, too
+    return rc;
 }
 
 }  // namespace fp
