@@ -2846,6 +2846,10 @@ int read_control(Sim *s) {
 // streams follow one another.
 // ---------------------------------------------------------------------------
 constexpr int kNoAllocMaxNodes = 524288;
+// Multigrid iterations before the solve goes on with the diagonal as its
+// preconditioner: meshes of ordinary shapes take 10 to 30, tangled ones (24^3,
+// nodes moved by 0.6 of a cell: 160) are left to the cheaper iterations
+constexpr int kNoAllocMgIters = 100;
 constexpr size_t kNoAllocVectors = 9;   // b, x, r, p, q, z and z_old (or D^-1), then FP32 scratch
 constexpr size_t kNoAllocDoubles = kNoAllocVectors * kNoAllocMaxNodes + 8 * (size_t)kMaxBlocks + 64;
 static __device__ __align__(256) double g_noalloc_scratch[kNoAllocDoubles];
@@ -2895,7 +2899,15 @@ int noalloc_solve(const Mesh *m, const double *rho_nodes, double *phi_nodes, dou
     FP_CUDA(cudaMemsetAsync(status, 0, sizeof(uint32_t), st));
     { k_node_to_int<<<(nin + 255) / 256, 256, 0, st>>>(nin, m->int_node.p, rho_nodes, nullptr, b); note_launch(); }
     FP_CUDA(cudaGetLastError());
-    if (m->mg_levels > 0 && mg_scratch(m) <= 4 * (size_t)kNoAllocMaxNodes) {
+    CgState h{};
+    auto finish = [&]() -> int {
+        FP_CUDA(cudaMemcpyAsync(&h, dst, sizeof(CgState), cudaMemcpyDeviceToHost, st));
+        FP_CUDA(cudaStreamSynchronize(st));
+        return PIC_OK;
+    };
+    bool solved = false;
+    const bool hierarchy = m->mg_levels > 0 && mg_scratch(m) <= 4 * (size_t)kNoAllocMaxNodes;
+    if (hierarchy) {
         MgArgs a = mg_args(m, v, scratch);
         a.part = part;
         a.st = dst;
@@ -2903,13 +2915,20 @@ int noalloc_solve(const Mesh *m, const double *rho_nodes, double *phi_nodes, dou
         a.abs_src = nullptr;
         a.fallback_tol2 = tol * tol;
         a.status = status;
+        a.max_iters = kNoAllocMgIters;
         a.verify = 1;
-        if ((rc = launch_mg(a, 0, st))) return rc;
-    } else {
+        if ((rc = launch_mg(a, 0, st)) || (rc = finish())) return rc;
+        solved = h.done && !h.failed;
+    }
+    if (!solved) {
         if (!m->L_rec.p) {
             set_error("pic_electrostatic_solve_noalloc: the mesh has no device copy yet (create a simulation on it first)");
             return PIC_ERR_STATE;
         }
+        // after the multigrid solve: from its iterate, the other vectors cleared
+        const bool x_zero = !hierarchy || !std::isfinite(h.rr);
+        for (size_t k = x_zero ? 1 : 2; k < 7; k++) FP_CUDA(cudaMemsetAsync(v[k], 0, pad, st));
+        FP_CUDA(cudaMemsetAsync(status, 0, sizeof(uint32_t), st));
         { k_recip_diag<<<(nin + 255) / 256, 256, 0, st>>>(nin, m->L_diag.p, v[6]); note_launch(); }
         PcgArgs a = matrix_args(m->Ls, m->Ls_val.p, m->L_rec);
         a.Dinv = v[6];
@@ -2928,13 +2947,10 @@ int noalloc_solve(const Mesh *m, const double *rho_nodes, double *phi_nodes, dou
         a.abs_inf = -1.0;
         a.status = status;
         a.max_iters = 20000;
-        a.x_zero = 1;
+        a.x_zero = x_zero;
         a.spin_limit = (int)kSpinLimit;
-        if ((rc = launch_pcg_runs(&a, 1, 0, st))) return rc;
+        if ((rc = launch_pcg_runs(&a, 1, 0, st)) || (rc = finish())) return rc;
     }
-    CgState h{};
-    FP_CUDA(cudaMemcpyAsync(&h, dst, sizeof(CgState), cudaMemcpyDeviceToHost, st));
-    FP_CUDA(cudaStreamSynchronize(st));
     if (h.failed || !h.done) {
         set_error("pic_electrostatic_solve_noalloc: PCG did not reach the tolerance");
         return PIC_ERR_CG_NO_CONVERGENCE;

@@ -29,9 +29,9 @@ def node_laplacian(box):
     vol = np.abs(np.linalg.det(d)) / 6.0
     k = W.EPS0 * vol[:, None, None] * np.einsum("tid,tjd->tij", g, g)
     L = sp.csr_matrix((k.ravel(), (np.repeat(t, 4, 1).ravel(), np.tile(t, (1, 4)).ravel())), shape=(n, n))
-    lo, hi = box.xyz.min(0), box.xyz.max(0)
+    lo, hi = box.ref_xyz.min(0), box.ref_xyz.max(0)
     eps = 1e-9 * (hi - lo)
-    inside = np.where(((box.xyz > lo + eps) & (box.xyz < hi - eps)).all(1))[0]
+    inside = np.where(((box.ref_xyz > lo + eps) & (box.ref_xyz < hi - eps)).all(1))[0]
     return L[inside][:, inside].tocsr(), inside
 
 
