@@ -306,6 +306,7 @@ int gnn_forward(Sim *s, const double *r, double *z, bool keep);
 int gnn_loss_grad(Sim *s, const double *r, double *loss, double *grad_host);
 int gnn_train(Sim *s, const pic_gnn_train_cfg *cfg, double *loss_out);
 int fpcg_newmark(Sim *s, int *iters_out);
+int noalloc_outcome(int done, int failed, uint32_t status);
 int electrostatic_solve_noalloc(const Mesh *m, const double *rho_nodes, double *phi_nodes, double tol,
                                 cudaStream_t st);
 

@@ -2854,6 +2854,19 @@ constexpr size_t kNoAllocVectors = 9;   // b, x, r, p, q, z and z_old (or D^-1),
 constexpr size_t kNoAllocDoubles = kNoAllocVectors * kNoAllocMaxNodes + 8 * (size_t)kMaxBlocks + 64;
 static __device__ __align__(256) double g_noalloc_scratch[kNoAllocDoubles];
 
+// The call's return code for what its solve left: state flags and status word
+int noalloc_outcome(int done, int failed, uint32_t status) {
+    if (status & ST_BARRIER) {
+        set_error("pic_electrostatic_solve_noalloc: a persistent solver kernel timed out at a grid barrier");
+        return PIC_ERR_CUDA;
+    }
+    if (failed || !done) {
+        set_error("pic_electrostatic_solve_noalloc: PCG did not reach the tolerance");
+        return PIC_ERR_CG_NO_CONVERGENCE;
+    }
+    return PIC_OK;
+}
+
 namespace {
 std::mutex g_noalloc_mutex;                            // of the address table
 constexpr int kNoAllocMaxDevices = 64;
@@ -2880,6 +2893,14 @@ int noalloc_scratch(double **out) {
     return PIC_OK;
 }
 
+// what a solve leaves, read back in one copy
+struct NoAllocResult {
+    CgState st;
+    GridBarrier gb;
+    uint32_t status;
+};
+static_assert(sizeof(NoAllocResult) <= 64 * sizeof(double), "behind the partials");
+
 // the solve in the scratch array at base, which the caller holds
 int noalloc_solve(const Mesh *m, const double *rho_nodes, double *phi_nodes, double tol, double *base,
                   cudaStream_t st) {
@@ -2890,20 +2911,22 @@ int noalloc_solve(const Mesh *m, const double *rho_nodes, double *phi_nodes, dou
     for (size_t k = 0; k < 7; k++) v[k] = base + k * kNoAllocMaxNodes;
     float *scratch = reinterpret_cast<float *>(base + 7 * (size_t)kNoAllocMaxNodes);
     double *b = v[0], *x = v[1], *part = base + kNoAllocVectors * kNoAllocMaxNodes;
-    CgState *dst = reinterpret_cast<CgState *>(part + 8 * (size_t)kMaxBlocks);
-    GridBarrier *gb = reinterpret_cast<GridBarrier *>(dst + 1);
-    uint32_t *status = reinterpret_cast<uint32_t *>(gb + 1);
+    NoAllocResult *res = reinterpret_cast<NoAllocResult *>(part + 8 * (size_t)kMaxBlocks);
+    CgState *dst = &res->st;
+    GridBarrier *gb = &res->gb;
+    uint32_t *status = &res->status;
     // the vectors are padded to whole slices, zeros past the rows
     const size_t pad = (size_t)(nin + 31) / 32 * 32 * sizeof(double);
     for (size_t k = 0; k < 7; k++) FP_CUDA(cudaMemsetAsync(v[k], 0, pad, st));
     FP_CUDA(cudaMemsetAsync(status, 0, sizeof(uint32_t), st));
     { k_node_to_int<<<(nin + 255) / 256, 256, 0, st>>>(nin, m->int_node.p, rho_nodes, nullptr, b); note_launch(); }
     FP_CUDA(cudaGetLastError());
-    CgState h{};
+    // waits for a solve; its outcome, and with it whether phi may be read
+    NoAllocResult h{};
     auto finish = [&]() -> int {
-        FP_CUDA(cudaMemcpyAsync(&h, dst, sizeof(CgState), cudaMemcpyDeviceToHost, st));
+        FP_CUDA(cudaMemcpyAsync(&h, res, sizeof(h), cudaMemcpyDeviceToHost, st));
         FP_CUDA(cudaStreamSynchronize(st));
-        return PIC_OK;
+        return noalloc_outcome(h.st.done, h.st.failed, h.status);
     };
     bool solved = false;
     const bool hierarchy = m->mg_levels > 0 && mg_scratch(m) <= 4 * (size_t)kNoAllocMaxNodes;
@@ -2917,8 +2940,10 @@ int noalloc_solve(const Mesh *m, const double *rho_nodes, double *phi_nodes, dou
         a.status = status;
         a.max_iters = kNoAllocMgIters;
         a.verify = 1;
-        if ((rc = launch_mg(a, 0, st)) || (rc = finish())) return rc;
-        solved = h.done && !h.failed;
+        if ((rc = launch_mg(a, 0, st))) return rc;
+        rc = finish();
+        if (rc && rc != PIC_ERR_CG_NO_CONVERGENCE) return rc;
+        solved = rc == PIC_OK;
     }
     if (!solved) {
         if (!m->L_rec.p) {
@@ -2926,7 +2951,7 @@ int noalloc_solve(const Mesh *m, const double *rho_nodes, double *phi_nodes, dou
             return PIC_ERR_STATE;
         }
         // after the multigrid solve: from its iterate, the other vectors cleared
-        const bool x_zero = !hierarchy || !std::isfinite(h.rr);
+        const bool x_zero = !hierarchy || !std::isfinite(h.st.rr);
         for (size_t k = x_zero ? 1 : 2; k < 7; k++) FP_CUDA(cudaMemsetAsync(v[k], 0, pad, st));
         FP_CUDA(cudaMemsetAsync(status, 0, sizeof(uint32_t), st));
         { k_recip_diag<<<(nin + 255) / 256, 256, 0, st>>>(nin, m->L_diag.p, v[6]); note_launch(); }
@@ -2950,10 +2975,6 @@ int noalloc_solve(const Mesh *m, const double *rho_nodes, double *phi_nodes, dou
         a.x_zero = x_zero;
         a.spin_limit = (int)kSpinLimit;
         if ((rc = launch_pcg_runs(&a, 1, 0, st)) || (rc = finish())) return rc;
-    }
-    if (h.failed || !h.done) {
-        set_error("pic_electrostatic_solve_noalloc: PCG did not reach the tolerance");
-        return PIC_ERR_CG_NO_CONVERGENCE;
     }
     { k_int_to_node<<<(nin + 255) / 256, 256, 0, st>>>(nin, m->int_node.p, x, phi_nodes); note_launch(); }
     FP_CUDA(cudaGetLastError());
