@@ -1342,7 +1342,8 @@ __global__ void __launch_bounds__(kPushBlock, 4) k_push_mixed(const PushArgs<flo
     }
     alive = __reduce_add_sync(0xFFFFFFFFu, alive);
     if (lane == 0) {
-        a.ke_part[gw] = (double)ke_hi + (double)ke_lo;
+        // (past the FP32 range the sum is infinite and its remainder NaN)
+        a.ke_part[gw] = isfinite(ke_hi) ? (double)ke_hi + (double)ke_lo : (double)ke_hi;
         if (alive) atomicAdd(a.n_alive_next, alive);
     }
 }
