@@ -2921,12 +2921,12 @@ int noalloc_solve(const Mesh *m, const double *rho_nodes, double *phi_nodes, dou
     FP_CUDA(cudaMemsetAsync(status, 0, sizeof(uint32_t), st));
     { k_node_to_int<<<(nin + 255) / 256, 256, 0, st>>>(nin, m->int_node.p, rho_nodes, nullptr, b); note_launch(); }
     FP_CUDA(cudaGetLastError());
-    // waits for a solve; its outcome, and with it whether phi may be read
+    // waits for a solve and reads back what it left
     NoAllocResult h{};
     auto finish = [&]() -> int {
         FP_CUDA(cudaMemcpyAsync(&h, res, sizeof(h), cudaMemcpyDeviceToHost, st));
         FP_CUDA(cudaStreamSynchronize(st));
-        return noalloc_outcome(h.st.done, h.st.failed, h.status);
+        return PIC_OK;
     };
     bool solved = false;
     const bool hierarchy = m->mg_levels > 0 && mg_scratch(m) <= 4 * (size_t)kNoAllocMaxNodes;
@@ -2940,10 +2940,10 @@ int noalloc_solve(const Mesh *m, const double *rho_nodes, double *phi_nodes, dou
         a.status = status;
         a.max_iters = kNoAllocMgIters;
         a.verify = 1;
-        if ((rc = launch_mg(a, 0, st))) return rc;
-        rc = finish();
-        if (rc && rc != PIC_ERR_CG_NO_CONVERGENCE) return rc;
-        solved = rc == PIC_OK;
+        if ((rc = launch_mg(a, 0, st)) || (rc = finish())) return rc;
+        // (short of the tolerance here is not a failure of the call)
+        if (h.status & ST_BARRIER) return noalloc_outcome(h.st.done, h.st.failed, h.status);
+        solved = h.st.done && !h.st.failed;
     }
     if (!solved) {
         if (!m->L_rec.p) {
@@ -2974,7 +2974,9 @@ int noalloc_solve(const Mesh *m, const double *rho_nodes, double *phi_nodes, dou
         a.max_iters = 20000;
         a.x_zero = x_zero;
         a.spin_limit = (int)kSpinLimit;
-        if ((rc = launch_pcg_runs(&a, 1, 0, st)) || (rc = finish())) return rc;
+        if ((rc = launch_pcg_runs(&a, 1, 0, st)) || (rc = finish()) ||
+            (rc = noalloc_outcome(h.st.done, h.st.failed, h.status)))
+            return rc;
     }
     { k_int_to_node<<<(nin + 255) / 256, 256, 0, st>>>(nin, m->int_node.p, x, phi_nodes); note_launch(); }
     FP_CUDA(cudaGetLastError());
