@@ -175,8 +175,10 @@ typedef struct {
     double completion_tol;   /* the gradient-subspace completion of each Newmark solve stops
                                 when its defect is <= completion_tol * max|rho + wall| (1e-16) */
     int32_t walk_cap;        /* max tets one particle visits in one step (64) */
-    int32_t solver_blocks_per_sm; /* blocks per SM of the persistent PCG (0: as many as fit for the
-                                     Newmark solve, two for the latency-bound completion) */
+    int32_t solver_blocks_per_sm; /* most blocks per SM of the persistent solvers (0: as many as fit).
+                                     The solves of one simulation run one block of 512 to 1,024
+                                     threads per SM, which every value allows; a batch's tuner
+                                     chooses its own count */
     int32_t max_species;     /* species slots (4) */
     int32_t profile;         /* 1: time the phases of every step with CUDA events (0) */
     void *stream;            /* cudaStream_t to run on; NULL = default stream */
@@ -186,8 +188,9 @@ typedef struct {
     int32_t curved_path;     /* 1: the path of a step is the Lagrange polynomial through r^{n+1}, r^n
                                 and the earlier positions at t_{n+1}, t_n, ... (Sec. III.B, Eq. path;
                                 degree = the Adams-Bashforth order in use, so it ramps up with the
-                                history), walked with Algorithm 1, exits found by Algorithm 2's
-                                bisection to 1e-15 of the step, Whitney-1 integrated over each in-cell
+                                history), walked with Algorithm 1, exits bracketed to 1e-15 of the step
+                                as by Algorithm 2's bisection (by false position where the bracket's
+                                inside end is known), Whitney-1 integrated over each in-cell
                                 piece by max(degree, 2)-point Gauss-Legendre (exact: the integrand has
                                 degree 2 deg - 1).  Adams-Bashforth pusher and PLAIN precision only
                                 (PIC_ERR_INVALID_ARG otherwise).  0: straight segments (default) */
@@ -199,7 +202,10 @@ void pic_config_default(pic_config *cfg);
 /* Creates a simulation on the mesh (which must outlive it).  Assembles the
  * system matrix of the field update: A = [*eps] + dt^2/4 [*S] + dt/(2c) [*I]
  * for the Newmark forms (Sec. II.B), A = [*eps] + dt^2 [*S] + (dt/c) [*I] for
- * the backward difference ([*I] = 0 without absorbing walls).  Errors:
+ * the backward difference ([*I] = 0 without absorbing walls).  The simulation
+ * holds A on the device twice in FP64, as sparse slices and as the records that
+ * its solver streams, and in MIXED once more in FP32 (64^3 cells: 0.23, 0.27 and
+ * 0.15 GB).  Errors:
  * PIC_ERR_INVALID_ARG (bad config), PIC_ERR_OOM, PIC_ERR_CUDA. */
 int pic_sim_create(const pic_mesh *mesh, const pic_config *cfg, pic_sim **out);
 void pic_sim_destroy(pic_sim *sim);
@@ -381,10 +387,14 @@ int pic_gnn_loss_grad(pic_sim *sim, const double *r_edges, double *loss, double 
  * blocks per SM; 80 registers, up to three; more blocks do not fit beside
  * each other's shared memory, and their candidates stand for four) by timing
  * each candidate on the batch's own systems (kept per batch shape).
- * Results are those of
- * pic_step on each member: bitwise when every member's solve gets the
- * blocks it would get alone (then the kernels and reduction orders are the
- * same), otherwise equal to the solve tolerance.  A member whose mesh has
+ * Results are those of pic_step on each member to the solve tolerance.
+ * Fields and particles are the same bits where every system is solved by the
+ * kernel and the blocks that solve it alone: no member has a multigrid
+ * hierarchy, the Newmark systems take at most one block per SM together (a
+ * block per 128 interior edges of a member, so 19,456 edges on 152 SMs), and
+ * they are of one kind (FP64 systems with cg_tol below 1e-13, or with more
+ * than 32 slots in a row of the matrix, are solved by another kernel, in a
+ * batch then all of them).  A member whose mesh has
  * 8,192 or more interior nodes completes with the multigrid-preconditioned
  * solve as under pic_step; the batch runs all completions in one launch (the
  * multigrid members' beside the others' Jacobi-PCG), and the tuner then

@@ -521,7 +521,7 @@ __global__ void __launch_bounds__(kThreads) k_max_abs_sum(int n, const double *_
 // counter that only grows plus acquire-loads; every wait is bounded, past its
 // bound the kernel records a timeout and every block leaves.
 // Measured on the 64^3 plasma ball (1.8M rows, MIXED, 60 iterations): 4.44 ->
-// 2.69 ms a solve, 45 us an iteration: the stream of 150 MB of records takes
+// 2.72 ms a solve, 45 us an iteration: the stream of 150 MB of records takes
 // 22 us of them at the copy rate (it was 232 MB), the vector phase 4 us, the
 // two barriers and the reduction 9 us.
 // ---------------------------------------------------------------------------
@@ -2257,8 +2257,9 @@ static int assign_blocks(PcgArgs *runs, int n_runs, int budget) {
 // form, whose iteration is bound by the FP64 pipes rather than by latency.  So
 // do relative tolerances below 1e-13, which the pipelined recurrence does not
 // reach (20^3 Laplacian, 1e-14: 3.0 ms with two restarts against 1.3 ms).  A run
-// gets the same blocks alone and in a batch, so its results are the same
-// bits.
+// gets the same blocks alone and in a batch, so its results are the same bits
+// there; where a run does not qualify or the runs' blocks exceed the SMs, all of
+// them take the streamed form, and agree with their solves alone to the tolerance.
 static int launch_small(PcgArgs *runs, int n_runs, cudaStream_t st, bool *launched) {
     const int most = std::min(sm_count(), kSmallBlocks);
     int G = 0;

@@ -64,8 +64,11 @@ class pic_batch_info_t(C.Structure):
                 ("completion_build", C.c_int32), ("pad_", C.c_int32), ("tune_newmark_ms", C.c_double * 9),
                 ("tune_completion_ms", C.c_double * 9)]
 
+# (blocks/SM, build) of the tuner's nine entries.  Builds 2 and 3 stand for four
+# blocks of build 0, whose time their entries repeat: the tuner never picks them,
+# and the names of the kernels that they once were are kept for callers only
 BATCH_BUILDS = ("64-register", "80-register", "40-register", "32-register")
-BATCH_TUNE_CANDIDATES = ((2, 0), (3, 0), (4, 0), (2, 1), (3, 1), (5, 2), (6, 2), (7, 3), (8, 3))   # (blocks/SM, build)
+BATCH_TUNE_CANDIDATES = ((2, 0), (3, 0), (4, 0), (2, 1), (3, 1), (5, 2), (6, 2), (7, 3), (8, 3))
 
 
 class pic_diag(C.Structure):
