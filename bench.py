@@ -45,12 +45,12 @@ CLOCK_LOG = None   # --clock-log: where the clock samples of the timed region go
 FP64_NOMINAL_TFLOPS = 1.25   # GB300 dense FP64 (non-tensor) nominal rate
 # DRAM bytes over algorithmic bytes of the MIXED Newmark launch
 # (k_pcg_persistent<1, 0>), from one ncu capture of that kernel (its current
-# code) on the 64^3 plasma ball: 10.374 GB (dram__bytes_read.sum +
+# code) on the 64^3 plasma ball: 10.379 GB (dram__bytes_read.sum +
 # dram__bytes_write.sum) for 60 FP32 + 2 FP64 iterations whose algorithmic
 # bytes are 14.440 GB (below 1: with the matrix loaded evict-first, the
 # vectors written each iteration stay in L2).  The FP64 Newmark form has no
 # capture of its current code: its traffic is reported as null.
-TRAFFIC_RATIO_MIXED = (10.271964 + 0.101604) / 14.439829
+TRAFFIC_RATIO_MIXED = (10.275731 + 0.103644) / 14.439829
 # DRAM bytes of one MIXED push launch (k_push_mixed<0>) on the 64^3 plasma-ball
 # mesh with 4M + 4M particles, from one ncu capture of the current kernel:
 # 0.445 + 0.352 GB (100 B per particle, per-tet bytes included); scaled to a
